@@ -47,6 +47,8 @@ __host__ __device__ __forceinline__ int64_t cell_count(int nx, int ny, int nz)
     return (int64_t)((nx + 3) >> 2) * ((ny + 3) >> 2) * ((nz + 3) >> 2) * 64;
 }
 
+constexpr int kSym64Tiles = 5;   // FP64 symmetric gravity: tiles of 512, 256, 128, 64 or 32 spheres
+
 // Static description of one pile (host-owned; re-uploaded on membership change).
 struct PileStatic {
     int64_t s0, ns;        // sphere range [s0, s0+ns) (home order == sorted range)
@@ -77,7 +79,7 @@ struct PileStatic {
     // a sphere's sum of |terms|) <= 2^61, |k| <= 120); ginv = 1 / gscale
     double ginv;
     float gscale_f;
-    int32_t pad_g;
+    int32_t gtile64;       // FP64 symmetric form: spheres per tile of this pile
     // the contact law's constants in FP32 for the mixed path (kn, kt, cn, ct,
     // mu_s, mu_r, mu_t, w0, h), rounded once on the host
     float lawf[9];
@@ -261,6 +263,9 @@ struct Sizes {
     int32_t gacc_on; // mixed symmetric gravity: piles of more than one tile leave their sums in gacc,
                      // which k_grav_acc_to_force turns into forces
     int32_t grav;    // some pile has self-gravity (G > 0)
+    // FP64 symmetric form: items of the piles with tiles of 512 >> c spheres
+    // are [g64_first[c], g64_first[c + 1]), run by at most g64_blocks[c] blocks
+    int64_t g64_first[6], g64_blocks[5];
 };
 
 // ---- kernel launchers (kernels_*.cu) -------------------------------------

@@ -35,6 +35,8 @@
 // k_grav_acc_to_force turns them into forces.  FP64 path: every item writes
 // its i-sums (one per b) and j-sums (one per a) as FP64 partials, and
 // k_grav_combine_sym64 adds a sphere's partials in tile order.
+#include <algorithm>
+
 #include "dem_internal.h"
 #include "devmath.cuh"
 #include "launch.cuh"
@@ -458,7 +460,7 @@ __global__ void __launch_bounds__(BS) k_gravity64(Arrays a, Sizes z)
 }
 
 // ---------------------------------------------------------------- symmetric form
-constexpr int kSymBS = 128, kSymIB = 4, kSymTile = kSymBS * kSymIB;   // 512 spheres per tile
+constexpr int kSymTile = 512;   // spheres per tile (large piles)
 // shape of the mixed path's 512-sphere tiles: warps per block x i-spheres per lane
 #ifndef DEM_SYM_WPB
 #define DEM_SYM_WPB 4
@@ -757,24 +759,61 @@ __global__ void DEM_GSYM_BOUNDS k_gravity32s(Arrays a, Sizes z)
     }
 }
 
+// r2^(-3/2) on as few FP64 instructions as possible: the FP64 unit (about 1.7
+// operations per clock and SM, against 128 for FP32 and 64 for integers) is
+// what bounds the FP64 pass, so whatever can be formed exactly elsewhere is.
+// y0 = the hardware's approximate rsqrt, a double with a 21-bit significand
+// (its low word is zero), |e| <= 2e-6 with e = 1 - r2 y0^2.  From the binomial
+// series of (1 - e)^(-3/2),
+//   r2^(-3/2) = y0^3 (1 + 3/2 e + 15/8 e^2 + O(e^3)),  35/16 |e|^3 < 2^-55;
+// y0^2 has 42 bits and is formed by an integer product (exact), the 15/8 e^2
+// term (below 2^-36) in FP32 with its bits widened by integer instructions:
+// 4 FP64 operations in all.  Largest relative error over 2^-20..2^20:
+// 2.3e-16, against 4.4e-16 for rsqrt(r2) cubed.  r2 is kept inside
+// [2^-1020, 2^1020] (y0^2 then stays a normal number): r2 = 0 still gives a
+// result that is not finite, an overflowed r2 zero.
+// Measured, 1.1e8 pairs / 152 SMs: 2.85 ms with rsqrt() cubed, 2.53 ms so.
+__device__ __forceinline__ double grav_inv3(double r2)
+{
+    r2 = __hiloint2double(min(max(__double2hiint(r2), 0x00300000), 0x7fb00000), __double2loint(r2));
+    double y0;
+    asm("rsqrt.approx.ftz.f64 %0, %1;" : "=d"(y0) : "d"(r2));
+    const unsigned yh = (unsigned)__double2hiint(y0);
+    const unsigned long long m = (yh & 0xfffffu) | 0x100000u, mm = m * m;   // in [2^40, 2^42)
+    const unsigned big = (unsigned)(mm >> 41);
+    const unsigned long long bits =
+        ((mm << (12 - big)) & 0xfffffffffffffull) | ((unsigned long long)(2 * (yh >> 20) - 1023 + big) << 52);
+    const double t = __longlong_as_double((long long)bits);
+    const double e = fma(-r2, t, 1.0), y3 = t * y0;
+    const int eh = __double2hiint(e) & 0x7fffffff;
+    const float ef = __int_as_float(eh > (897 << 20) ? (eh - (896 << 20)) << 3 : 0);
+    const int cb = __float_as_int(1.875f * ef * ef);
+    const double q = fma(1.5, e, __hiloint2double(cb > 0 ? (cb >> 3) + (896 << 20) : 0, cb << 29));
+    return fma(y3, q, y3);
+}
+
 // FP64 path, symmetric form: the same tile pairs and ring as the mixed path
 // in double precision (scalar: no packed FP64 instructions), partial sums in
-// FP64 and combined in FP64.  Shared memory: tile b (32 B per sphere), its
-// aggregates and the per-warp j-sums (4 x 512 x 32 B): 82 KB per block.
-template <bool MASK>
-__device__ __forceinline__ dbl4 sym_ring64(dbl4 pj, int aj, const dbl4 (&xi)[kSymIB], const int (&ai)[kSymIB],
-                                           double (&ax)[kSymIB], double (&ay)[kSymIB], double (&az)[kSymIB],
-                                           double eps2)
+// FP64 and combined in FP64.  WPB warps with 32 IB i-spheres each: tiles of
+// 32 WPB IB spheres, chosen per pile by its size alone (sym_tile64 in
+// world.cpp), one launch per tile size that the world's piles use.  The ring's
+// shuffles hide behind the FP64 unit, so IB is small; what counts is that
+// every SM has items left when the others finish: at 1,000 spheres, 3 items of
+// 512 x 512 pairs took 1,561 us on 3 SMs, 528 items of 32 x 32 use the chip.
+// Shared memory: tile b (32 B per sphere), the per-warp j-sums and tile b's
+// aggregates.
+template <bool MASK, int IB>
+__device__ __forceinline__ dbl4 sym_ring64(dbl4 pj, int aj, const dbl4 (&xi)[IB], const int (&ai)[IB],
+                                           double (&ax)[IB], double (&ay)[IB], double (&az)[IB], double eps2)
 {
     const int src = (threadIdx.x + 1) & 31;
     double fx = 0.0, fy = 0.0, fz = 0.0;
+#pragma unroll 2
     for (int s = 0; s < 32; ++s) {
 #pragma unroll
-        for (int k = 0; k < kSymIB; ++k) {
+        for (int k = 0; k < IB; ++k) {
             const double dx = pj.x - xi[k].x, dy = pj.y - xi[k].y, dz = pj.z - xi[k].z;
-            const double r2 = fma(dz, dz, fma(dy, dy, fma(dx, dx, eps2)));
-            const double inv = rsqrt(r2);
-            const double inv3 = (inv * inv) * inv;
+            const double inv3 = grav_inv3(fma(dz, dz, fma(dy, dy, fma(dx, dx, eps2))));
             double si = pj.w * inv3, sj = -xi[k].w * inv3;
             if (MASK && aj == ai[k]) si = sj = 0.0;
             ax[k] = fma(dx, si, ax[k]);
@@ -796,8 +835,10 @@ __device__ __forceinline__ dbl4 sym_ring64(dbl4 pj, int aj, const dbl4 (&xi)[kSy
     return make_dbl4(fx, fy, fz, 0.0);
 }
 
+template <int WPB, int IB>
 __device__ __forceinline__ void gravity64s_item(const Arrays &a, const int4 it, dbl4 *sp, int *sag, dbl4 *sj)
 {
+    constexpr int kBS = 32 * WPB, kTile = kBS * IB;
     const int p = it.x;
     if (a.enabled[p] == 0 || a.pd[p].failed) return;
     const PileStatic &S = a.ps[p];
@@ -808,37 +849,35 @@ __device__ __forceinline__ void gravity64s_item(const Arrays &a, const int4 it, 
     const bool diag = ta == tb;
     const double eps2 = S.eps2;
     const int w = threadIdx.x >> 5, l = threadIdx.x & 31;
-    const int jb0 = tb * kSymTile;
-    const int nj = min(kSymTile, ns - jb0);
-    for (int m = threadIdx.x; m < kSymTile; m += kSymBS) {
+    const int jb0 = tb * kTile;
+    const int nj = min(kTile, ns - jb0);
+    for (int m = threadIdx.x; m < kTile; m += kBS) {
         const int j = jb0 + m;
         sp[m] = j < ns ? a.gpos64[s0 + j] : make_dbl4(1.0e150, 1.0e150, 1.0e150, 0.0);
         sag[m] = j < ns ? a.sph_agg[s0 + j] : -1;
     }
-    dbl4 xi[kSymIB];
-    int ai[kSymIB];
-    double ax[kSymIB], ay[kSymIB], az[kSymIB];
-    const int i0 = ta * kSymTile + w * (32 * kSymIB) + l;
+    dbl4 xi[IB];
+    int ai[IB];
+    double ax[IB], ay[IB], az[IB];
+    const int i0 = ta * kTile + w * (32 * IB) + l;
 #pragma unroll
-    for (int k = 0; k < kSymIB; ++k) {
+    for (int k = 0; k < IB; ++k) {
         const int i = i0 + 32 * k;
         const bool ok = i < ns;
         xi[k] = ok ? a.gpos64[s0 + i] : make_dbl4(0.0, 0.0, 0.0, 0.0);
         ai[k] = ok ? a.sph_agg[s0 + i] : -2;
         ax[k] = ay[k] = az[k] = 0.0;
     }
-    const bool masked = diag || a.sph_agg[s0 + (int64_t)ta * kSymTile + kSymTile - 1] == a.sph_agg[s0 + jb0];
+    const bool masked = diag || a.sph_agg[s0 + (int64_t)ta * kTile + kTile - 1] == a.sph_agg[s0 + jb0];
     __syncthreads();
     if (diag) {
         for (int jj = 0; jj < nj; ++jj) {
             const dbl4 pj = sp[jj];
             const int aj = sag[jj];
 #pragma unroll
-            for (int k = 0; k < kSymIB; ++k) {
+            for (int k = 0; k < IB; ++k) {
                 const double dx = pj.x - xi[k].x, dy = pj.y - xi[k].y, dz = pj.z - xi[k].z;
-                const double r2 = fma(dz, dz, fma(dy, dy, fma(dx, dx, eps2)));
-                const double inv = rsqrt(r2);
-                double si = (pj.w * inv) * (inv * inv);
+                double si = pj.w * grav_inv3(fma(dz, dz, fma(dy, dy, fma(dx, dx, eps2))));
                 si = aj == ai[k] ? 0.0 : si;
                 ax[k] = fma(dx, si, ax[k]);
                 ay[k] = fma(dy, si, ay[k]);
@@ -849,19 +888,24 @@ __device__ __forceinline__ void gravity64s_item(const Arrays &a, const int4 it, 
         for (int c = 0; c * 32 < nj; ++c) {
             const dbl4 pj = sp[c * 32 + l];
             const int aj = sag[c * 32 + l];
-            sj[w * kSymTile + c * 32 + l] = masked ? sym_ring64<true>(pj, aj, xi, ai, ax, ay, az, eps2)
-                                                   : sym_ring64<false>(pj, aj, xi, ai, ax, ay, az, eps2);
+            sj[w * kTile + c * 32 + l] = masked ? sym_ring64<true, IB>(pj, aj, xi, ai, ax, ay, az, eps2)
+                                                : sym_ring64<false, IB>(pj, aj, xi, ai, ax, ay, az, eps2);
         }
         __syncthreads();
-        for (int m = threadIdx.x; m < nj; m += kSymBS) {
-            const dbl4 u0 = sj[m], u1 = sj[kSymTile + m], u2 = sj[2 * kSymTile + m], u3 = sj[3 * kSymTile + m];
-            ((dbl4 *)a.gpart)[sym_slot(a, p, ns, T + ta, jb0 + m)] =
-                make_dbl4(((u0.x + u1.x) + u2.x) + u3.x, ((u0.y + u1.y) + u2.y) + u3.y,
-                          ((u0.z + u1.z) + u2.z) + u3.z, 0.0);
+        for (int m = threadIdx.x; m < nj; m += kBS) {
+            dbl4 u = sj[m];
+#pragma unroll
+            for (int v = 1; v < WPB; ++v) {
+                const dbl4 t = sj[v * kTile + m];
+                u.x += t.x;
+                u.y += t.y;
+                u.z += t.z;
+            }
+            ((dbl4 *)a.gpart)[sym_slot(a, p, ns, T + ta, jb0 + m)] = make_dbl4(u.x, u.y, u.z, 0.0);
         }
     }
 #pragma unroll
-    for (int k = 0; k < kSymIB; ++k) {
+    for (int k = 0; k < IB; ++k) {
         const int i = i0 + 32 * k;
         if (i >= ns) continue;
         if (T == 1) {
@@ -873,27 +917,42 @@ __device__ __forceinline__ void gravity64s_item(const Arrays &a, const int4 it, 
     }
 }
 
-constexpr size_t kSym64Smem = sizeof(dbl4) * kSymTile * 5 + sizeof(int) * kSymTile;
+constexpr size_t sym64_smem(int tile, int wpb) { return (size_t)tile * (sizeof(dbl4) * (1 + wpb) + sizeof(int)); }
 
-__global__ void __launch_bounds__(kSymBS) k_gravity64s(Arrays a, Sizes z)
+template <int WPB, int IB>
+__global__ void __launch_bounds__(32 * WPB) k_gravity64s(Arrays a, Sizes z, int64_t first, int64_t count)
 {
     pdl_enter();
+    constexpr int kTile = 32 * WPB * IB;
     extern __shared__ __align__(32) unsigned char sm64[];
     dbl4 *sp = (dbl4 *)sm64;
-    dbl4 *sj = sp + kSymTile;
-    int *sag = (int *)(sj + 4 * kSymTile);
+    dbl4 *sj = sp + kTile;
+    int *sag = (int *)(sj + WPB * kTile);
     __shared__ int next;
     for (;;) {
         __syncthreads();
-        if (threadIdx.x == 0) next = grab_item(a.gcounter, z.GI);
+        if (threadIdx.x == 0) next = grab_item(a.gcounter, count);
         __syncthreads();
         const int item = next;
-        if (item >= z.GI) return;
-        gravity64s_item(a, a.gitems[item], sp, sag, sj);
+        if (item >= count) return;
+        gravity64s_item<WPB, IB>(a, a.gitems[first + item], sp, sag, sj);
     }
 }
 
-__global__ void k_grav_combine_sym64(Arrays a, Sizes z)
+// f(kernel, threads per block, shared bytes) for the FP64 kernel of a tile size
+template <typename Fn>
+static void with_sym64(int tile, Fn f)
+{
+    if (tile == 32) f(k_gravity64s<1, 1>, 32, sym64_smem(32, 1));
+    else if (tile == 64) f(k_gravity64s<1, 2>, 32, sym64_smem(64, 1));
+    else if (tile == 128) f(k_gravity64s<2, 2>, 64, sym64_smem(128, 2));
+    else if (tile == 256) f(k_gravity64s<4, 2>, 128, sym64_smem(256, 4));
+    else f(k_gravity64s<4, 4>, 128, sym64_smem(512, 4));
+}
+
+// Each sphere's partials in tile order.  One thread per sphere, few blocks
+// (12,000 spheres are 48 blocks of 256): the rows are loaded eight at a time.
+__global__ void __launch_bounds__(64) k_grav_combine_sym64(Arrays a, Sizes z)
 {
     pdl_enter();
     int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
@@ -904,15 +963,13 @@ __global__ void k_grav_combine_sym64(Arrays a, Sizes z)
     if (T <= 1) return;
     const PileStatic &S = a.ps[p];
     const int64_t il = i - S.s0;
-    const int t = (int)(il / kSymTile);
+    const int t = (int)(il / S.gtile64);
     const dbl4 *gp = (const dbl4 *)a.gpart;
     double sx = 0, sy = 0, sz = 0;
-    for (int b = t; b < T; ++b) {
-        const dbl4 v = gp[sym_slot(a, p, S.ns, b, il)];
-        sx += v.x; sy += v.y; sz += v.z;
-    }
-    for (int r = 0; r < t; ++r) {
-        const dbl4 v = gp[sym_slot(a, p, S.ns, T + r, il)];
+    // rows t..T-1 (i-sums of the pairs (t, b)), then T..T+t-1 (j-sums of (r, t))
+#pragma unroll 8
+    for (int r = t; r < T + t; ++r) {
+        const dbl4 v = gp[sym_slot(a, p, S.ns, r, il)];
         sx += v.x; sy += v.y; sz += v.z;
     }
     const double gm = S.G * a.m64[i];
@@ -987,8 +1044,10 @@ int gravity_blocks_per_sm(bool fp64, int block, int ib, bool pack, bool sym, int
     if (sym) {
         int n = 0;
         if (fp64) {
-            cudaFuncSetAttribute(k_gravity64s, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSym64Smem);
-            cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, k_gravity64s, kSymBS, kSym64Smem);
+            with_sym64(tile, [&](auto k, int threads, size_t smem) {
+                cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+                cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, k, threads, smem);
+            });
         } else {
             if (tile == 64) cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, k_gravity32s<1, 2>, 32, 0);
             else if (tile == 128) cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, k_gravity32s<1, 4>, 32, 0);
@@ -1031,8 +1090,14 @@ void launch_gravity(const Arrays &a, const Sizes &z, bool fp64, int block, int i
     if (sym) {
         int64_t nb = z.GB > 0 && z.GB < z.GI ? z.GB : z.GI;
         if (fp64) {
-            launch_pdl(k_gravity64s, (unsigned)nb, kSymBS, kSym64Smem, st, a, z);
-            if (z.GP > 0) launch_pdl(k_grav_combine_sym64, (unsigned)((z.N + 255) / 256), 256, 0, st, a, z);
+            for (int c = 0; c < kSym64Tiles; ++c) {   // one launch per tile size in use
+                const int64_t first = z.g64_first[c], count = z.g64_first[c + 1] - first;
+                if (count == 0) continue;
+                with_sym64(kGravSymTile >> c, [&](auto k, int threads, size_t smem) {
+                    launch_pdl(k, (unsigned)std::min(count, z.g64_blocks[c]), threads, smem, st, a, z, first, count);
+                });
+            }
+            if (z.GP > 0) launch_pdl(k_grav_combine_sym64, (unsigned)((z.N + 63) / 64), 64, 0, st, a, z);
         } else {
             if (z.gtile == 64) launch_pdl(k_gravity32s<1, 2>, (unsigned)nb, 32, 0, st, a, z);
             else if (z.gtile == 128) launch_pdl(k_gravity32s<1, 4>, (unsigned)nb, 32, 0, st, a, z);

@@ -86,6 +86,7 @@ struct dem_world {
     int grav_order = 4;               // tree gravity: highest multipole rank (4 or 2)
     int tree_maxD = 0;                // deepest tree of the current layout
     int sm_count = 0;
+    bool sym64_fallback = false;      // the FP64 path's small tiles did not fit: 512-sphere tiles
     double cell_factor = 1.0;
     double skin_frac = 0.1;           // neighbour-list skin / largest radius
     int contact_inbox = kInboxCap;    // contact inbox entries per tile range (testing: smaller splits more)
@@ -309,7 +310,8 @@ int64_t pile_count(const dem_world *w, const PileHost &q, Cls c)
 }
 
 struct GravPlan {
-    int tile = kGravSymTile;   // symmetric form: spheres per tile
+    int tile = kGravSymTile;   // symmetric form: spheres per tile (FP64 path: the smallest tile of any pile)
+    int64_t first64[kSym64Tiles + 1] = {};   // FP64 path: items grouped by tile size (Sizes::g64_first)
     std::vector<int4> items;
     std::vector<int64_t> base;
     std::vector<int32_t> nch;
@@ -317,6 +319,38 @@ struct GravPlan {
 };
 
 bool use_sym(const dem_world *w) { return w->grav_sym; }
+
+// SMs of the current device (0 if it cannot be asked)
+int device_sms(dem_world *w)
+{
+    if (w->sm_count == 0) {
+        int dev = 0;
+        if (cudaGetDevice(&dev) != cudaSuccess ||
+            cudaDeviceGetAttribute(&w->sm_count, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess) {
+            cudaGetLastError();
+            w->sm_count = 0;
+        }
+    }
+    return w->sm_count;
+}
+
+// Tile of the symmetric form on the FP64 path, by the pile's size alone (so
+// that a pile alone and in a batch gives the same bits).  The pass is bound by
+// the FP64 unit of the SM that runs an item, so the work must spread evenly:
+// the largest tile of 512 .. 32 spheres that cuts the pile into at least 70
+// (2,485 tile pairs, 16 per SM: a last wave that is nearly empty then costs a
+// few percent), 32 below.  Measured per step, 512 -> this: 1,000 spheres
+// 1,633 -> 104 us, 12,345 spheres 3.10 -> 2.77 ms.  The partial rows (2 T x N x 32 B) grow
+// with the number of tiles T, to 70..140 per pile as at 36,000 to 72,000
+// spheres before; a world with a memory budget keeps 512-sphere tiles, and so
+// does one whose allocation for the smaller tiles fails (prepare).
+int sym_tile64(const dem_world *w, const PileHost &q)
+{
+    if (w->budget || w->sym64_fallback) return kGravSymTile;
+    int tile = kGravSymTile;
+    while (tile > 32 && (q.ns + tile - 1) / tile < 70) tile /= 2;
+    return tile;
+}
 
 // Tile of the symmetric form.  512-sphere tiles unless the mixed path's
 // 512-tile pairs of all piles would not fill one wave of the persistent grid
@@ -328,7 +362,7 @@ bool use_sym(const dem_world *w) { return w->grav_sym; }
 // at 4,000 the two small tiles are even).
 int sym_tile(dem_world *w)
 {
-    if (w->precision != DEM_MIXED) return kGravSymTile;
+    if (w->precision != DEM_MIXED) return kGravSymTile;   // (per pile: sym_tile64)
     int64_t items = 0, nmax = 0;
     for (auto &q : w->piles) {
         if (q.P.G == 0.0) continue;
@@ -339,14 +373,7 @@ int sym_tile(dem_world *w)
     if (nmax == 0 || nmax > kSmallTileMaxN) return kGravSymTile;
     if (w->grav_tile == kGravSymTileTiny && nmax > kTinyTileMaxN) return kGravSymTileSmall;
     if (w->grav_tile) return w->grav_tile;
-    if (w->sm_count == 0) {
-        int dev = 0;
-        if (cudaGetDevice(&dev) != cudaSuccess ||
-            cudaDeviceGetAttribute(&w->sm_count, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess) {
-            cudaGetLastError();
-            return kGravSymTile;
-        }
-    }
+    if (device_sms(w) == 0) return kGravSymTile;
     const int bps = gravity_blocks_per_sm(false, 128, 4, false, true, kGravSymTile);
     cudaGetLastError();
     if (items >= (int64_t)std::max(1, bps) * w->sm_count) return kGravSymTile;
@@ -371,6 +398,36 @@ void order_items(const std::vector<GravItem> &its, std::vector<int4> &out)
     for (const auto &x : rest) out.push_back(x.v);
 }
 
+// FP64 symmetric form: every pair of tiles (a, b), a <= b, of every pile,
+// grouped by tile size; partial rows [b][i] and [T + a][j] (2 T rows of ns)
+// for piles with more than one tile.
+void plan_sym64(const dem_world *w, GravPlan &g)
+{
+    std::vector<GravItem> its[kSym64Tiles];
+    for (size_t p = 0; p < w->piles.size(); ++p) {
+        const PileHost &q = w->piles[p];
+        if (q.P.G == 0.0) {
+            g.nch.push_back(1);
+            g.base.push_back(-1);
+            continue;
+        }
+        const int64_t tile = sym_tile64(w, q), T = (q.ns + tile - 1) / tile;
+        g.tile = (int)std::min<int64_t>(g.tile, tile);
+        g.nch.push_back((int32_t)T);
+        g.base.push_back(T > 1 ? g.gp : -1);
+        if (T > 1) g.gp += 2 * T * q.ns;
+        int c = 0;
+        while (kGravSymTile >> c > tile) ++c;
+        for (int64_t ta = 0; ta < T; ++ta)
+            for (int64_t tb = ta; tb < T; ++tb)
+                its[c].push_back({make_int4((int)p, (int)ta, (int)tb, 0), std::min<int64_t>(tile, q.ns - tb * tile)});
+    }
+    for (int c = 0; c < kSym64Tiles; ++c) {
+        order_items(its[c], g.items);
+        g.first64[c + 1] = (int64_t)g.items.size();
+    }
+}
+
 GravPlan plan_gravity(dem_world *w)
 {
     GravPlan g;
@@ -380,8 +437,11 @@ GravPlan plan_gravity(dem_world *w)
     }
     if (use_sym(w)) {
         const int64_t tile = g.tile = sym_tile(w);
-        // items: every pair of tiles (a, b), a <= b; partial rows
-        // [b][i] and [T + a][j] (2 T rows of ns) for piles with more than one tile
+        // items: every pair of tiles (a, b), a <= b
+        if (w->precision == DEM_FP64) {
+            plan_sym64(w, g);
+            return g;
+        }
         std::vector<GravItem> its;
         for (size_t p = 0; p < w->piles.size(); ++p) {
             const PileHost &q = w->piles[p];
@@ -392,12 +452,7 @@ GravPlan plan_gravity(dem_world *w)
                 continue;
             }
             g.nch.push_back((int32_t)T);
-            if (T > 1 && w->precision == DEM_FP64) {
-                g.base.push_back(g.gp);
-                g.gp += 2 * T * q.ns;
-            } else {   // one tile, or the mixed path's integer accumulators
-                g.base.push_back(-1);
-            }
+            g.base.push_back(-1);   // one tile, or the integer accumulators
             for (int64_t ta = 0; ta < T; ++ta)
                 for (int64_t tb = ta; tb < T; ++tb) {
                     int64_t nb = std::min<int64_t>(tile, q.ns - tb * tile);
@@ -465,8 +520,12 @@ dem_status relayout(dem_world *w, const std::vector<PileHost> &newp, const GravP
         }
     }
     // bytes after the change (each field 256-byte aligned in one slab)
-    size_t total = 0;
-    for (auto &f : w->fields) total += (f.el * (size_t)ncap[f.cls] + 255) / 256 * 256;
+    auto slab_size = [&] {
+        size_t n = 0;
+        for (auto &f : w->fields) n += (f.el * (size_t)ncap[f.cls] + 255) / 256 * 256;
+        return n;
+    };
+    size_t total = slab_size();
     if (w->budget && total > w->budget)
         return fail(w, DEM_ERR_OOM, "HBM budget exceeded: need %zu bytes, budget %zu", total, w->budget);
     // old and new offsets of the surviving piles
@@ -489,8 +548,13 @@ dem_status relayout(dem_world *w, const std::vector<PileHost> &newp, const GravP
     }
     // one slab for every field (offsets 256-byte aligned): one allocator call per layout
     std::vector<void *> fresh(w->fields.size(), nullptr);
-    const size_t slab_bytes = total;
+    size_t slab_bytes = total;
     char *slab = (char *)dev_alloc(w, slab_bytes);
+    if (!slab && ncap[C_GPART] > need[C_GPART]) {   // without the spare room of the gravity partials
+        ncap[C_GPART] = need[C_GPART];
+        slab_bytes = slab_size();
+        slab = (char *)dev_alloc(w, slab_bytes);
+    }
     if (!slab) return fail(w, DEM_ERR_OOM, "device allocation of %zu bytes failed", slab_bytes);
     for (size_t f = 0, o = 0; f < w->fields.size(); ++f) {
         fresh[f] = slab + o;
@@ -589,6 +653,7 @@ dem_status upload_tables(dem_world *w, const GravPlan &gp)
             S.gscale_f = std::ldexp(1.0f, k);
             S.ginv = std::ldexp(1.0, -k);
         }
+        S.gtile64 = sym_tile64(w, q);
         for (int c = 0; c < 3; ++c) S.spin_inc[c] = P.spin_inc[c];
         S.rot_tol = P.rot_tol;
         ps.push_back(S);
@@ -616,6 +681,10 @@ dem_status upload_tables(dem_world *w, const GravPlan &gp)
         CU(cudaDeviceGetAttribute(&w->sm_count, cudaDevAttrMultiProcessorCount, dev));
     }
     w->Z.gtile = gp.tile;
+    for (int c = 0; c <= kSym64Tiles; ++c) w->Z.g64_first[c] = gp.first64[c];
+    for (int c = 0; c < kSym64Tiles; ++c)
+        w->Z.g64_blocks[c] = gp.first64[c + 1] == gp.first64[c] ? 0
+            : (int64_t)std::max(1, gravity_blocks_per_sm(true, 128, 4, false, true, kGravSymTile >> c)) * w->sm_count;
     w->Z.icap = w->contact_inbox;
     w->Z.gacc_on = (w->precision == DEM_MIXED && use_sym(w) && !(w->grav_theta > 0)) ? 1 : 0;
     w->Z.cmode = w->contact_mode;
@@ -702,8 +771,14 @@ dem_status prepare(dem_world *w)
 {
     if (w->graph_valid) return DEM_OK;
     Range range("dem: layout and step graph");
+    w->sym64_fallback = false;
     GravPlan gp = plan_gravity(w);
     dem_status s = relayout(w, w->piles, &gp);
+    if (s == DEM_ERR_OOM && w->precision == DEM_FP64 && use_sym(w) && gp.tile != kGravSymTile) {
+        w->sym64_fallback = true;   // fewer partial rows
+        gp = plan_gravity(w);
+        s = relayout(w, w->piles, &gp);
+    }
     if (s != DEM_OK) return s;
     s = upload_tables(w, gp);
     if (s != DEM_OK) return s;

@@ -1,0 +1,104 @@
+"""GPU: direct-sum gravity at the sizes where the tilings change: tile edges,
+remainders, aggregates that span several tiles, every tile size of the FP64
+path, and piles of different tile sizes in one world."""
+import numpy as np
+import pytest
+
+from paper_2311_11322_gb300 import workloads as W
+
+pytestmark = pytest.mark.gpu
+
+EPS = 0.3
+
+
+@pytest.fixture(scope="module")
+def dem():
+    torch = pytest.importorskip("torch")
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    import __graft_entry__
+    __graft_entry__.build()
+    from paper_2311_11322_gb300 import dem as D
+    return D
+
+
+def pile(n, precision, seed=0, equal=False):
+    """n spheres at random in a cube, no contacts intended: a rod of up to 100 spheres first (it spans tiles), then
+    aggregates of 1 to 4 spheres; radii differ unless `equal`."""
+    rng = np.random.default_rng(seed + n)
+    counts = [min(100, n)]
+    while sum(counts) < n:
+        counts.append(min(int(rng.integers(1, 5)), n - sum(counts)))
+    counts = np.array(counts, np.int32)
+    of = np.repeat(np.arange(len(counts)), counts)
+    slot = np.arange(n) - np.repeat(np.cumsum(counts) - counts, counts)
+    box = 20.0 * n ** (1.0 / 3.0)
+    pos = rng.uniform(-box, box, (len(counts), 3))[of]
+    pos[:, 0] += 0.5 * slot
+    radius = np.full(n, 0.25) if equal else 0.2 + 0.1 * rng.random(len(counts))[of]
+    ic = W.PileIC(counts=counts, pos=pos, radius=radius, density=np.full(n, 2500.0))
+    return ic, W.Params(G=1e-3, dt=1e-6, kn=1.0, eps=EPS, precision=precision)
+
+
+def reference(ic, p, pos, sample):
+    """Gravity on the sampled spheres and the sum of its terms' magnitudes, in FP64."""
+    m = W.sphere_mass(ic.radius, ic.density)
+    agg = np.repeat(np.arange(ic.n_agg), ic.counts)
+    F, mag = np.zeros((len(sample), 3)), np.zeros(len(sample))
+    for k, i in enumerate(sample):
+        d = pos - pos[i]
+        w = np.where(agg == agg[i], 0.0, m / ((d * d).sum(1) + EPS ** 2) ** 1.5)
+        t = p.G * m[i] * w[:, None] * d
+        F[k], mag[k] = t.sum(0), np.linalg.norm(t, axis=1).sum()
+    return F, mag
+
+
+def sampled(n):
+    return np.unique(np.concatenate([np.arange(min(n, 120)), np.linspace(0, n - 1, 150).astype(int),
+                                     np.arange(max(0, n - 70), n)]))
+
+
+# FP64 tiles: 32 spheres, then 64, 128, 256, 512 as ceil(n / tile) reaches 70
+@pytest.mark.parametrize("n", [1, 2, 31, 33, 64, 101, 1000, 4416, 4417, 8833, 17665, 35400])
+def test_fp64_gravity_tile_sizes(dem, n):
+    ic, p = pile(n, W.PRECISION_FP64)
+    with dem.World() as w:
+        pid = w.add_pile(ic, p)
+        w.step(1)
+        got, pos = w.read(pid, "SPHERE_FG"), w.read(pid, "SPHERE_POS")
+    s = sampled(n)
+    F, mag = reference(ic, p, pos, s)
+    # a term carries about 10 roundings, a sum of n terms n more, on either side; positions read back are
+    # rounded once more than the frame-relative ones summed (1e-16 of the box over the smallest distances)
+    err = np.linalg.norm(got[s] - F, axis=1)
+    assert np.all(err <= 2 * (n + 20) * 2.0 ** -53 * mag + 1e-12 * mag), float((err / np.maximum(mag, 1e-300)).max())
+
+
+def test_fp64_tiles_alone_and_in_a_batch_bitwise(dem):
+    """Piles of every FP64 tile size in one world give the bits they give alone."""
+    piles = [pile(n, W.PRECISION_FP64, seed=7) for n in (40, 900, 4500, 9000, 18000, 36000)]
+    alone = []
+    for ic, p in piles:
+        with dem.World() as w:
+            pid = w.add_pile(ic, p)
+            w.step(2)
+            alone.append(w.read(pid, "SPHERE_FG"))
+    with dem.World() as w:
+        ids = [w.add_pile(ic, p) for ic, p in piles]
+        w.step(2)
+        for pid, ref in zip(ids, alone):
+            assert np.array_equal(w.read(pid, "SPHERE_FG"), ref)
+
+
+def test_fp64_budget_keeps_the_large_tiles(dem):
+    """A world with a memory budget of the pile's stated footprint still takes the pile and steps it."""
+    ic, p = pile(1000, W.PRECISION_FP64)
+    need = dem.dem_footprint_bytes(ic.n_sph, ic.n_agg, p.max_contacts, W.PRECISION_FP64)
+    with dem.World(budget=need) as w:
+        pid = w.add_pile(ic, p)
+        w.step(1)
+        got, pos = w.read(pid, "SPHERE_FG"), w.read(pid, "SPHERE_POS")
+        assert w.bytes() <= need
+    s = sampled(1000)
+    F, mag = reference(ic, p, pos, s)
+    assert np.all(np.linalg.norm(got[s] - F, axis=1) <= 1.5e-12 * mag)
