@@ -127,7 +127,11 @@ enum dem_field {
 enum { DEM_FLAG_SLOTS = 1, DEM_FLAG_NONFINITE = 2, DEM_FLAG_OVERLAP = 4, DEM_FLAG_TREE = 8,
        DEM_FLAG_GRAV_RANGE = 16 };
 
-/* Kernels that dem_step_profiled can time. */
+/* Kernels that dem_step_profiled can time.  AGG_BEGIN includes the pile's
+ * opening reduction, AGG_END its closing one, and GATHER the whole way from
+ * aggregates to sorted spheres, with the cell sort and the candidate lists in
+ * the steps that rebuild them: PILE_BEGIN, KEYS, SCAN, SCATTER, CELL_ORDER and
+ * PILE_END have no kernel of their own (their times read 0). */
 enum dem_kernel {
     DEM_K_AGG_BEGIN = 0, DEM_K_PILE_BEGIN = 1, DEM_K_KEYS = 2, DEM_K_SCAN = 3, DEM_K_SCATTER = 4,
     DEM_K_CELL_ORDER = 5, DEM_K_GATHER = 6, DEM_K_CONTACT = 7, DEM_K_GRAVITY = 8,
@@ -276,13 +280,11 @@ dem_status dem_remove_pile(dem_world *w, int32_t pile_id);
  * when grav_ib is even, 0 = scalar FP32), "grav_sym" (1 = symmetric
  * tile-pair form, each pair evaluated once and applied to both spheres, the
  * default in both precisions; 0 = one-sided form shaped by the keys above),
- * "grav_tile" (spheres per tile of the symmetric form in the mixed path:
- * 512, or 128 or 256 for worlds whose piles all have at most 8,192 spheres,
- * or 64 when they have at most 2,048 -- more, smaller work items when the
- * 512-sphere tile pairs would not fill the GPU; 0 = choose automatically
- * (when the 512-sphere tile pairs of all piles fill less than one wave of
- * the persistent grid: 64 up to 2,048 spheres, else 128), the default;
- * larger piles always use 512),
+ * "grav_tile" (spheres per tile of the symmetric form in the mixed path: 64,
+ * 128, 256 or 512; a size whose pairs would number more than 2^20 is doubled
+ * until they do not; 0 = choose automatically, the default: 64 in worlds
+ * whose piles all have at most 8,192 spheres and whose 512-sphere tile pairs
+ * would fill less than one wave, else 256),
  * "grav_theta" (mixed path: > 0 replaces the direct sum by tree gravity with
  * this opening angle, in [0, 1): cells of an octree rebuilt every step with
  * multipoles up to the hexadecapole (Sec. 2.1), leaves of ~4 spheres summed

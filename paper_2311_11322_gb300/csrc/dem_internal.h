@@ -19,8 +19,9 @@ __host__ __device__ __forceinline__ dbl4 make_dbl4(double x, double y, double z,
 
 constexpr int kMaxK = 64;          // largest max_contacts
 constexpr int kScanTile = 2048;    // cells per scan block (256 threads x 8)
-constexpr int kAggChunk = 512;     // aggregates per pile-reduction block
+constexpr int kAggChunk = 512;     // aggregates per chunk of a pile reduction
 constexpr int kPartialDoubles = 16;
+constexpr int kChunkWarps = kAggChunk / 32;
 // Contact pass: tiles of consecutive sorted spheres, one block each; the
 // candidate lists of a pile hold kEntPerSphere entries per sphere on average
 // at the default skin (more for larger skins, in proportion to the candidate
@@ -79,6 +80,8 @@ struct PileStatic {
     // a sphere's sum of |terms|) <= 2^61, |k| <= 120); ginv = 1 / gscale
     double ginv;
     float gscale_f;
+    float umass;           // the spheres' mass in FP32 if all have the same, else 0
+    int32_t pad_u;
     int32_t gtile64;       // FP64 symmetric form: spheres per tile of this pile
     // the contact law's constants in FP32 for the mixed path (kn, kt, cn, ct,
     // mu_s, mu_r, mu_t, w0, h), rounded once on the host
@@ -153,7 +156,6 @@ struct Arrays {
     double *s64, *m64;   // radius, mass
     float4 *bh, *bl;     // mixed: body offset hi/lo with radius hi/lo in .w
     int32_t *key;        // cell index within the pile
-    int32_t *rank;       // rank among spheres counted into the same cell
     int32_t *sorted;     // sorted position (pile-local) -> home index (pile-local)
     // sorted copies for the contact pass
     // mixed: per sphere two 16-byte halves of one 32-byte sector each:
@@ -164,7 +166,8 @@ struct Arrays {
     float4 *svw;
     float4 *sph_;                   // mixed: pos hi (+s hi; rebuild steps only)
     dbl4 *dp_, *dv_, *dw_;          // fp64: pos (+s), vel (+agg), spin (+home id)
-    int32_t *sagg;                  // aggregate (pile-local) of each sorted position
+    int32_t *sagg;                  // aggregate (pile-local) of each sorted position (while a rebuild
+                                    // sorts: each home sphere's rank in its cell)
     // candidate lists (compressed rows per sorted sphere, entries in the
     // order of the partners' home indices), double-buffered by PileDyn::cpar
     // so that a rebuild can carry the history over from the previous lists:
@@ -174,14 +177,15 @@ struct Arrays {
     int32_t *ccnt[2], *coff[2];
     int2 *cand[2];
     int32_t *cand_id[2];
-    // contact tiles: (pile slot, first sorted position, spheres, 0); entries
-    // of each tile and their pile-local base (rebuild steps)
+    // contact tiles: (pile slot, first sorted position, spheres, 0); entries of
+    // each tile's four 32-sphere slices and their pile-local base (rebuild steps)
     int4 *ctile;
     int32_t *ctile_cnt, *ctile_base;
     // gravity inputs / outputs
     float4 *gpos32;      // mixed: pos hi (+mass)
     dbl4 *gpos64;     // fp64: pos (+mass)
     dbl4 *fg;         // gravity on each sphere (from other aggregates)
+    dbl4 *fe;         // mixed, worlds with a planet: its force on each sphere
     // contact outputs at each sphere's home index, interleaved: [2i] = force, [2i+1] = torque
     float4 *ftc32;
     dbl4 *ftc64;
@@ -216,10 +220,12 @@ struct Arrays {
     float *aref;
     // cells
     int32_t *ccount, *cstart, *tile_sum;
+    unsigned *lbar;                // barrier words of k_lists (zero between launches)
     // pile reductions
     double *chunk_part;            // [chunks][kPartialDoubles]
     int32_t *chunk_pile;           // [chunks] pile slot of each chunk
-    int32_t *pile_arrive;          // [piles] chunk blocks of a reduction finished so far (0 between launches)
+    double *warp_part;             // [chunks][kChunkWarps][3] the planet's force by 32 aggregates
+    int32_t *pile_arrive;          // [piles] blocks of a closing reduction finished so far (0 between launches)
     double *bulk_part;             // [chunks][32] bulk-shape sums (kBulkParts used)
     PileWatch *watch;              // [piles]
     // gravity work list and j-chunk partial sums
@@ -257,41 +263,39 @@ struct Sizes {
     int64_t TN, TL, TG;   // tree nodes, leaves and 32-sphere groups of all piles (TN = 0: direct sum)
     int32_t K;    // history slots per sphere (world-wide)
     int32_t adapt;   // some pile integrates rotation with the adaptive RK5(4)
-    int32_t gtile;   // spheres per tile of the symmetric gravity form (512, or 128 in the mixed path)
+    int32_t gtile;   // spheres per tile of the symmetric gravity form (mixed path)
     int32_t icap;    // contact inbox entries used per tile range (<= the kernel's capacity)
     int32_t cmode;   // contact pass: 0 = one thread per sphere, 1 = tiles with a shared-memory inbox
     int32_t gacc_on; // mixed symmetric gravity: piles of more than one tile leave their sums in gacc,
-                     // which k_grav_acc_to_force turns into forces
+                     // which k_grav_acc_to_force (1) or k_agg_end (2) turns into forces
     int32_t grav;    // some pile has self-gravity (G > 0)
     // FP64 symmetric form: items of the piles with tiles of 512 >> c spheres
     // are [g64_first[c], g64_first[c + 1]), run by at most g64_blocks[c] blocks
     int64_t g64_first[6], g64_blocks[5];
+    int64_t LB;      // blocks of k_lists that are resident at once
 };
 
 // ---- kernel launchers (kernels_*.cu) -------------------------------------
 void launch_agg_begin(const Arrays &a, const Sizes &z, bool fp64, cudaStream_t st);
-void launch_pile_begin(const Arrays &a, const Sizes &z, cudaStream_t st);
-void launch_keys(const Arrays &a, const Sizes &z, bool fp64, cudaStream_t st);
-void launch_scan(const Arrays &a, const Sizes &z, cudaStream_t st);
-void launch_scatter(const Arrays &a, const Sizes &z, cudaStream_t st);
-void launch_cell_order(const Arrays &a, const Sizes &z, cudaStream_t st);
-void launch_gather(const Arrays &a, const Sizes &z, bool fp64, cudaStream_t st);
+void launch_lists(const Arrays &a, const Sizes &z, bool fp64, cudaStream_t st);
+int lists_blocks_per_sm(bool fp64);
 void launch_contact(const Arrays &a, const Sizes &z, bool fp64, int K, cudaStream_t st);
 cudaError_t contact_setup(bool fp64, int K);
 // sym: symmetric tile-pair form (items are (pile, tile a, tile b), gnchunk =
-// tiles per pile); tiles of 512 spheres, or of 128 (mixed path, small piles)
-constexpr int kGravSymTile = 512, kGravSymTileSmall = 128, kGravSymTileTiny = 64;
-constexpr int64_t kTinyTileMaxN = 2048;   // largest pile that may use 64-sphere tiles
-// largest pile (spheres) of a world that may use tiles smaller than 512
-#ifndef DEM_SMALL_TILE_MAX
-#define DEM_SMALL_TILE_MAX 8192
-#endif
-constexpr int64_t kSmallTileMaxN = DEM_SMALL_TILE_MAX;
+// tiles per pile)
+constexpr int kGravSymTile = 512, kGravSymTileLarge = 256, kGravSymTileTiny = 64;
+constexpr int64_t kTinyTileMaxN = 8192;   // largest pile (spheres) whose world may use 64-sphere tiles by itself
+constexpr int64_t kSymMaxItems = 1 << 20; // longest work list a tuned tile size may make
+// worlds in which k_agg_end turns the gravity sums into forces itself: a
+// thread converts its members' sums one after the other, which costs less than
+// a launch while the whole world is a wave of blocks.  Measured per step, with
+// the kernel of its own -> without: 7,466 spheres 66.1 -> 64.8 us, 1,000 and
+// 20,000 the same; on 256 piles k_agg_end was four times slower.
+constexpr int64_t kGaccFuseMax = 8192;
 void launch_gravity(const Arrays &a, const Sizes &z, bool fp64, int block, int ib, bool pack,
                     bool sym, cudaStream_t st);
 int gravity_blocks_per_sm(bool fp64, int block, int ib, bool pack, bool sym, int tile);
 void launch_agg_end(const Arrays &a, const Sizes &z, bool fp64, cudaStream_t st);
-void launch_pile_end(const Arrays &a, const Sizes &z, cudaStream_t st);
 void launch_fill_ids(const Arrays &a, const Sizes &z, cudaStream_t st);
 // order: highest multipole rank of accepted cells (2 or 4)
 void launch_tree_gravity(const Arrays &a, const Sizes &z, int max_depth, int order, cudaStream_t st);

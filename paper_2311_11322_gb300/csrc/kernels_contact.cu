@@ -5,15 +5,13 @@
 // the contact point at the centre of the intersection circle (Sec. 2.2.4,
 // Eq. lever_arm).
 //
-// Candidate lists.  At a rebuild (a new cell sort) every sphere lists the
-// spheres of other aggregates whose centres are closer than the radii sum
+// Candidate lists (built in kernels_lists.cu): at a rebuild every sphere lists
+// the spheres of other aggregates whose centres are closer than the radii sum
 // plus the skin, in the order of their home indices, in compressed rows per
-// sorted sphere (k_cand_count, k_cand_scan, k_cand_fill); k_cand_link then
-// gives every entry the position of the same pair in the partner's list and
-// marks the entries whose sphere owns the pair (the lower home index).  The
-// lists stay complete until some aggregate may have moved half the skin
-// (checked at the drift).  The candidate test is exact and symmetric, so
-// both spheres of a pair always list each other.
+// sorted sphere; every entry has the position of the same pair in the
+// partner's list and whether its sphere owns the pair (the lower home index).
+// The lists stay complete until some aggregate may have moved half the skin
+// (checked at the drift).
 //
 // Shares of a pair.  Both spheres' shares come from one evaluation with the
 // owner as sphere a:
@@ -66,6 +64,7 @@
 #include "dem_internal.h"
 #include "devmath.cuh"
 #include "launch.cuh"
+#include "reduce.cuh"
 
 namespace dem {
 
@@ -296,384 +295,10 @@ template <> struct CT<true> {
     static constexpr int kCap = kInboxCap / 2;
 };
 
-__device__ __forceinline__ bool pile_live(const Arrays &a, int p)
-{
-    return a.enabled[p] != 0 && a.pd[p].failed == 0;
-}
-
-__device__ __forceinline__ int wrapc(int c, int n) { return c < 0 ? c + n : (c >= n ? c - n : c); }
-
-__device__ __forceinline__ int cellc_f(float x, float inv_cell, int n)
-{
-    float f = floorf(__fmul_rn(x, inv_cell));
-    f = fminf(fmaxf(f, -1.0e9f), 1.0e9f);
-    int m = ((int)f) % n;
-    return m < 0 ? m + n : m;
-}
-
-__device__ __forceinline__ int cellc_d(double x, double inv_cell, int n)
-{
-    double f = floor(__dmul_rn(x, inv_cell));
-    f = fmin(fmax(f, -1.0e9), 1.0e9);
-    int m = ((int)f) % n;
-    return m < 0 ? m + n : m;
-}
-
 __device__ __forceinline__ float pow2f(int e) { return __int_as_float((e + 127) << 23); }
 __device__ __forceinline__ float4 as_f4(int4 v)
 {
     return make_float4(__int_as_float(v.x), __int_as_float(v.y), __int_as_float(v.z), __int_as_float(v.w));
-}
-
-// Candidate test of sphere k (own data) against sorted position kk.  Exact and
-// symmetric: swapping the spheres gives the same answer.
-struct CandMe {
-    int4 xq;        // mixed
-    float4 ph;      // mixed: position hi, radius hi
-    dbl4 p;         // fp64
-    int agg;
-};
-
-template <bool FP64>
-__device__ __forceinline__ bool cand_test(const Arrays &a, const PileStatic &S, const CandMe &m, int64_t kk)
-{
-    if constexpr (FP64) {
-        const dbl4 q = a.dp_[kk];
-        const double dx = q.x - m.p.x, dy = q.y - m.p.y, dz = q.z - m.p.z;
-        const double t = m.p.w + q.w + S.skin;
-        return __fma_rn(dz, dz, __fma_rn(dy, dy, __dmul_rn(dx, dx))) < __dmul_rn(t, t);
-    } else {
-        // FP32 test first (it rejects the spheres of other wraps of the grid,
-        // whose 32-bit fixed-point difference would alias): the FP32 centres
-        // are the rounded float-float positions, so a margin of a few units in
-        // the last place of both keeps every candidate; the margin depends on
-        // both spheres alike, so the test stays symmetric
-        const float4 q = a.sph_[kk];
-        const float dx = __fsub_rn(q.x, m.ph.x), dy = __fsub_rn(q.y, m.ph.y), dz = __fsub_rn(q.z, m.ph.z);
-        const float big = __fadd_rn(fmaxf(fabsf(q.x), fmaxf(fabsf(q.y), fabsf(q.z))),
-                                    fmaxf(fabsf(m.ph.x), fmaxf(fabsf(m.ph.y), fabsf(m.ph.z))));
-        const float sr = __fadd_rn(q.w, m.ph.w);
-        const float tc = __fadd_rn(__fadd_rn(sr, (float)S.skin), __fmaf_rn(1e-6f, big, __fmul_rn(1e-5f, sr)));
-        if (!(__fmaf_rn(dz, dz, __fmaf_rn(dy, dy, __fmul_rn(dx, dx))) < __fmul_rn(tc, tc))) return false;
-        const int4 B = a.xqr[2 * kk];
-        const int ex = (int)((unsigned)B.x - (unsigned)m.xq.x);
-        const int ey = (int)((unsigned)B.y - (unsigned)m.xq.y);
-        const int ez = (int)((unsigned)B.z - (unsigned)m.xq.z);
-        const long long D = (long long)ex * ex + (long long)ey * ey + (long long)ez * ez;
-        // two quanta more than the skin: the rounding remainders cannot hide a contact
-        const long long t = (long long)m.xq.w + B.w + S.skin_q + 2;
-        return D < t * t;
-    }
-}
-
-// Visit every sphere of the 27 neighbour cells of sorted position k (the
-// three x-neighbours of a (y, z) row as one index range when they are
-// consecutive), calling f(kk) for the candidates.
-template <bool FP64, typename Fn>
-__device__ __forceinline__ void for_candidates(const Arrays &a, const PileStatic &S, int64_t k,
-                                               const CandMe &m, Fn f)
-{
-    int cx, cy, cz;
-    if constexpr (FP64) {
-        cx = cellc_d(m.p.x, S.inv_cell, S.nx);
-        cy = cellc_d(m.p.y, S.inv_cell, S.ny);
-        cz = cellc_d(m.p.z, S.inv_cell, S.nz);
-    } else {
-        const float ic = (float)S.inv_cell;
-        cx = cellc_f(m.ph.x, ic, S.nx);
-        cy = cellc_f(m.ph.y, ic, S.ny);
-        cz = cellc_f(m.ph.z, ic, S.nz);
-    }
-    const int32_t *cstart = a.cstart + S.c0, *ccount = a.ccount + S.c0;
-    const int64_t s0 = S.s0;
-    // without wrap-around the three x-neighbours are consecutive cell ids
-    // except across a brick boundary: one or two index ranges
-    const bool nowrap = cx >= 1 && cx + 1 < S.nx;
-    const int split = (cx & 3) == 0 ? 1 : (cx & 3) == 3 ? 2 : 3;   // first cell of the second range
-    for (int dz = -1; dz <= 1; ++dz)
-        for (int dy = -1; dy <= 1; ++dy) {
-            const int yy = wrapc(cy + dy, S.ny), zz = wrapc(cz + dz, S.nz);
-            int beg[3], end[3], nr;
-            if (nowrap) {
-                const int64_t cl = cell_id(cx - 1, yy, zz, S.nx, S.ny);
-                const int64_t cs = cell_id(cx - 1 + split, yy, zz, S.nx, S.ny);
-                const int64_t ce = cell_id(cx + 1, yy, zz, S.nx, S.ny);
-                if (split == 3) {
-                    beg[0] = cstart[cl];
-                    end[0] = cstart[ce] + ccount[ce];
-                    nr = 1;
-                } else {
-                    const int64_t cm = split == 1 ? cl : cell_id(cx, yy, zz, S.nx, S.ny);
-                    beg[0] = cstart[cl];
-                    end[0] = cstart[cm] + ccount[cm];
-                    beg[1] = cstart[cs];
-                    end[1] = cstart[ce] + ccount[ce];
-                    nr = 2;
-                }
-            } else {
-                nr = 0;
-                for (int ddx = -1; ddx <= 1; ++ddx) {
-                    const int64_t c = cell_id(wrapc(cx + ddx, S.nx), yy, zz, S.nx, S.ny);
-                    beg[nr] = cstart[c];
-                    end[nr] = cstart[c] + ccount[c];
-                    ++nr;
-                }
-            }
-            for (int r = 0; r < nr; ++r)
-                for (int t = beg[r]; t < end[r]; ++t) {
-                    const int64_t kk = s0 + t;
-                    if (kk == k || a.sagg[kk] == m.agg) continue;
-                    if (cand_test<FP64>(a, S, m, kk)) f(t);
-                }
-        }
-}
-
-template <bool FP64>
-__device__ __forceinline__ void load_me(const Arrays &a, int64_t k, CandMe &m)
-{
-    if constexpr (FP64) m.p = a.dp_[k];
-    else {
-        m.xq = a.xqr[2 * k];
-        m.ph = a.sph_[k];
-    }
-    m.agg = a.sagg[k];
-}
-
-// ---------------------------------------------------------------- rebuild
-__device__ __forceinline__ bool tile_rebuilds(const Arrays &a, int4 tl)
-{
-    return pile_live(a, tl.x) && a.pd[tl.x].rebuild;
-}
-
-// Whether any pile rebuilds this step (the block's threads read the piles'
-// flags together): in most steps no pile does, and the rebuild kernels end here.
-__device__ __forceinline__ bool any_rebuild(const Arrays &a, const Sizes &z)
-{
-    int mine = 0;
-    for (int p = threadIdx.x; p < z.P; p += blockDim.x) mine |= pile_live(a, p) && a.pd[p].rebuild;
-    return __syncthreads_or(mine) != 0;
-}
-
-// Candidates per sphere (new list buffer) and per tile.
-template <bool FP64>
-__global__ void __launch_bounds__(kCTile) k_cand_count(Arrays a, Sizes z)
-{
-    pdl_enter();
-    __shared__ int red[kCTile / 32];
-    if (!any_rebuild(a, z)) return;
-    for (int64_t tile = blockIdx.x; tile < z.CT; tile += gridDim.x) {
-    const int4 tl = a.ctile[tile];
-    if (!tile_rebuilds(a, tl)) continue;
-    const int p = tl.x;
-    const PileStatic &S = a.ps[p];
-    const int lp = a.pd[p].cpar ^ 1;
-    int n = 0;
-    if ((int)threadIdx.x < tl.z) {
-        const int64_t k = S.s0 + tl.y + threadIdx.x;
-        CandMe m;
-        load_me<FP64>(a, k, m);
-        for_candidates<FP64>(a, S, k, m, [&](int) { ++n; });
-        a.ccnt[lp][k] = n;
-    }
-    // entries of the tile: every slice of 32 spheres (a warp) is as wide as
-    // its longest list
-    const int wmax = __reduce_max_sync(0xffffffffu, n);
-    if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = 32 * wmax;
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        int s = 0;
-        for (int w = 0; w < kCTile / 32; ++w) s += red[w];
-        a.ctile_cnt[tile] = s;
-    }
-    __syncthreads();   // red[] is reused by the next tile
-    }
-}
-
-// One block per pile: exclusive scan of the tiles' entry counts.  Lists that
-// do not fit the pile's entries flag the pile (frozen at the end of the step).
-__global__ void __launch_bounds__(1024) k_cand_scan(Arrays a, Sizes z)
-{
-    pdl_enter();
-    const int p = blockIdx.x;
-    if (!pile_live(a, p) || !a.pd[p].rebuild) return;
-    const PileStatic &S = a.ps[p];
-    __shared__ long long buf[1024];
-    __shared__ long long carry;
-    if (threadIdx.x == 0) carry = 0;
-    __syncthreads();
-    for (int64_t base = 0; base < S.nct; base += 1024) {
-        const int64_t t = base + threadIdx.x;
-        const long long v = t < S.nct ? a.ctile_cnt[S.ct0 + t] : 0;
-        buf[threadIdx.x] = v;
-        __syncthreads();
-        for (int o = 1; o < 1024; o <<= 1) {
-            const long long add = threadIdx.x >= (unsigned)o ? buf[threadIdx.x - o] : 0;
-            __syncthreads();
-            buf[threadIdx.x] += add;
-            __syncthreads();
-        }
-        const long long incl = buf[threadIdx.x];
-        if (t < S.nct) a.ctile_base[S.ct0 + t] = (int32_t)(carry + incl - v);
-        __syncthreads();
-        if (threadIdx.x == 1023) carry += incl;
-        __syncthreads();
-    }
-    if (threadIdx.x == 0 && carry > S.ne) {
-        atomicOr(&a.pd[p].flags, DEM_FLAG_SLOTS);
-        for (int64_t t = 0; t < S.nct; ++t) a.ctile_base[S.ct0 + t] = -1;
-    }
-}
-
-// Offsets, then the candidates themselves, sorted by partner home index.
-// Sliced layout: the 32 spheres of a slice (a warp) store entry e of their
-// lists side by side, so sphere k's entry e is at coff[k] + 32 e (coalesced
-// when a warp walks its lists together).
-constexpr int kFillCap = 20;   // candidates sorted in shared memory per sphere (more: in place)
-
-template <bool FP64>
-__device__ __forceinline__ void cand_fill_tile(const Arrays &a, int4 tl, int base, int *sw,
-                                               int2 (*s_list)[kCTile])
-{
-    const int p = tl.x;
-    const PileStatic &S = a.ps[p];
-    const int lp = a.pd[p].cpar ^ 1;
-    const bool mine = (int)threadIdx.x < tl.z;
-    const int64_t k = S.s0 + tl.y + threadIdx.x;
-    const int n = mine ? a.ccnt[lp][k] : 0;
-    const int wmax = __reduce_max_sync(0xffffffffu, n);
-    const int wid = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    if (lane == 0) sw[wid] = 32 * wmax;
-    __syncthreads();
-    int sb = base;
-    for (int w = 0; w < wid; ++w) sb += sw[w];
-    if (!mine) return;
-    const int off = sb + lane;
-    a.coff[lp][k] = off;
-    int32_t *ids = a.cand_id[lp] + S.e0 + off;
-    int2 *cd = a.cand[lp] + S.e0 + off;
-    const int32_t *srt = a.sorted + S.s0;
-    CandMe m;
-    load_me<FP64>(a, k, m);
-    int j = 0;
-    if (n <= kFillCap) {
-        // insertion by partner home index in shared memory, then one write
-        int2 *l = &s_list[0][threadIdx.x];
-        for_candidates<FP64>(a, S, k, m, [&](int t) {
-            if (j >= n) return;   // (the count pass visited the same candidates)
-            const int id = srt[t];
-            int y = j++;
-            while (y > 0 && l[(y - 1) * kCTile].x > id) {
-                l[y * kCTile] = l[(y - 1) * kCTile];
-                --y;
-            }
-            l[y * kCTile] = make_int2(id, t);
-        });
-        for (int y = 0; y < j; ++y) {
-            const int2 v = l[y * kCTile];
-            ids[32 * y] = v.x;
-            cd[32 * y] = make_int2(v.y, 0);
-        }
-        return;
-    }
-    for_candidates<FP64>(a, S, k, m, [&](int t) {
-        if (j >= n) return;
-        // long list: insertion by partner home index in place
-        const int id = srt[t];
-        int y = j++;
-        while (y > 0 && ids[32 * (y - 1)] > id) {
-            ids[32 * y] = ids[32 * (y - 1)];
-            cd[32 * y] = cd[32 * (y - 1)];
-            --y;
-        }
-        ids[32 * y] = id;
-        cd[32 * y] = make_int2(t, 0);
-    });
-}
-
-template <bool FP64>
-__global__ void __launch_bounds__(kCTile) k_cand_fill(Arrays a, Sizes z)
-{
-    pdl_enter();
-    __shared__ int sw[kCTile / 32];
-    __shared__ int2 s_list[kFillCap][kCTile];   // (partner home index, sorted position)
-    if (!any_rebuild(a, z)) return;
-    for (int64_t tile = blockIdx.x; tile < z.CT; tile += gridDim.x) {
-        __syncthreads();   // sw[] of the previous tile
-        const int4 tl = a.ctile[tile];
-        if (!tile_rebuilds(a, tl)) continue;
-        const int base = a.ctile_base[tile];
-        if (base < 0) continue;
-        cand_fill_tile<FP64>(a, tl, base, sw, s_list);
-    }
-}
-
-
-// Owner bit and mirror entry of every list entry; history carried from the
-// previous lists (by the home indices of both spheres) into hist_rm.
-template <bool FP64>
-__device__ __forceinline__ void cand_link_sphere(const Arrays &a, int4 tl)
-{
-    typedef typename CT<FP64>::H H;
-    const int p = tl.x;
-    const PileStatic &S = a.ps[p];
-    const PileDyn &D = a.pd[p];
-    const int lp = D.cpar ^ 1, op = D.cpar, par = D.parity;
-    const int64_t s0 = S.s0, e0 = S.e0;
-    const int kl = tl.y + threadIdx.x;
-    const int me = a.sorted[s0 + kl];
-    const int n = a.ccnt[lp][s0 + kl], off = a.coff[lp][s0 + kl];
-    // the previous list of this home sphere
-    const int kprev = a.pos_of_home[par][s0 + me];
-    const int pn = a.ccnt[op][s0 + kprev], poff = a.coff[op][s0 + kprev];
-    const int32_t *pids = a.cand_id[op] + e0 + poff;
-    const H *hprev;
-    H *hrm;
-    if constexpr (FP64) { hprev = a.hist64[par] + e0; hrm = a.hist64_rm + e0; }
-    else { hprev = a.hist32[par] + e0; hrm = a.hist32_rm + e0; }
-    int cursor = 0;
-    for (int e = 0; e < n; ++e) {
-        const int f = off + 32 * e;
-        const int2 c = a.cand[lp][e0 + f];
-        const int kk = c.x;
-        const int id = a.cand_id[lp][e0 + f];
-        // my entry in the partner's list: binary search by home index
-        const int pn2 = a.ccnt[lp][s0 + kk], po2 = a.coff[lp][s0 + kk];
-        const int32_t *ids2 = a.cand_id[lp] + e0 + po2;
-        int lo = 0, hi = pn2 - 1, mir = -1;
-        while (lo <= hi) {
-            const int mid = (lo + hi) >> 1;
-            const int v = ids2[32 * mid];
-            if (v == me) { mir = po2 + 32 * mid; break; }
-            if (v < me) lo = mid + 1; else hi = mid - 1;
-        }
-        if (mir < 0) atomicOr(&a.pd[p].flags, DEM_FLAG_SLOTS);   // lists not symmetric: cannot happen
-        const bool owned = me < id;
-        a.cand[lp][e0 + f] = make_int2(kk | (owned ? (int)0x80000000u : 0), mir < 0 ? 0 : mir);
-        if (!owned) continue;
-        // carried history: the same partner in the previous list (both lists
-        // are in partner order, so one forward cursor finds it)
-        H h;
-        if constexpr (FP64) h = make_dbl4(0.0, 0.0, 0.0, 0.0);
-        else h = make_float4(0.f, 0.f, 0.f, 0.f);
-        while (cursor < pn && pids[32 * cursor] < id) ++cursor;
-        if (cursor < pn && pids[32 * cursor] == id) {
-            const H g = hprev[poff + 32 * cursor];
-            if (g.w != 0) h = g;
-        }
-        hrm[f] = h;
-    }
-}
-
-template <bool FP64>
-__global__ void __launch_bounds__(kCTile) k_cand_link(Arrays a, Sizes z)
-{
-    pdl_enter();
-    if (!any_rebuild(a, z)) return;
-    for (int64_t tile = blockIdx.x; tile < z.CT; tile += gridDim.x) {
-        const int4 tl = a.ctile[tile];
-        if (!tile_rebuilds(a, tl) || a.ctile_base[tile] < 0 || (int)threadIdx.x >= tl.z) continue;
-        cand_link_sphere<FP64>(a, tl);
-    }
 }
 
 // ---------------------------------------------------------------- step
@@ -893,9 +518,14 @@ __global__ void __launch_bounds__(kCTile, FP64 ? 2 : 4) k_contact(Arrays a, Size
     int *ws = (int *)((unsigned char *)queue + SM::queue_bytes);
     __shared__ int pile_flags;
 
-    const int4 tl = a.ctile[blockIdx.x];
+    // the first blocks finish the piles' opening reductions
+    if (blockIdx.x < z.P) {
+        open_pile<kCTile>(a, blockIdx.x);
+        return;
+    }
+    const int4 tl = a.ctile[blockIdx.x - z.P];
     const int p = tl.x;
-    if (!pile_live(a, p)) return;
+    if (!pile_active(a, p)) return;
     const PileStatic &S = a.ps[p];
     const PileDyn &D = a.pd[p];
     if (D.flags & DEM_FLAG_SLOTS) return;          // lists could not be built: frozen this step
@@ -1103,7 +733,11 @@ __global__ void __launch_bounds__(128) k_contact_sphere(Arrays a, Sizes z)
 {
     pdl_enter();
     typedef typename CT<FP64>::H H;
-    const int64_t kb0 = (int64_t)blockIdx.x * 128;
+    if (blockIdx.x < z.P) {   // the first blocks finish the piles' opening reductions
+        open_pile<128>(a, blockIdx.x);
+        return;
+    }
+    const int64_t kb0 = (int64_t)(blockIdx.x - z.P) * 128;
     const int64_t k = kb0 + threadIdx.x;
     __shared__ int4 s_x[FP64 ? 1 : 2 * 128];
     __shared__ float4 s_v[FP64 ? 1 : 2 * 128];
@@ -1118,7 +752,7 @@ __global__ void __launch_bounds__(128) k_contact_sphere(Arrays a, Sizes z)
     }
     if (k >= z.N) return;
     const int p = a.sph_pile[k];
-    if (!pile_live(a, p)) return;
+    if (!pile_active(a, p)) return;
     const PileStatic &S = a.ps[p];
     const PileDyn &D = a.pd[p];
     if (D.flags & DEM_FLAG_SLOTS) return;
@@ -1155,24 +789,13 @@ cudaError_t contact_setup(bool fp64, int)
 void launch_contact(const Arrays &a, const Sizes &z, bool fp64, int, cudaStream_t st)
 {
     if (z.N == 0 || z.CT == 0) return;
-    const unsigned nt = (unsigned)z.CT;
-    // the rebuild kernels walk the tiles with a grid of a few blocks per SM:
-    // in steps without a rebuild they only read each tile's pile flags
-    const unsigned ng = (unsigned)(z.CT < 512 ? z.CT : 512);
+    const unsigned nt = (unsigned)(z.CT + z.P), ns = (unsigned)((z.N + 127) / 128 + z.P);
     if (fp64) {
-        launch_pdl(k_cand_count<true>, ng, kCTile, 0, st, a, z);
-        launch_pdl(k_cand_scan, (unsigned)z.P, 1024, 0, st, a, z);
-        launch_pdl(k_cand_fill<true>, ng, kCTile, 0, st, a, z);
-        launch_pdl(k_cand_link<true>, ng, kCTile, 0, st, a, z);
         if (z.cmode == 1) launch_pdl(k_contact<true>, nt, kCTile, Smem<true>::total, st, a, z);
-        else launch_pdl(k_contact_sphere<true>, (unsigned)((z.N + 127) / 128), 128, 0, st, a, z);
+        else launch_pdl(k_contact_sphere<true>, ns, 128, 0, st, a, z);
     } else {
-        launch_pdl(k_cand_count<false>, ng, kCTile, 0, st, a, z);
-        launch_pdl(k_cand_scan, (unsigned)z.P, 1024, 0, st, a, z);
-        launch_pdl(k_cand_fill<false>, ng, kCTile, 0, st, a, z);
-        launch_pdl(k_cand_link<false>, ng, kCTile, 0, st, a, z);
         if (z.cmode == 1) launch_pdl(k_contact<false>, nt, kCTile, Smem<false>::total, st, a, z);
-        else launch_pdl(k_contact_sphere<false>, (unsigned)((z.N + 127) / 128), 128, 0, st, a, z);
+        else launch_pdl(k_contact_sphere<false>, ns, 128, 0, st, a, z);
     }
 }
 

@@ -19,26 +19,27 @@
 // terms), and k_grav_combine adds them in FP64 in range order (deterministic).
 //
 // Symmetric form (default; packed FP32 in the mixed path, scalar FP64 in the
-// FP64 path).  The pair term is antisymmetric
-// (Newton's third law): F_ij = -F_ji.  The pile is cut into tiles of 512
-// spheres; a work item is a pair of tiles (a, b), a < b, and evaluates each of
-// its 512 x 512 pairs once, adding the term to sphere i of tile a and its
-// negative to sphere j of tile b.  Each warp keeps 128 i-spheres in registers
-// (4 per lane) and passes 32 j-spheres round the warp by register shuffles,
-// each j carrying its own running sum, so a j-sphere visits all 128 i-spheres
-// of the warp in 32 steps; per pair this costs 16 FP32 instructions and one
-// reciprocal square root where the one-sided form needs 24 and two.  Items
-// (a, a) take the one-sided form.  Mixed path: every item adds its FP32
-// i-sums and j-sums, scaled by a power of two and rounded once, to 64-bit
-// integer accumulators per sphere (atomic integer adds, which give the same
-// result in any order, so nothing depends on the schedule);
-// k_grav_acc_to_force turns them into forces.  FP64 path: every item writes
-// its i-sums (one per b) and j-sums (one per a) as FP64 partials, and
-// k_grav_combine_sym64 adds a sphere's partials in tile order.
+// FP64 path).  The pair term is antisymmetric (Newton's third law): F_ij =
+// -F_ji.  The pile is cut into tiles; a work item is a pair of tiles (a, b), a
+// < b, and evaluates each of its pairs once, adding the term to sphere i of
+// tile a and its negative to sphere j of tile b.  Each lane of a warp keeps a
+// few i-spheres in registers and meets the j-spheres in turn, 32 at a time
+// round the warp; every j's running sum travels with it by register shuffles,
+// so a j-sphere visits all i-spheres of the warp in 32 steps; per pair this
+// costs 16 FP32 operations and one reciprocal square root where the one-sided
+// form needs 24 and two.  Items (a, a) take the one-sided form.  Mixed path:
+// every item adds its FP32 i-sums and j-sums, scaled by a power of two and
+// rounded once, to 64-bit integer accumulators per sphere (atomic integer
+// adds, which give the same result in any order, so nothing depends on the
+// schedule), which k_grav_acc_to_force or k_agg_end turn into forces.  FP64
+// path: every item writes its i-sums (one per b) and j-sums (one per a) as
+// FP64 partials, and k_grav_combine_sym64 adds a sphere's partials in a fixed
+// order.
 #include <algorithm>
 
 #include "dem_internal.h"
 #include "devmath.cuh"
+#include "expand.cuh"
 #include "launch.cuh"
 
 namespace dem {
@@ -328,17 +329,47 @@ __device__ __forceinline__ void gravity32p_item(const Arrays &a, const int4 it, 
         }
 }
 
-// Next work item of a persistent grid.  Every block takes items until it
-// draws one past the end, so a launch makes exactly GI + gridDim.x draws; the
-// last draw puts the counter back to zero for the next launch (the counter
-// is zeroed once when the layout is uploaded), so no memset node is needed
-// between the kernels of a step.
-__device__ __forceinline__ int grab_item(int32_t *counter, int64_t GI)
-{
-    const int v = atomicAdd(counter, 1);
-    if ((int64_t)v == GI + (int64_t)gridDim.x - 1) atomicExch(counter, 0);
-    return v;
-}
+// Work items of a persistent grid: a block starts with item blockIdx.x and
+// draws further ones from a counter, the grid's size on.  A launch of more
+// items than blocks makes exactly `items` draws (one per further item, one
+// per block that finds none left); the last puts the counter back to zero for
+// the next launch (it is zeroed once when the layout is uploaded), so no memset
+// node is needed between the kernels of a step.  With a block per item
+// nothing is drawn: two round trips to L2 less in the small worlds.
+// Call with the whole block.
+struct Items {
+    int64_t n;
+    int32_t *counter;
+    int *slot;   // shared
+    bool first = true;
+    __device__ __forceinline__ Items(int32_t *c, int64_t items, int *sh) : n(items), counter(c), slot(sh) {}
+    // next item, or -1; thread 0 calls done() once the block has finished an item
+    template <typename Fn>
+    __device__ __forceinline__ int next(Fn done)
+    {
+        if (first) {
+            first = false;
+            return (int64_t)blockIdx.x < n ? (int)blockIdx.x : -1;
+        }
+        __syncthreads();   // the block is done with its item (and has read *slot)
+        const bool draw = n > (int64_t)gridDim.x;
+        if (threadIdx.x == 0) {
+            done();
+            if (draw) {
+                const int v = atomicAdd(counter, 1);
+                if ((int64_t)v == n - 1) atomicExch(counter, 0);
+                *slot = (int64_t)v + gridDim.x < n ? v + (int)gridDim.x : -1;
+            }
+        }
+        if (!draw) return -1;
+        __syncthreads();
+        return *slot;
+    }
+    __device__ __forceinline__ int next()
+    {
+        return next([] {});
+    }
+};
 
 template <int BS, int NP>
 __global__ void __launch_bounds__(BS) k_gravity32p(Arrays a, Sizes z)
@@ -349,18 +380,12 @@ __global__ void __launch_bounds__(BS) k_gravity32p(Arrays a, Sizes z)
     __shared__ int excl[2];
     __shared__ double sacc[6 * NP * BS];
     __shared__ int next;
-    for (;;) {
-        __syncthreads();
-        if (threadIdx.x == 0) next = grab_item(a.gcounter, z.GI);
-        __syncthreads();
-        const int item = next;
-        if (item >= z.GI) return;
-        gravity32p_item<BS, NP>(a, a.gitems[item], sp, sag, excl, sacc);
-    }
+    Items items(a.gcounter, z.GI, &next);
+    for (int item; (item = items.next()) >= 0;) gravity32p_item<BS, NP>(a, a.gitems[item], sp, sag, excl, sacc);
 }
 
-// Persistent grid: each block takes the next item from a counter (see
-// grab_item) until the list is exhausted.  Items are listed largest first;
+// Persistent grid: each block takes the next item from a counter (see Items)
+// until the list is exhausted.  Items are listed largest first;
 // which block runs an item does not change its result, so the sums stay
 // deterministic.
 template <int BS, int IB>
@@ -371,14 +396,8 @@ __global__ void __launch_bounds__(BS) k_gravity32(Arrays a, Sizes z)
     __shared__ int sag[BS];
     __shared__ int excl[2];
     __shared__ int next;
-    for (;;) {
-        __syncthreads();
-        if (threadIdx.x == 0) next = grab_item(a.gcounter, z.GI);
-        __syncthreads();
-        const int item = next;
-        if (item >= z.GI) return;
-        gravity32_item<BS, IB>(a, a.gitems[item], sp, sag, excl);
-    }
+    Items items(a.gcounter, z.GI, &next);
+    for (int item; (item = items.next()) >= 0;) gravity32_item<BS, IB>(a, a.gitems[item], sp, sag, excl);
 }
 
 template <int BS, int IB>
@@ -460,21 +479,6 @@ __global__ void __launch_bounds__(BS) k_gravity64(Arrays a, Sizes z)
 }
 
 // ---------------------------------------------------------------- symmetric form
-constexpr int kSymTile = 512;   // spheres per tile (large piles)
-// shape of the mixed path's 512-sphere tiles: warps per block x i-spheres per lane
-#ifndef DEM_SYM_WPB
-#define DEM_SYM_WPB 4
-#endif
-constexpr int kBigWPB = DEM_SYM_WPB, kBigIB = 512 / (32 * DEM_SYM_WPB);
-static_assert(32 * kBigWPB * kBigIB == kSymTile, "512-sphere tiles");
-// launch bounds of the symmetric kernel (optionally with a minimum number of
-// resident blocks per SM, which caps its registers)
-#ifdef DEM_GSYM_MINB
-#define DEM_GSYM_BOUNDS __launch_bounds__(32 * WPB, DEM_GSYM_MINB)
-#else
-#define DEM_GSYM_BOUNDS __launch_bounds__(32 * WPB)
-#endif
-
 // Mixed symmetric form: add one tile item's FP32 sum on home sphere s to its
 // 64-bit integer accumulators.  The sum is scaled by the pile's power of two
 // (exact) and rounded to the nearest integer once; integer additions are
@@ -554,39 +558,49 @@ __device__ __forceinline__ float4 sym_ring(float4 pj, int aj, const float4 (&xi)
     return make_float4(fx, fy, fz, 0.f);
 }
 
-// ring steps unrolled per loop iteration (a tuning constant)
-#ifndef DEM_RING_UNROLL
-#define DEM_RING_UNROLL 16
-#endif
-constexpr int kRingUnroll = DEM_RING_UNROLL;
-
-// Packed ring (unmasked tile pairs): each lane holds two j-spheres, packed
-// into the two halves of 64-bit registers, and its 4 i-spheres duplicated into
-// both halves, so one f32x2 instruction evaluates the same step of two pairs.
-// A chunk is 64 j-spheres (j and j + 32 in lane l).  The i-sums are kept per
-// half and added at the end of the item; the j-sums travel with their j.
-template <int IB>
-__device__ __forceinline__ void sym_ring2(const float4 &pa, const float4 &pb,
-                                          const f2_t (&xx)[IB], const f2_t (&xy)[IB],
+// Packed ring (unmasked tile pairs): each lane holds its IB i-spheres
+// duplicated into both halves of 64-bit registers and meets two j-spheres a
+// step, packed, so one f32x2 instruction evaluates the same step of two pairs.
+// A chunk is 64 j-spheres: slot m of the staged tile holds j = m and m + 32
+// (xy: their x and y, zm: z and mass), and lane l meets slot (l + s) mod 32 in
+// step s, read from shared memory (two conflict-free 16-byte loads); only the
+// j-sums travel from lane to lane.  The i-sums are kept per half and added at
+// the end of the item.
+//
+// What bounds it: the FP32 pipe and the register reads that feed it.  A pair
+// costs 16 FP32 lane operations and one rsqrt; an f32x2 operation with three
+// different register operands takes 3.2 cycles of a scheduler, not 2, one that
+// shares an operand with the instruction before it 2.3, and a shuffle costs
+// the pipe about as much as an operation.  So IB is large: the shuffles (6
+// per step) are spread over 2 IB pairs and the registers' 4 resident blocks
+// are enough to fill the pipe.  Measured, 100,000 spheres in 512 x 512 tiles: 4
+// i-spheres and shuffled j-spheres (14 shuffles per 8 pairs) 2.70 ms, this
+// 2.61 ms (without any shuffle 2.41 ms, a timing probe on as many pairs).
+//
+// UNI: every sphere of the pile has the same mass, which the caller applies
+// to the sums: two operations of the 16 less (200,000 equal spheres 11.1 ->
+// 9.7 ms per step with it and the ring above).
+template <int IB, bool UNI>
+__device__ __forceinline__ void sym_ring2(const ulonglong2 *xy, const ulonglong2 *zm,
+                                          const f2_t (&xx)[IB], const f2_t (&xy_)[IB],
                                           const f2_t (&xz)[IB], const f2_t (&nm2)[IB],
                                           f2_t (&qx)[IB], f2_t (&qy)[IB], f2_t (&qz)[IB],
                                           f2_t e2, float4 &fa, float4 &fb)
 {
-    const int src = (threadIdx.x + 1) & 31;
-    f2_t jx = f2_pack(pa.x, pb.x), jy = f2_pack(pa.y, pb.y), jz = f2_pack(pa.z, pb.z),
-         jm = f2_pack(pa.w, pb.w);
+    const int l = threadIdx.x & 31, src = (l + 1) & 31;
     f2_t fx = f2_pack(0.f, 0.f), fy = fx, fz = fx;
-#pragma unroll kRingUnroll
+#pragma unroll 8
     for (int s = 0; s < 32; ++s) {
+        const ulonglong2 ja = xy[(l + s) & 31], jb = zm[(l + s) & 31];
 #pragma unroll
         for (int k = 0; k < IB; ++k) {
-            const f2_t dx = f2_sub(jx, xx[k]), dy = f2_sub(jy, xy[k]), dz = f2_sub(jz, xz[k]);
+            const f2_t dx = f2_sub(ja.x, xx[k]), dy = f2_sub(ja.y, xy_[k]), dz = f2_sub(jb.x, xz[k]);
             const f2_t r2 = f2_fma(dz, dz, f2_fma(dy, dy, f2_fma(dx, dx, e2)));
             float ra, rb;
             f2_unpack(r2, ra, rb);
             const f2_t inv = f2_pack(rsqrtf(ra), rsqrtf(rb));
             const f2_t inv3 = f2_mul(f2_mul(inv, inv), inv);
-            const f2_t si = f2_mul(jm, inv3), sj = f2_mul(nm2[k], inv3);
+            const f2_t si = UNI ? inv3 : f2_mul(jb.y, inv3), sj = UNI ? inv3 : f2_mul(nm2[k], inv3);
             qx[k] = f2_fma(dx, si, qx[k]);
             qy[k] = f2_fma(dy, si, qy[k]);
             qz[k] = f2_fma(dz, si, qz[k]);
@@ -594,10 +608,6 @@ __device__ __forceinline__ void sym_ring2(const float4 &pa, const float4 &pb,
             fy = f2_fma(dy, sj, fy);
             fz = f2_fma(dz, sj, fz);
         }
-        jx = __shfl_sync(0xffffffffu, jx, src);
-        jy = __shfl_sync(0xffffffffu, jy, src);
-        jz = __shfl_sync(0xffffffffu, jz, src);
-        jm = __shfl_sync(0xffffffffu, jm, src);
         fx = __shfl_sync(0xffffffffu, fx, src);
         fy = __shfl_sync(0xffffffffu, fy, src);
         fz = __shfl_sync(0xffffffffu, fz, src);
@@ -610,16 +620,62 @@ __device__ __forceinline__ void sym_ring2(const float4 &pa, const float4 &pb,
     fb = make_float4(bx, by, bz, 0.f);
 }
 
+// All chunks of the staged tile through the packed ring; the lane's i-sums
+// and the warp's j-sums (sj), with the masses applied.
+template <int IB, bool UNI>
+__device__ __forceinline__ void sym_rings(const ulonglong2 *xy, const ulonglong2 *zm, int nj, const float4 (&xi)[IB],
+                                          float mass, float eps2, float (&ax)[IB], float (&ay)[IB], float (&az)[IB],
+                                          float4 *sj)
+{
+    const int l = threadIdx.x & 31;
+    f2_t xx[IB], xy_[IB], xz[IB], nm2[IB], qx[IB], qy[IB], qz[IB];
+    const f2_t zero2 = f2_pack(0.f, 0.f);
+#pragma unroll
+    for (int k = 0; k < IB; ++k) {
+        xx[k] = f2_pack(xi[k].x, xi[k].x);
+        xy_[k] = f2_pack(xi[k].y, xi[k].y);
+        xz[k] = f2_pack(xi[k].z, xi[k].z);
+        nm2[k] = f2_pack(-xi[k].w, -xi[k].w);
+        qx[k] = qy[k] = qz[k] = zero2;
+    }
+    const f2_t e2 = f2_pack(eps2, eps2);
+    for (int c = 0; c * 64 < nj; ++c) {
+        float4 fa, fb;
+        sym_ring2<IB, UNI>(xy + 32 * c, zm + 32 * c, xx, xy_, xz, nm2, qx, qy, qz, e2, fa, fb);
+        if (UNI) {
+            fa = make_float4(-mass * fa.x, -mass * fa.y, -mass * fa.z, 0.f);
+            fb = make_float4(-mass * fb.x, -mass * fb.y, -mass * fb.z, 0.f);
+        }
+        sj[c * 64 + l] = fa;
+        sj[c * 64 + 32 + l] = fb;
+    }
+#pragma unroll
+    for (int k = 0; k < IB; ++k) {
+        float lo, hi;
+        f2_unpack(qx[k], lo, hi);
+        ax[k] = lo + hi;
+        f2_unpack(qy[k], lo, hi);
+        ay[k] = lo + hi;
+        f2_unpack(qz[k], lo, hi);
+        az[k] = lo + hi;
+        if (UNI) {
+            ax[k] *= mass;
+            ay[k] *= mass;
+            az[k] *= mass;
+        }
+    }
+}
+
 // Work item (pile, tile a, tile b): the symmetric pass for a < b, the
-// one-sided pass over the tile itself for a == b.  sp/sag: tile b staged in
-// shared memory; sj: per-warp j-sums.  WPB warps per block, each with
-// 32 x IB i-spheres: tiles of 32 WPB IB spheres (512 for the large-pile
-// form, 128 for small piles whose 512-sphere tile pairs would not fill the GPU).
+// one-sided pass over the tile itself for a == b.  xy/zm/sag: tile b staged in
+// shared memory (see sym_ring2); sj: per-warp j-sums.  WPB warps per block,
+// each with 32 x IB i-spheres: tiles of 32 WPB IB spheres.
 template <int WPB, int IB>
-__device__ __forceinline__ void gravity32s_item(const Arrays &a, const int4 it, float4 *sp, int *sag,
-                                                float4 *sj, int *bad)
+__device__ __forceinline__ void gravity32s_item(const Arrays &a, const int4 it, ulonglong2 *xy, ulonglong2 *zm,
+                                                int *sag, float4 *sj, int *bad)
 {
     constexpr int kSymBS = 32 * WPB, kSymTile = kSymBS * IB;
+    static_assert(kSymTile % 64 == 0, "whole chunks");
     const int p = it.x;
     if (a.enabled[p] == 0 || a.pd[p].failed) return;
     const PileStatic &S = a.ps[p];
@@ -632,78 +688,70 @@ __device__ __forceinline__ void gravity32s_item(const Arrays &a, const int4 it, 
     const int w = threadIdx.x >> 5, l = threadIdx.x & 31;
     const int jb0 = tb * kSymTile;
     const int nj = min(kSymTile, ns - jb0);
-    for (int m = threadIdx.x; m < kSymTile; m += kSymBS) {
-        const int j = jb0 + m;
-        sp[m] = j < ns ? a.gpos32[s0 + j] : make_float4(1.0e18f, 1.0e18f, 1.0e18f, 0.f);
-        sag[m] = j < ns ? a.sph_agg[s0 + j] : -1;
+    // spheres past the end: massless, and so far away that r^-3 underflows to
+    // zero (where no masses enter), on opposite sides for i and j
+    auto load = [&](int j, float far) {
+        return j < ns ? a.gpos32[s0 + j] : make_float4(far, far, far, 0.f);
+    };
+    for (int m = threadIdx.x; m < kSymTile / 2; m += kSymBS) {
+        const int j = jb0 + ((m >> 5) << 6) + (m & 31);
+        const float4 u = load(j, 1.0e18f), v = load(j + 32, 1.0e18f);
+        xy[m] = make_ulonglong2(f2_pack(u.x, v.x), f2_pack(u.y, v.y));
+        zm[m] = make_ulonglong2(f2_pack(u.z, v.z), f2_pack(u.w, v.w));
     }
+    for (int m = threadIdx.x; m < kSymTile; m += kSymBS) sag[m] = jb0 + m < ns ? a.sph_agg[s0 + jb0 + m] : -1;
+    // staged sphere m of the tile
+    auto staged = [&](int m) {
+        const int c = ((m >> 6) << 5) + (m & 31), h = (m >> 5) & 1;
+        const float *q = (const float *)(xy + c) + h, *r = (const float *)(zm + c) + h;
+        return make_float4(q[0], q[2], r[0], r[2]);
+    };
     float4 xi[IB];
-    float nm[IB];
-    int ai[IB];
     float ax[IB], ay[IB], az[IB];
     const int i0 = ta * kSymTile + w * (32 * IB) + l;
 #pragma unroll
     for (int k = 0; k < IB; ++k) {
-        const int i = i0 + 32 * k;
-        const bool ok = i < ns;
-        xi[k] = ok ? a.gpos32[s0 + i] : make_float4(0.f, 0.f, 0.f, 0.f);
-        ai[k] = ok ? a.sph_agg[s0 + i] : -2;
-        nm[k] = -xi[k].w;
+        xi[k] = load(i0 + 32 * k, -1.0e18f);
         ax[k] = ay[k] = az[k] = 0.f;
     }
     // an aggregate can span the two tiles only if it spans their boundary
     const bool masked = diag || a.sph_agg[s0 + (int64_t)ta * kSymTile + kSymTile - 1] == a.sph_agg[s0 + jb0];
     __syncthreads();
-    if (diag) {
-        for (int jj = 0; jj < nj; ++jj) {
-            const float4 pj = sp[jj];
-            const int aj = sag[jj];
+    if (masked) {
+        int ai[IB];
+        float nm[IB];
 #pragma unroll
-            for (int k = 0; k < IB; ++k) {
-                const float dx = pj.x - xi[k].x, dy = pj.y - xi[k].y, dz = pj.z - xi[k].z;
-                const float r2 = fmaf(dz, dz, fmaf(dy, dy, fmaf(dx, dx, eps2)));
-                const float inv = rsqrtf(r2);
-                float si = (pj.w * inv) * (inv * inv);
-                si = aj == ai[k] ? 0.f : si;
-                ax[k] = fmaf(dx, si, ax[k]);
-                ay[k] = fmaf(dy, si, ay[k]);
-                az[k] = fmaf(dz, si, az[k]);
+        for (int k = 0; k < IB; ++k) {
+            ai[k] = i0 + 32 * k < ns ? a.sph_agg[s0 + i0 + 32 * k] : -2;
+            nm[k] = -xi[k].w;
+        }
+        if (diag) {
+            for (int jj = 0; jj < nj; ++jj) {
+                const float4 pj = staged(jj);
+                const int aj = sag[jj];
+#pragma unroll
+                for (int k = 0; k < IB; ++k) {
+                    const float dx = pj.x - xi[k].x, dy = pj.y - xi[k].y, dz = pj.z - xi[k].z;
+                    const float r2 = fmaf(dz, dz, fmaf(dy, dy, fmaf(dx, dx, eps2)));
+                    const float inv = rsqrtf(r2);
+                    float si = (pj.w * inv) * (inv * inv);
+                    si = aj == ai[k] ? 0.f : si;
+                    ax[k] = fmaf(dx, si, ax[k]);
+                    ay[k] = fmaf(dy, si, ay[k]);
+                    az[k] = fmaf(dz, si, az[k]);
+                }
+            }
+        } else {
+            for (int c = 0; c * 32 < nj; ++c) {
+                const float4 pj = staged(c * 32 + l);
+                const int aj = sag[c * 32 + l];
+                sj[w * kSymTile + c * 32 + l] = sym_ring<true, IB>(pj, aj, xi, nm, ai, ax, ay, az, eps2);
             }
         }
-    } else if (masked) {
-        for (int c = 0; c * 32 < nj; ++c) {
-            const float4 pj = sp[c * 32 + l];
-            const int aj = sag[c * 32 + l];
-            sj[w * kSymTile + c * 32 + l] = sym_ring<true, IB>(pj, aj, xi, nm, ai, ax, ay, az, eps2);
-        }
+    } else if (S.umass > 0.f) {
+        sym_rings<IB, true>(xy, zm, nj, xi, S.umass, eps2, ax, ay, az, sj + w * kSymTile);
     } else {
-        f2_t xx[IB], xy[IB], xz[IB], nm2[IB], qx[IB], qy[IB], qz[IB];
-        const f2_t zero2 = f2_pack(0.f, 0.f);
-#pragma unroll
-        for (int k = 0; k < IB; ++k) {
-            xx[k] = f2_pack(xi[k].x, xi[k].x);
-            xy[k] = f2_pack(xi[k].y, xi[k].y);
-            xz[k] = f2_pack(xi[k].z, xi[k].z);
-            nm2[k] = f2_pack(nm[k], nm[k]);
-            qx[k] = qy[k] = qz[k] = zero2;
-        }
-        const f2_t e2 = f2_pack(eps2, eps2);
-        for (int c = 0; c * 64 < nj; ++c) {
-            float4 fa, fb;
-            sym_ring2<IB>(sp[c * 64 + l], sp[c * 64 + 32 + l], xx, xy, xz, nm2, qx, qy, qz, e2, fa, fb);
-            sj[w * kSymTile + c * 64 + l] = fa;
-            sj[w * kSymTile + c * 64 + 32 + l] = fb;
-        }
-#pragma unroll
-        for (int k = 0; k < IB; ++k) {
-            float lo, hi;
-            f2_unpack(qx[k], lo, hi);
-            ax[k] = lo + hi;
-            f2_unpack(qy[k], lo, hi);
-            ay[k] = lo + hi;
-            f2_unpack(qz[k], lo, hi);
-            az[k] = lo + hi;
-        }
+        sym_rings<IB, false>(xy, zm, nj, xi, 0.f, eps2, ax, ay, az, sj + w * kSymTile);
     }
     if (!diag) {
         __syncthreads();
@@ -733,63 +781,38 @@ __device__ __forceinline__ void gravity32s_item(const Arrays &a, const int4 it, 
 }
 
 template <int WPB, int IB>
-__global__ void DEM_GSYM_BOUNDS k_gravity32s(Arrays a, Sizes z)
+__global__ void __launch_bounds__(32 * WPB) k_gravity32s(Arrays a, Sizes z)
 {
     pdl_enter();
     constexpr int kTile = 32 * WPB * IB;
-    __shared__ float4 sp[kTile];
+    __shared__ ulonglong2 xy[kTile / 2], zm[kTile / 2];
     __shared__ int sag[kTile];
     __shared__ float4 sj[WPB * kTile];
-    __shared__ int next, bad, bad_pile;   // flags raised by the block's last item, and its pile
+    __shared__ int next, bad;   // bad: flags raised by the block's item
     if (threadIdx.x == 0) bad = 0;
-    for (;;) {
-        __syncthreads();
-        if (threadIdx.x == 0) {
-            if (bad) {
-                atomicOr(&a.pd[bad_pile].flags, bad);
-                bad = 0;
-            }
-            next = grab_item(a.gcounter, z.GI);
-            if (next < z.GI) bad_pile = a.gitems[next].x;
+    Items items(a.gcounter, z.GI, &next);
+    int p = 0;
+    auto raise = [&] {
+        if (bad) {
+            atomicOr(&a.pd[p].flags, bad);
+            bad = 0;
         }
-        __syncthreads();
-        const int item = next;
-        if (item >= z.GI) return;
-        gravity32s_item<WPB, IB>(a, a.gitems[item], sp, sag, sj, &bad);
+    };
+    for (int item; (item = items.next(raise)) >= 0;) {
+        const int4 it = a.gitems[item];
+        p = it.x;
+        gravity32s_item<WPB, IB>(a, it, xy, zm, sag, sj, &bad);
     }
 }
 
-// r2^(-3/2) on as few FP64 instructions as possible: the FP64 unit (about 1.7
-// operations per clock and SM, against 128 for FP32 and 64 for integers) is
-// what bounds the FP64 pass, so whatever can be formed exactly elsewhere is.
-// y0 = the hardware's approximate rsqrt, a double with a 21-bit significand
-// (its low word is zero), |e| <= 2e-6 with e = 1 - r2 y0^2.  From the binomial
-// series of (1 - e)^(-3/2),
-//   r2^(-3/2) = y0^3 (1 + 3/2 e + 15/8 e^2 + O(e^3)),  35/16 |e|^3 < 2^-55;
-// y0^2 has 42 bits and is formed by an integer product (exact), the 15/8 e^2
-// term (below 2^-36) in FP32 with its bits widened by integer instructions:
-// 4 FP64 operations in all.  Largest relative error over 2^-20..2^20:
-// 2.3e-16, against 4.4e-16 for rsqrt(r2) cubed.  r2 is kept inside
-// [2^-1020, 2^1020] (y0^2 then stays a normal number): r2 = 0 still gives a
-// result that is not finite, an overflowed r2 zero.
-// Measured, 1.1e8 pairs / 152 SMs: 2.85 ms with rsqrt() cubed, 2.53 ms so.
-__device__ __forceinline__ double grav_inv3(double r2)
+// f(kernel, threads per block) for the mixed kernel of a tile size
+template <typename Fn>
+static void with_sym32(int tile, Fn f)
 {
-    r2 = __hiloint2double(min(max(__double2hiint(r2), 0x00300000), 0x7fb00000), __double2loint(r2));
-    double y0;
-    asm("rsqrt.approx.ftz.f64 %0, %1;" : "=d"(y0) : "d"(r2));
-    const unsigned yh = (unsigned)__double2hiint(y0);
-    const unsigned long long m = (yh & 0xfffffu) | 0x100000u, mm = m * m;   // in [2^40, 2^42)
-    const unsigned big = (unsigned)(mm >> 41);
-    const unsigned long long bits =
-        ((mm << (12 - big)) & 0xfffffffffffffull) | ((unsigned long long)(2 * (yh >> 20) - 1023 + big) << 52);
-    const double t = __longlong_as_double((long long)bits);
-    const double e = fma(-r2, t, 1.0), y3 = t * y0;
-    const int eh = __double2hiint(e) & 0x7fffffff;
-    const float ef = __int_as_float(eh > (897 << 20) ? (eh - (896 << 20)) << 3 : 0);
-    const int cb = __float_as_int(1.875f * ef * ef);
-    const double q = fma(1.5, e, __hiloint2double(cb > 0 ? (cb >> 3) + (896 << 20) : 0, cb << 29));
-    return fma(y3, q, y3);
+    if (tile == 64) f(k_gravity32s<1, 2>, 32);
+    else if (tile == 128) f(k_gravity32s<1, 4>, 32);
+    else if (tile == 256) f(k_gravity32s<1, 8>, 32);
+    else f(k_gravity32s<2, 8>, 64);
 }
 
 // FP64 path, symmetric form: the same tile pairs and ring as the mixed path
@@ -813,7 +836,7 @@ __device__ __forceinline__ dbl4 sym_ring64(dbl4 pj, int aj, const dbl4 (&xi)[IB]
 #pragma unroll
         for (int k = 0; k < IB; ++k) {
             const double dx = pj.x - xi[k].x, dy = pj.y - xi[k].y, dz = pj.z - xi[k].z;
-            const double inv3 = grav_inv3(fma(dz, dz, fma(dy, dy, fma(dx, dx, eps2))));
+            const double inv3 = inv_r3(fma(dz, dz, fma(dy, dy, fma(dx, dx, eps2))));
             double si = pj.w * inv3, sj = -xi[k].w * inv3;
             if (MASK && aj == ai[k]) si = sj = 0.0;
             ax[k] = fma(dx, si, ax[k]);
@@ -877,7 +900,7 @@ __device__ __forceinline__ void gravity64s_item(const Arrays &a, const int4 it, 
 #pragma unroll
             for (int k = 0; k < IB; ++k) {
                 const double dx = pj.x - xi[k].x, dy = pj.y - xi[k].y, dz = pj.z - xi[k].z;
-                double si = pj.w * grav_inv3(fma(dz, dz, fma(dy, dy, fma(dx, dx, eps2))));
+                double si = pj.w * inv_r3(fma(dz, dz, fma(dy, dy, fma(dx, dx, eps2))));
                 si = aj == ai[k] ? 0.0 : si;
                 ax[k] = fma(dx, si, ax[k]);
                 ay[k] = fma(dy, si, ay[k]);
@@ -929,14 +952,8 @@ __global__ void __launch_bounds__(32 * WPB) k_gravity64s(Arrays a, Sizes z, int6
     dbl4 *sj = sp + kTile;
     int *sag = (int *)(sj + WPB * kTile);
     __shared__ int next;
-    for (;;) {
-        __syncthreads();
-        if (threadIdx.x == 0) next = grab_item(a.gcounter, count);
-        __syncthreads();
-        const int item = next;
-        if (item >= count) return;
-        gravity64s_item<WPB, IB>(a, a.gitems[first + item], sp, sag, sj);
-    }
+    Items items(a.gcounter, count, &next);
+    for (int item; (item = items.next()) >= 0;) gravity64s_item<WPB, IB>(a, a.gitems[first + item], sp, sag, sj);
 }
 
 // f(kernel, threads per block, shared bytes) for the FP64 kernel of a tile size
@@ -950,29 +967,44 @@ static void with_sym64(int tile, Fn f)
     else f(k_gravity64s<4, 4>, 128, sym64_smem(512, 4));
 }
 
-// Each sphere's partials in tile order.  One thread per sphere, few blocks
-// (12,000 spheres are 48 blocks of 256): the rows are loaded eight at a time.
-__global__ void __launch_bounds__(64) k_grav_combine_sym64(Arrays a, Sizes z)
+// Each sphere's partials, by kCombLanes lanes: lane q adds rows q, q + 8, ...
+// in order, then the lanes by a fixed tree (the same for every pile and
+// batch).  With a thread per sphere, 1,000 spheres were 16 blocks, each thread
+// walking its 32 rows: 15.3 us, 7.5 so (ncu).
+constexpr int kCombLanes = 8, kCombThreads = 128;
+
+__global__ void __launch_bounds__(kCombThreads) k_grav_combine_sym64(Arrays a, Sizes z)
 {
     pdl_enter();
-    int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= z.N) return;
-    int p = a.sph_pile[i];
-    if (a.enabled[p] == 0 || a.pd[p].failed) return;
-    const int T = a.gnchunk[p];
-    if (T <= 1) return;
-    const PileStatic &S = a.ps[p];
-    const int64_t il = i - S.s0;
-    const int t = (int)(il / S.gtile64);
-    const dbl4 *gp = (const dbl4 *)a.gpart;
+    // 16 spheres a block; a warp's lanes: 4 consecutive spheres x 8 row lanes
+    const int lane = threadIdx.x & 31, q = lane >> 2;
+    const int64_t i = (int64_t)blockIdx.x * (kCombThreads / kCombLanes) + (threadIdx.x >> 5) * 4 + (lane & 3);
     double sx = 0, sy = 0, sz = 0;
-    // rows t..T-1 (i-sums of the pairs (t, b)), then T..T+t-1 (j-sums of (r, t))
-#pragma unroll 8
-    for (int r = t; r < T + t; ++r) {
-        const dbl4 v = gp[sym_slot(a, p, S.ns, r, il)];
-        sx += v.x; sy += v.y; sz += v.z;
+    int p = -1;
+    if (i < z.N) {
+        p = a.sph_pile[i];
+        if (a.enabled[p] == 0 || a.pd[p].failed || a.gnchunk[p] <= 1) p = -1;
     }
-    const double gm = S.G * a.m64[i];
+    if (p >= 0) {
+        const int T = a.gnchunk[p];
+        const PileStatic &S = a.ps[p];
+        const int64_t il = i - S.s0;
+        const int t = (int)(il / S.gtile64);
+        const dbl4 *gp = (const dbl4 *)a.gpart;
+        // rows t..T-1 (i-sums of the pairs (t, b)), then T..T+t-1 (j-sums of (r, t))
+#pragma unroll 4
+        for (int r = t + q; r < T + t; r += kCombLanes) {
+            const dbl4 v = gp[sym_slot(a, p, S.ns, r, il)];
+            sx += v.x; sy += v.y; sz += v.z;
+        }
+    }
+    for (int o = 4; o < 32; o <<= 1) {
+        sx += __shfl_xor_sync(0xffffffffu, sx, o);
+        sy += __shfl_xor_sync(0xffffffffu, sy, o);
+        sz += __shfl_xor_sync(0xffffffffu, sz, o);
+    }
+    if (p < 0 || q != 0) return;
+    const double gm = a.ps[p].G * a.m64[i];
     a.fg[i] = make_dbl4(gm * sx, gm * sy, gm * sz, 0.0);
 }
 
@@ -1049,10 +1081,9 @@ int gravity_blocks_per_sm(bool fp64, int block, int ib, bool pack, bool sym, int
                 cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, k, threads, smem);
             });
         } else {
-            if (tile == 64) cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, k_gravity32s<1, 2>, 32, 0);
-            else if (tile == 128) cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, k_gravity32s<1, 4>, 32, 0);
-            else if (tile == 256) cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, k_gravity32s<2, 4>, 64, 0);
-            else cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, k_gravity32s<kBigWPB, kBigIB>, 32 * kBigWPB, 0);
+            with_sym32(tile, [&](auto k, int threads) {
+                cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, k, threads, 0);
+            });
         }
         return n;
     }
@@ -1065,7 +1096,8 @@ int gravity_blocks_per_sm(bool fp64, int block, int ib, bool pack, bool sym, int
 // tile into F_i = G m_i sum 2^-k and clear the accumulators for the next step
 // (one thread per sphere: the accumulators are read once, coalesced, with
 // every sphere in flight; done inside the per-aggregate pass instead, one
-// thread walking an aggregate's members, it was 4x slower on 256 small piles).
+// thread walking an aggregate's members, it was 4x slower on 256 small piles,
+// but worlds of at most kGaccFuseMax spheres save the launch, see there).
 __global__ void k_grav_acc_to_force(Arrays a, Sizes z)
 {
     pdl_enter();
@@ -1074,13 +1106,7 @@ __global__ void k_grav_acc_to_force(Arrays a, Sizes z)
     int p = a.sph_pile[i];
     if (a.enabled[p] == 0 || a.pd[p].failed) return;
     if (a.gnchunk[p] <= 1) return;
-    const PileStatic &S = a.ps[p];
-    longlong2 *g = (longlong2 *)(a.gacc + 4 * i);
-    const longlong2 xy = g[0], zw = g[1];
-    g[0] = make_longlong2(0, 0);
-    g[1] = make_longlong2(0, 0);
-    const double gm = S.G * a.m64[i] * S.ginv;
-    a.fg[i] = make_dbl4(gm * (double)xy.x, gm * (double)xy.y, gm * (double)zw.x, 0.0);
+    a.fg[i] = gacc_force(a, a.ps[p], i, gacc_load(a, i));
 }
 
 void launch_gravity(const Arrays &a, const Sizes &z, bool fp64, int block, int ib, bool pack,
@@ -1097,13 +1123,12 @@ void launch_gravity(const Arrays &a, const Sizes &z, bool fp64, int block, int i
                     launch_pdl(k, (unsigned)std::min(count, z.g64_blocks[c]), threads, smem, st, a, z, first, count);
                 });
             }
-            if (z.GP > 0) launch_pdl(k_grav_combine_sym64, (unsigned)((z.N + 63) / 64), 64, 0, st, a, z);
+            constexpr int per = kCombThreads / kCombLanes;
+            if (z.GP > 0)
+                launch_pdl(k_grav_combine_sym64, (unsigned)((z.N + per - 1) / per), kCombThreads, 0, st, a, z);
         } else {
-            if (z.gtile == 64) launch_pdl(k_gravity32s<1, 2>, (unsigned)nb, 32, 0, st, a, z);
-            else if (z.gtile == 128) launch_pdl(k_gravity32s<1, 4>, (unsigned)nb, 32, 0, st, a, z);
-            else if (z.gtile == 256) launch_pdl(k_gravity32s<2, 4>, (unsigned)nb, 64, 0, st, a, z);
-            else launch_pdl(k_gravity32s<kBigWPB, kBigIB>, (unsigned)nb, 32 * kBigWPB, 0, st, a, z);
-            if (z.gacc_on) launch_pdl(k_grav_acc_to_force, (unsigned)((z.N + 255) / 256), 256, 0, st, a, z);
+            with_sym32(z.gtile, [&](auto k, int threads) { launch_pdl(k, (unsigned)nb, threads, 0, st, a, z); });
+            if (z.gacc_on == 1) launch_pdl(k_grav_acc_to_force, (unsigned)((z.N + 255) / 256), 256, 0, st, a, z);
         }
         return;
     }

@@ -1,7 +1,6 @@
-// kernels_step.cu -- per-step kernels other than the contact pass and gravity:
-// rigid-body kick/drift/rotation, pile reductions, sphere expansion and cell
-// keys, the counting sort into cells, the sorted gather, and the reduction of
-// sphere forces onto aggregates with the closing kick.
+// kernels_step.cu -- the aggregate kernels that open and close a step:
+// rigid-body kick/drift/rotation, and the reduction of sphere forces onto
+// aggregates with the closing kick and the end of the piles' step.
 //
 // Paper references: leapfrog with predicted velocities (Sec. 2.1), aggregate
 // mass and COM (Sec. 2.2.1, Eq. agg_mass, Eq. agg_position), Euler's equations
@@ -9,16 +8,15 @@
 // aggregate force and torque sums (Sec. 2.2.3-2.2.4, Eq. agg_gravity,
 // Eq. gravity_torque, Eq. agg_contact_accel, contact torque at the contact
 // point), YORP increment (Sec. 4.1), point-mass planet (Sec. 4.2).
+#include <type_traits>
+
 #include "dem_internal.h"
 #include "devmath.cuh"
+#include "expand.cuh"
 #include "launch.cuh"
+#include "reduce.cuh"
 
 namespace dem {
-
-__device__ __forceinline__ bool pile_active(const Arrays &a, int p)
-{
-    return a.enabled[p] != 0 && a.pd[p].failed == 0;
-}
 
 // ---------------------------------------------------------------- ids
 __device__ int find_slot(const PileStatic *ps, int P, int64_t idx, int which)
@@ -333,11 +331,13 @@ __device__ __forceinline__ void agg_begin_mixed(const Arrays &a, int64_t g, int 
     a.rec32[g] = rec;
 }
 
+constexpr int kAggThreads = 128;   // threads per block of the aggregate kernels, an aggregate each
+
 template <bool FP64, bool ADAPT>
-__global__ void k_agg_begin(Arrays a, Sizes z)
+__global__ void __launch_bounds__(kAggThreads) k_agg_begin(Arrays a, Sizes z)
 {
     pdl_enter();
-    int64_t g = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    int64_t g = (int64_t)blockIdx.x * kAggThreads + threadIdx.x;
     if (g >= z.A) return;
     int p = a.agg_pile[g];
     if (!pile_active(a, p)) return;
@@ -348,333 +348,19 @@ __global__ void k_agg_begin(Arrays a, Sizes z)
 void launch_agg_begin(const Arrays &a, const Sizes &z, bool fp64, cudaStream_t st)
 {
     if (z.A == 0) return;
-    unsigned nb = (unsigned)((z.A + 127) / 128);
+    const unsigned nb = (unsigned)((z.A + kAggThreads - 1) / kAggThreads);
     // the adaptive rotor needs many more registers: its variant runs only when
     // some pile asks for it
     if (z.adapt) {
-        if (fp64) launch_pdl(k_agg_begin<true, true>, nb, 128, 0, st, a, z);
-        else launch_pdl(k_agg_begin<false, true>, nb, 128, 0, st, a, z);
+        if (fp64) launch_pdl(k_agg_begin<true, true>, nb, kAggThreads, 0, st, a, z);
+        else launch_pdl(k_agg_begin<false, true>, nb, kAggThreads, 0, st, a, z);
     } else {
-        if (fp64) launch_pdl(k_agg_begin<true, false>, nb, 128, 0, st, a, z);
-        else launch_pdl(k_agg_begin<false, false>, nb, 128, 0, st, a, z);
+        if (fp64) launch_pdl(k_agg_begin<true, false>, nb, kAggThreads, 0, st, a, z);
+        else launch_pdl(k_agg_begin<false, false>, nb, kAggThreads, 0, st, a, z);
     }
 }
 
-// ---------------------------------------------------------------- pile reductions
-// Block b sums kAggChunk aggregates of one pile.  Mode 0 (after the drift):
-// sum M, sum M r, sum M v.  Mode 1 (after the closing kick): sum of the planet
-// force on the pile.  The last of a pile's chunk blocks to finish (counted in
-// pile_arrive, which it puts back to zero) then adds the pile's chunk sums and
-// updates the pile: thread t adds chunks t, t+128, ... in order and
-// block_sum7 combines the threads in a fixed order, so the result does not
-// depend on which block came last.  Fixed orders throughout: deterministic.
-// Without a planet the closing pass has nothing to sum: the pile's first
-// chunk block alone updates it.
-// Sum of v over the block's 128 threads in a fixed order (each warp by
-// shuffles, then the four warp sums in warp order); the result is in
-// thread 0.  ws: 4 x 7 scratch doubles.
-__device__ __forceinline__ void block_sum7(double (&v)[7], double *ws)
-{
-    for (int o = 16; o > 0; o >>= 1)
-        for (int k = 0; k < 7; ++k) v[k] += __shfl_down_sync(0xffffffffu, v[k], o);
-    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-    if (lane == 0)
-        for (int k = 0; k < 7; ++k) ws[7 * wid + k] = v[k];
-    __syncthreads();
-    if (threadIdx.x == 0)
-        for (int k = 0; k < 7; ++k) v[k] = (ws[k] + ws[7 + k]) + (ws[14 + k] + ws[21 + k]);
-}
-
-// The same in float-float (mixed path: FP32 units only).
-__device__ __forceinline__ void block_sum7(ff (&v)[7], ff *ws)
-{
-    for (int o = 16; o > 0; o >>= 1)
-        for (int k = 0; k < 7; ++k) {
-            const ff t = {__shfl_down_sync(0xffffffffu, v[k].hi, o), __shfl_down_sync(0xffffffffu, v[k].lo, o)};
-            v[k] = ff_add(v[k], t);
-        }
-    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-    if (lane == 0)
-        for (int k = 0; k < 7; ++k) ws[7 * wid + k] = v[k];
-    __syncthreads();
-    if (threadIdx.x == 0)
-        for (int k = 0; k < 7; ++k) v[k] = ff_add(ff_add(ws[k], ws[7 + k]), ff_add(ws[14 + k], ws[21 + k]));
-}
-
-template <int MODE>
-__device__ void pile_finalize_block(const Arrays &a, int p, double (&sh)[7][128])
-{
-    const PileStatic &S = a.ps[p];
-    double s[7] = {0, 0, 0, 0, 0, 0, 0};
-    if (MODE == 0 || S.ext_mass > 0) {   // the closing pass sums only the planet's reaction
-        for (int64_t ch = S.ch0 + threadIdx.x; ch < S.ch0 + S.nch; ch += blockDim.x)
-            for (int k = 0; k < 7; ++k) s[k] += __ldcg(a.chunk_part + ch * kPartialDoubles + k);
-        __syncthreads();   // sh is free again
-        block_sum7(s, &sh[0][0]);
-    }
-    if (threadIdx.x != 0) return;
-    PileDyn &D = a.pd[p];
-    const double h = S.h;
-    if (MODE == 0) {
-        for (int c = 0; c < 3; ++c) {
-            D.Rc[c] = s[1 + c] / s[0];
-            D.Vc[c] = s[4 + c] / s[0];
-            const ff rc = ff_of(D.Rc[c]);
-            D.Rcf[c] = make_float2(rc.hi, rc.lo);
-        }
-        if (S.ext_mass > 0) {   // planet: kick with the stored acceleration, drift
-            for (int c = 0; c < 3; ++c) {
-                D.P_vel[c] += 0.5 * h * D.P_acc[c];
-                D.P_pos[c] += h * D.P_vel[c];
-            }
-        }
-    } else {
-        if (S.ext_mass > 0) {   // planet: reaction of the pile, closing kick
-            for (int c = 0; c < 3; ++c) {
-                D.P_acc[c] = -s[c] / S.ext_mass;
-                D.P_vel[c] += 0.5 * h * D.P_acc[c];
-            }
-        }
-        for (int c = 0; c < 3; ++c) {
-            D.O[c] = D.Rc[c];
-            D.V[c] = D.Vc[c];
-            D.hVf[c] = (float)(h * D.Vc[c]);
-            D.Of[c] = D.Rcf[c];
-            const ff vc = ff_of(D.Vc[c]);
-            D.Vf[c] = make_float2(vc.hi, vc.lo);
-        }
-        D.steps += 1;
-        D.parity ^= 1;
-        if (D.flags & (DEM_FLAG_SLOTS | DEM_FLAG_NONFINITE | DEM_FLAG_GRAV_RANGE)) D.failed = 1;
-        if (D.rebuild) {
-            D.rebuilds += 1;
-            D.cpar ^= 1;   // the lists built this step become the current ones
-        }
-        D.rebuilt_prev = D.rebuild;
-        D.rebuild = S.skin <= 0.0 ? 1 : 0;
-    }
-}
-
-template <int MODE>
-__global__ void __launch_bounds__(128) k_pile_reduce(Arrays a, Sizes z)
-{
-    pdl_enter();
-    int64_t ch = blockIdx.x;
-    if (ch >= z.CH) return;
-    int p = a.chunk_pile[ch];
-    __shared__ double sh[7][128];
-    __shared__ int last;
-    if (MODE == 1 && !(a.ps[p].ext_mass > 0)) {
-        // no planet: nothing to sum, the pile's first chunk block finishes it
-        if (ch != a.ps[p].ch0 || !pile_active(a, p)) return;
-        pile_finalize_block<MODE>(a, p, sh);
-        return;
-    }
-    double acc[7] = {0, 0, 0, 0, 0, 0, 0};
-    ff accf[7];
-    for (int k = 0; k < 7; ++k) accf[k] = ff{0.f, 0.f};
-    const bool act = pile_active(a, p);
-    if (act) {
-        const PileStatic &S = a.ps[p];
-        int64_t beg = S.a0 + (ch - S.ch0) * kAggChunk;
-        int64_t end = beg + kAggChunk;
-        if (end > S.a0 + S.na) end = S.a0 + S.na;
-        if (MODE == 0 && a.out_ff) {
-            // mixed path: float-float state, M as FP32 (the sums fix the
-            // frame origin and velocity, whose exact values do not enter any
-            // result: positions and velocities are taken relative to them
-            // exactly).  The thread's kAggChunk / 128 aggregates are loaded
-            // together, then added in index order.
-            constexpr int kPer = kAggChunk / 128;
-            static_assert(kAggChunk % 128 == 0, "k_pile_reduce runs 128 threads per chunk");
-            const PileDyn &D = a.pd[p];
-            float Mf[kPer];
-            ff rr[kPer][3], vv[kPer][3];
-#pragma unroll
-            for (int t = 0; t < kPer; ++t) {
-                const int64_t g = beg + threadIdx.x + 128 * t;
-                const bool in = g < end;
-                Mf[t] = in ? (float)a.M[g] : 0.f;
-                for (int c = 0; c < 3; ++c) {
-                    rr[t][c] = in ? ldff(a.r + 3 * g + c) : ff{0.f, 0.f};
-                    vv[t][c] = in ? ldff(a.v + 3 * g + c) : ff{0.f, 0.f};
-                }
-            }
-#pragma unroll
-            for (int t = 0; t < kPer; ++t) {
-                const int64_t g = beg + threadIdx.x + 128 * t;
-                if (g >= end) break;
-                if (D.rebuild) {   // new neighbour-list reference, as the test forms it
-                    float *ar = a.aref + 8 * g;
-                    for (int c = 0; c < 3; ++c) ar[c] = ff_sub(rr[t][c], ff_of2(D.Of[c])).hi - D.hVf[c];
-                    for (int c = 0; c < 4; ++c) ar[3 + c] = ldff(a.q + 4 * g + c).hi;
-                }
-                accf[0] = ff_addf(accf[0], Mf[t]);
-                for (int c = 0; c < 3; ++c) {
-                    accf[1 + c] = ff_add(accf[1 + c], ff_mul(ff{Mf[t], 0.f}, rr[t][c]));
-                    accf[4 + c] = ff_add(accf[4 + c], ff_mul(ff{Mf[t], 0.f}, vv[t][c]));
-                }
-            }
-        } else
-        for (int64_t g = beg + threadIdx.x; g < end; g += blockDim.x) {
-            if (MODE == 0) {
-                if (a.pd[p].rebuild) {   // new neighbour-list reference
-                    const PileDyn &D = a.pd[p];
-                    float *ar = a.aref + 8 * g;
-                    for (int c = 0; c < 3; ++c) ar[c] = (float)(a.r[3 * g + c] - D.O[c] - S.h * D.V[c]);
-                    for (int c = 0; c < 4; ++c) ar[3 + c] = (float)a.q[4 * g + c];
-                }
-                double M = a.M[g];
-                acc[0] += M;
-                for (int c = 0; c < 3; ++c) {
-                    acc[1 + c] += M * a.r[3 * g + c];
-                    acc[4 + c] += M * a.v[3 * g + c];
-                }
-            } else if (a.out_ff) {   // mixed path: the parts are float-float pairs
-                const float2 *o32 = (const float2 *)(a.out[2] + 6 * g);
-                for (int c = 0; c < 3; ++c) accf[c] = ff_add(accf[c], ff_of2(o32[c]));
-            } else {
-                for (int c = 0; c < 3; ++c) acc[c] += a.out[2][6 * g + c];
-            }
-        }
-    }
-    if (a.out_ff) {
-        // mixed path: the block's sum in float-float on the FP32 units (the
-        // FP64 units of this part are ~75 times slower), one conversion
-        block_sum7(accf, reinterpret_cast<ff *>(&sh[0][0]));
-        if (threadIdx.x == 0)
-            for (int k = 0; k < 7; ++k) acc[k] = ff_value(accf[k]);
-    } else {
-        block_sum7(acc, &sh[0][0]);
-    }
-    if (threadIdx.x == 0) {
-        for (int k = 0; k < 7; ++k) a.chunk_part[ch * kPartialDoubles + k] = acc[k];
-        __threadfence();   // the sums are visible before this block is counted
-        last = atomicAdd(a.pile_arrive + p, 1) == (int)a.ps[p].nch - 1;
-        if (last) a.pile_arrive[p] = 0;
-    }
-    __syncthreads();
-    if (!last || !act) return;
-    __threadfence();
-    pile_finalize_block<MODE>(a, p, sh);
-}
-
-void launch_pile_begin(const Arrays &a, const Sizes &z, cudaStream_t st)
-{
-    if (z.CH == 0) return;
-    launch_pdl(k_pile_reduce<0>, (unsigned)z.CH, 128, 0, st, a, z);
-}
-
-void launch_pile_end(const Arrays &a, const Sizes &z, cudaStream_t st)
-{
-    if (z.CH == 0) return;
-    launch_pdl(k_pile_reduce<1>, (unsigned)z.CH, 128, 0, st, a, z);
-}
-
-// ---------------------------------------------------------------- expansion
-// Sphere centre relative to the pile frame, r_i - O = (r_A - O) + R(q_A) b_i.
-// Mixed: float-float, bitwise identical wherever it is inlined.
-__device__ __forceinline__ void expand_mixed(const AggRecMixed &rec, float4 bh, float4 bl,
-                                             ff &px, ff &py, ff &pz)
-{
-    ff rx = ff_dot3(rec.Rh + 0, rec.Rl + 0, bh.x, bh.y, bh.z, bl.x, bl.y, bl.z);
-    ff ry = ff_dot3(rec.Rh + 3, rec.Rl + 3, bh.x, bh.y, bh.z, bl.x, bl.y, bl.z);
-    ff rz = ff_dot3(rec.Rh + 6, rec.Rl + 6, bh.x, bh.y, bh.z, bl.x, bl.y, bl.z);
-    ff cx = {rec.ch[0], rec.cl[0]}, cy = {rec.ch[1], rec.cl[1]}, cz = {rec.ch[2], rec.cl[2]};
-    px = ff_add(cx, rx);
-    py = ff_add(cy, ry);
-    pz = ff_add(cz, rz);
-}
-
-__device__ __forceinline__ double3 expand_64(const AggRec64 &rec, const double *b)
-{
-    const double *R = rec.R;
-    double x = __fma_rn(R[2], b[2], __fma_rn(R[1], b[1], __dmul_rn(R[0], b[0])));
-    double y = __fma_rn(R[5], b[2], __fma_rn(R[4], b[1], __dmul_rn(R[3], b[0])));
-    double zz = __fma_rn(R[8], b[2], __fma_rn(R[7], b[1], __dmul_rn(R[6], b[0])));
-    return d3(__dadd_rn(rec.c[0], x), __dadd_rn(rec.c[1], y), __dadd_rn(rec.c[2], zz));
-}
-
-__device__ __forceinline__ int wrap_cell(int c, int n)
-{
-    int m = c % n;
-    return m < 0 ? m + n : m;
-}
-
-__device__ __forceinline__ int cell_coord_f(float x, float inv_cell, int n)
-{
-    float f = floorf(__fmul_rn(x, inv_cell));
-    f = fminf(fmaxf(f, -1.0e9f), 1.0e9f);
-    return wrap_cell((int)f, n);
-}
-
-__device__ __forceinline__ int cell_coord_d(double x, double inv_cell, int n)
-{
-    double f = floor(__dmul_rn(x, inv_cell));
-    f = fmin(fmax(f, -1.0e9), 1.0e9);
-    return wrap_cell((int)f, n);
-}
-
-// Per sphere (home order): expand, cell key, atomic count into the cell (the
-// returned rank is made deterministic later by ordering each cell), gravity
-// input (position relative to the pile frame, mass).  A pile without
-// self-gravity needs no gravity input: in its steps without a rebuild there
-// is nothing to do.
-template <bool FP64>
-__global__ void k_keys(Arrays a, Sizes z)
-{
-    pdl_enter();
-    int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= z.N) return;
-    int p = a.sph_pile[i];
-    if (!pile_active(a, p)) return;
-    const PileStatic &S = a.ps[p];
-    const bool grav = S.G != 0.0;
-    if (!grav && !a.pd[p].rebuild) return;
-    int64_t g = S.a0 + a.sph_agg[i];
-    int cx, cy, cz;
-    if (FP64) {
-        double3 pos = expand_64(a.rec64[g], a.b64 + 3 * i);
-        cx = cell_coord_d(pos.x, S.inv_cell, S.nx);
-        cy = cell_coord_d(pos.y, S.inv_cell, S.ny);
-        cz = cell_coord_d(pos.z, S.inv_cell, S.nz);
-        if (grav) a.gpos64[i] = make_dbl4(pos.x, pos.y, pos.z, a.m64[i]);
-    } else {
-        ff px, py, pz;
-        expand_mixed(a.rec32[g], a.bh[i], a.bl[i], px, py, pz);
-        float ic = (float)S.inv_cell;
-        cx = cell_coord_f(px.hi, ic, S.nx);
-        cy = cell_coord_f(py.hi, ic, S.ny);
-        cz = cell_coord_f(pz.hi, ic, S.nz);
-        if (grav) a.gpos32[i] = make_float4(px.hi, py.hi, pz.hi, (float)a.m64[i]);
-    }
-    if (!a.pd[p].rebuild) return;   // cell list kept from the last rebuild
-    const int key = (int)cell_id(cx, cy, cz, S.nx, S.ny);
-    a.key[i] = key;
-    a.rank[i] = atomicAdd(a.ccount + S.c0 + key, 1);
-}
-
-__device__ int tile_pile(const Arrays &a, const Sizes &z, int64_t t);
-
-// Zero the cell counts of the piles that rebuild this step.
-__global__ void k_clear_cells(Arrays a, Sizes z)
-{
-    pdl_enter();
-    int64_t c = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (c >= z.C) return;
-    int p = tile_pile(a, z, c / kScanTile);
-    if (pile_active(a, p) && a.pd[p].rebuild) a.ccount[c] = 0;
-}
-
-void launch_keys(const Arrays &a, const Sizes &z, bool fp64, cudaStream_t st)
-{
-    if (z.N == 0) return;
-    launch_pdl(k_clear_cells, (unsigned)((z.C + 255) / 256), 256, 0, st, a, z);
-    unsigned nb = (unsigned)((z.N + 255) / 256);
-    if (fp64) launch_pdl(k_keys<true>, nb, 256, 0, st, a, z);
-    else launch_pdl(k_keys<false>, nb, 256, 0, st, a, z);
-}
-
+// ---------------------------------------------------------------- host requests
 // Host request (after a state write or a new layout): the next step rebuilds
 // the cell list and hit lists of pile `slot` (all piles for slot < 0).
 __global__ void k_force_rebuild(Arrays a, Sizes z, int slot)
@@ -693,245 +379,19 @@ void launch_force_rebuild(const Arrays &a, const Sizes &z, int slot, cudaStream_
     launch_pdl(k_force_rebuild, (unsigned)((z.P + 127) / 128), 128, 0, st, a, z, slot);
 }
 
-// ---------------------------------------------------------------- scan of cell counts
-// Tiles of kScanTile cells never straddle piles (cell ranges are padded).
-__device__ int tile_pile(const Arrays &a, const Sizes &z, int64_t t)
-{
-    int lo = 0, hi = (int)z.P - 1;
-    while (lo < hi) {
-        int mid = (lo + hi + 1) >> 1;
-        if (a.ps[mid].t0 <= t) lo = mid; else hi = mid - 1;
-    }
-    return lo;
-}
-
-__global__ void k_scan_tiles(Arrays a, Sizes z)
-{
-    pdl_enter();
-    int64_t t = blockIdx.x;
-    int p = tile_pile(a, z, t);
-    if (!pile_active(a, p) || !a.pd[p].rebuild) return;
-    const int32_t *c = a.ccount + t * kScanTile;
-    int s = 0;
-    for (int k = threadIdx.x; k < kScanTile; k += blockDim.x) s += c[k];
-    for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
-    __shared__ int ws[8];
-    if ((threadIdx.x & 31) == 0) ws[threadIdx.x >> 5] = s;
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        int tot = 0;
-        for (int k = 0; k < (int)(blockDim.x >> 5); ++k) tot += ws[k];
-        a.tile_sum[t] = tot;
-    }
-}
-
-// One block per pile: exclusive scan of its tile sums (in place).
-__global__ void k_scan_piles(Arrays a, Sizes z)
-{
-    pdl_enter();
-    int p = blockIdx.x;
-    if (!pile_active(a, p) || !a.pd[p].rebuild) return;
-    const PileStatic &S = a.ps[p];
-    __shared__ int buf[1024];
-    __shared__ int carry;
-    if (threadIdx.x == 0) carry = 0;
-    __syncthreads();
-    for (int64_t base = 0; base < S.nt; base += 1024) {
-        int64_t t = base + threadIdx.x;
-        int v = t < S.nt ? a.tile_sum[S.t0 + t] : 0;
-        buf[threadIdx.x] = v;
-        __syncthreads();
-        for (int o = 1; o < 1024; o <<= 1) {
-            int add = threadIdx.x >= (unsigned)o ? buf[threadIdx.x - o] : 0;
-            __syncthreads();
-            buf[threadIdx.x] += add;
-            __syncthreads();
-        }
-        int incl = buf[threadIdx.x];
-        if (t < S.nt) a.tile_sum[S.t0 + t] = carry + incl - v;
-        __syncthreads();
-        if (threadIdx.x == 1023) carry += incl;
-        __syncthreads();
-    }
-}
-
-// One block (256 threads x 8 cells) per tile: exclusive scan plus tile offset.
-__global__ void k_scan_cells(Arrays a, Sizes z)
-{
-    pdl_enter();
-    int64_t t = blockIdx.x;
-    int p = tile_pile(a, z, t);
-    if (!pile_active(a, p) || !a.pd[p].rebuild) return;
-    const int32_t *c = a.ccount + t * kScanTile;
-    int32_t *o = a.cstart + t * kScanTile;
-    int v[8];
-    int loc = 0;
-    for (int k = 0; k < 8; ++k) {
-        v[k] = c[threadIdx.x * 8 + k];
-        loc += v[k];
-    }
-    __shared__ int buf[256];
-    buf[threadIdx.x] = loc;
-    __syncthreads();
-    for (int off = 1; off < 256; off <<= 1) {
-        int add = threadIdx.x >= (unsigned)off ? buf[threadIdx.x - off] : 0;
-        __syncthreads();
-        buf[threadIdx.x] += add;
-        __syncthreads();
-    }
-    int run = a.tile_sum[t] + buf[threadIdx.x] - loc;
-    for (int k = 0; k < 8; ++k) {
-        o[threadIdx.x * 8 + k] = run;
-        run += v[k];
-    }
-}
-
-void launch_scan(const Arrays &a, const Sizes &z, cudaStream_t st)
-{
-    if (z.T == 0) return;
-    launch_pdl(k_scan_tiles, (unsigned)z.T, 256, 0, st, a, z);
-    launch_pdl(k_scan_piles, (unsigned)z.P, 1024, 0, st, a, z);
-    launch_pdl(k_scan_cells, (unsigned)z.T, 256, 0, st, a, z);
-}
-
-// ---------------------------------------------------------------- scatter and cell order
-__global__ void k_scatter(Arrays a, Sizes z)
-{
-    pdl_enter();
-    int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= z.N) return;
-    int p = a.sph_pile[i];
-    if (!pile_active(a, p) || !a.pd[p].rebuild) return;
-    const PileStatic &S = a.ps[p];
-    int slot = a.cstart[S.c0 + a.key[i]] + a.rank[i];
-    a.sorted[S.s0 + slot] = (int32_t)(i - S.s0);
-}
-
-void launch_scatter(const Arrays &a, const Sizes &z, cudaStream_t st)
-{
-    if (z.N == 0) return;
-    launch_pdl(k_scatter, (unsigned)((z.N + 255) / 256), 256, 0, st, a, z);
-}
-
-// The thread at the first position of each cell sorts that cell's entries by
-// home index (insertion sort; cells hold a handful of spheres), which makes
-// the order of neighbours, and so every contact sum, deterministic.
-__global__ void k_cell_order(Arrays a, Sizes z)
-{
-    pdl_enter();
-    int64_t k = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (k >= z.N) return;
-    int p = a.sph_pile[k];
-    if (!pile_active(a, p) || !a.pd[p].rebuild) return;
-    const PileStatic &S = a.ps[p];
-    int32_t *srt = a.sorted + S.s0;
-    int kl = (int)(k - S.s0);
-    int key = a.key[S.s0 + srt[kl]];
-    int start = a.cstart[S.c0 + key];
-    if (kl != start) return;
-    int n = a.ccount[S.c0 + key];
-    for (int x = 1; x < n; ++x) {
-        int v = srt[start + x];
-        int y = x - 1;
-        while (y >= 0 && srt[start + y] > v) {
-            srt[start + y + 1] = srt[start + y];
-            --y;
-        }
-        srt[start + y + 1] = v;
-    }
-}
-
-void launch_cell_order(const Arrays &a, const Sizes &z, cudaStream_t st)
-{
-    if (z.N == 0) return;
-    launch_pdl(k_cell_order, (unsigned)((z.N + 255) / 256), 256, 0, st, a, z);
-}
-
-// ---------------------------------------------------------------- gather
-// Sorted copies for the contact pass: position (float-float in mixed), predicted
-// velocity v_i = [v_A + h/2 a_A] + w_A x (r_i - r_A) (Eq. pred-vel), spin, ids.
-template <bool FP64>
-__global__ void k_gather(Arrays a, Sizes z)
-{
-    pdl_enter();
-    int64_t k = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (k >= z.N) return;
-    int p = a.sph_pile[k];
-    if (!pile_active(a, p)) return;
-    const PileStatic &S = a.ps[p];
-    int hl = a.sorted[k];
-    int64_t i = S.s0 + hl;
-    // the sorted order changes only at rebuilds: the sorted aggregate ids are
-    // written in a rebuild step (and read here otherwise); the home -> sorted
-    // map, which k_cand_link reads at the next rebuild to find each sphere's
-    // previous list, is double-buffered by parity and written in a rebuild
-    // step and the step after it
-    const PileDyn &D = a.pd[p];
-    const bool fresh = D.rebuild != 0, refresh = fresh || D.rebuilt_prev != 0;
-    const int al = fresh ? a.sph_agg[i] : a.sagg[k];
-    int64_t g = S.a0 + al;
-    if (refresh) a.pos_of_home[D.parity ^ 1][i] = (int32_t)(k - S.s0);
-    if (fresh) a.sagg[k] = al;
-    if (FP64) {
-        const AggRec64 &rec = a.rec64[g];
-        const double *b = a.b64 + 3 * i;
-        double3 pos = expand_64(rec, b);
-        double3 rb = mat_mul(rec.R, d3(b[0], b[1], b[2]));
-        double3 w = ld3(rec.w);
-        double3 v = ld3(rec.vb) + cross(w, rb);
-        a.dp_[k] = make_dbl4(pos.x, pos.y, pos.z, a.s64[i]);
-        a.dv_[k] = make_dbl4(v.x, v.y, v.z, (double)al);
-        a.dw_[k] = make_dbl4(w.x, w.y, w.z, (double)hl);
-    } else {
-        const AggRecMixed &rec = a.rec32[g];
-        float4 bh = a.bh[i], bl = a.bl[i];
-        ff px, py, pz;
-        expand_mixed(rec, bh, bl, px, py, pz);
-        float3 rb = f3(rec.Rh[0] * bh.x + rec.Rh[1] * bh.y + rec.Rh[2] * bh.z,
-                       rec.Rh[3] * bh.x + rec.Rh[4] * bh.y + rec.Rh[5] * bh.z,
-                       rec.Rh[6] * bh.x + rec.Rh[7] * bh.y + rec.Rh[8] * bh.z);
-        float3 w = f3(rec.w[0], rec.w[1], rec.w[2]);
-        float3 v = f3(rec.vb[0], rec.vb[1], rec.vb[2]) + cross(w, rb);
-        // fixed point in quanta q = 2^qexp: low 32 bits of round((r_i - O) / q)
-        // per axis (differences of nearby spheres are exact int32) and
-        // round(radius / q), with what the rounding left in FP32
-        const int e = -S.qexp;
-        float4 rm;
-        const int X = ff_to_fixed(px, e, rm.x), Y = ff_to_fixed(py, e, rm.y), Z = ff_to_fixed(pz, e, rm.z);
-        const int Sr = ff_to_fixed(ff{bh.w, bl.w}, e, rm.w);
-        a.xqr[2 * k] = make_int4(X, Y, Z, Sr);
-        a.xqr[2 * k + 1] = make_int4(__float_as_int(rm.x), __float_as_int(rm.y), __float_as_int(rm.z),
-                                     __float_as_int(rm.w));
-        if (fresh) a.sph_[k] = make_float4(px.hi, py.hi, pz.hi, bh.w);
-        a.svw[2 * k] = make_float4(v.x, v.y, v.z, __int_as_float(al));
-        a.svw[2 * k + 1] = make_float4(w.x, w.y, w.z, __int_as_float(hl));
-    }
-}
-
-void launch_gather(const Arrays &a, const Sizes &z, bool fp64, cudaStream_t st)
-{
-    if (z.N == 0) return;
-    unsigned nb = (unsigned)((z.N + 255) / 256);
-    if (fp64) launch_pdl(k_gather<true>, nb, 256, 0, st, a, z);
-    else launch_pdl(k_gather<false>, nb, 256, 0, st, a, z);
-}
-
 // ---------------------------------------------------------------- step end
 // Per aggregate: F_A = sum_i (F_c,i + F_g,i + F_e,i) and
 // N_A = sum_i [(r_i - r_A) x F_i + tau_i], kept separately for contact,
 // gravity and planet; a_A = F_A / M; closing half kick of COM and spin; YORP
 // increment dw: v_A += dw x (r_A - R_pile), w_A += dw (rigid rotation of the
 // whole pile).  Members are contiguous (spheres stored in aggregate order).
-// GRAV = false: no pile of the world has self-gravity (the gravity sums are
-// left out, and with them their registers).
-template <bool FP64, bool GRAV>
-__global__ void __launch_bounds__(128) k_agg_end(Arrays a, Sizes z)
+// GRAV = 0: no pile of the world has self-gravity (the gravity sums are left
+// out, and with them their registers); 2: the sphere gravity of piles with
+// more than one tile is still in the integer accumulators (Sizes::gacc_on).
+// Fsum: the planet's force on the aggregate.
+template <bool FP64, int GRAV, typename T>
+__device__ __forceinline__ void agg_end(const Arrays &a, int64_t g, int p, T (&Fsum)[3])
 {
-    pdl_enter();
-    int64_t g = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (g >= z.A) return;
-    int p = a.agg_pile[g];
-    if (!pile_active(a, p)) return;
     const PileStatic &S = a.ps[p];
     const PileDyn &D = a.pd[p];
     const double h = S.h;
@@ -940,8 +400,6 @@ __global__ void __launch_bounds__(128) k_agg_end(Arrays a, Sizes z)
     double3 Fc, Nc, Fg, Ng;
     double3 Fe = d3(0, 0, 0), Ne = d3(0, 0, 0);
     const bool planet = S.ext_mass > 0;
-    double3 Pp = planet ? ld3(D.P_pos) : d3(0, 0, 0);
-    double3 O = ld3(D.O);
     if constexpr (FP64) {
         Fc = Nc = Fg = Ng = d3(0, 0, 0);
         const AggRec64 &rec = a.rec64[g];
@@ -958,9 +416,7 @@ __global__ void __launch_bounds__(128) k_agg_end(Arrays a, Sizes z)
             Fg = Fg + fg;
             Ng = Ng + cross(lever, fg);
             if (planet) {
-                const double3 d = Pp - (O + expand_64(rec, b));
-                const double inv = 1.0 / sqrt(dot(d, d));
-                const double3 fe = (S.G * S.ext_mass * a.m64[i] * inv * inv * inv) * d;
+                const double3 fe = planet_force(S.G * S.ext_mass, a.m64[i], ld3(D.P_pos), ld3(D.O) + expand_64(rec, b));
                 Fe = Fe + fe;
                 Ne = Ne + cross(lever, fe);
             }
@@ -988,39 +444,57 @@ __global__ void __launch_bounds__(128) k_agg_end(Arrays a, Sizes z)
         // a pile without self-gravity has zero sphere gravity: not read
         const bool grav = GRAV && S.G != 0.0;
         const dbl4 g0 = make_dbl4(0.0, 0.0, 0.0, 0.0);
-        auto gravity_of = [&](int64_t i) -> dbl4 { return grav ? a.fg[i] : g0; };
-        int t2 = 0;
-        if (!planet) {   // the loads of two members issued together
-            for (; t2 + 1 < n; t2 += 2) {
-                const int64_t i = i0 + t2;
-                const float4 bha = a.bh[i], bhb = a.bh[i + 1];
-                float4 fa, ta, fb, tb;
-                ld_f4x2(a.ftc32 + 2 * i, fa, ta);
-                ld_f4x2(a.ftc32 + 2 * i + 2, fb, tb);
-                const dbl4 ga = gravity_of(i), gb = gravity_of(i + 1);
-                term(bha, fa, ta, ga);
-                term(bhb, fb, tb, gb);
+        const bool sums = GRAV == 2 && grav && a.gnchunk[p] > 1;
+        auto gravity_of = [&](int64_t i) -> dbl4 {
+            if (sums) {
+                const dbl4 f = gacc_force(a, S, i, gacc_load(a, i));
+                a.fg[i] = f;
+                return f;
+            }
+            return grav ? a.fg[i] : g0;
+        };
+        auto gravity_of2 = [&](int64_t i, dbl4 &ga, dbl4 &gb) {
+            if (sums) {   // both spheres' sums loaded before either is cleared
+                const GaccSums x = gacc_load(a, i), y = gacc_load(a, i + 1);
+                a.fg[i] = ga = gacc_force(a, S, i, x);
+                a.fg[i + 1] = gb = gacc_force(a, S, i + 1, y);
+                return;
+            }
+            ga = gravity_of(i);
+            gb = gravity_of(i + 1);
+        };
+        auto planet_term = [&](float4 bh, dbl4 e) {
+            const float3 lever = mat_mulf(Rh, f3(bh.x, bh.y, bh.z));
+            const double3 fe = d3(e.x, e.y, e.z);
+            Fe = Fe + fe;
+            Ne = Ne + cross(d3(lever.x, lever.y, lever.z), fe);
+        };
+        auto planet_of = [&](int64_t i) -> dbl4 { return planet ? a.fe[i] : g0; };
+        int t = 0;
+        for (; t + 1 < n; t += 2) {   // the loads of two members issued together
+            const int64_t i = i0 + t;
+            const float4 bha = a.bh[i], bhb = a.bh[i + 1];
+            float4 fa, ta, fb, tb;
+            ld_f4x2(a.ftc32 + 2 * i, fa, ta);
+            ld_f4x2(a.ftc32 + 2 * i + 2, fb, tb);
+            const dbl4 ea = planet_of(i), eb = planet_of(i + 1);
+            dbl4 ga, gb;
+            gravity_of2(i, ga, gb);
+            term(bha, fa, ta, ga);
+            term(bhb, fb, tb, gb);
+            if (planet) {
+                planet_term(bha, ea);
+                planet_term(bhb, eb);
             }
         }
-        for (int t = t2; t < n; ++t) {
-            int64_t i = i0 + t;
+        if (t < n) {
+            const int64_t i = i0 + t;
             const float4 bh = a.bh[i];
             float4 fc, tc;
             ld_f4x2(a.ftc32 + 2 * i, fc, tc);
+            const dbl4 e = planet_of(i);
             term(bh, fc, tc, gravity_of(i));
-            if (planet) {
-                const float3 lever = mat_mulf(Rh, f3(bh.x, bh.y, bh.z));
-                ff px, py, pz;
-                expand_mixed(rec, bh, a.bl[i], px, py, pz);
-                const double3 pos = O + d3((double)px.hi + (double)px.lo, (double)py.hi + (double)py.lo,
-                                           (double)pz.hi + (double)pz.lo);
-                const double3 d = Pp - pos;
-                const double inv = 1.0 / sqrt(dot(d, d));
-                const double3 fe = (S.G * S.ext_mass * a.m64[i] * inv * inv * inv) * d;
-                const double3 lv = d3(lever.x, lever.y, lever.z);
-                Fe = Fe + fe;
-                Ne = Ne + cross(lv, fe);
-            }
+            if (planet) planet_term(bh, e);
         }
         // the parts as float-float pairs (readout only), the totals formed in
         // float-float and converted once (FP64 instructions are ~60 times
@@ -1030,6 +504,8 @@ __global__ void __launch_bounds__(128) k_agg_end(Arrays a, Sizes z)
         if (planet) {
             part[12] = ff_of(Fe.x); part[13] = ff_of(Fe.y); part[14] = ff_of(Fe.z);
             part[15] = ff_of(Ne.x); part[16] = ff_of(Ne.y); part[17] = ff_of(Ne.z);
+            if constexpr (!FP64)
+                for (int c = 0; c < 3; ++c) Fsum[c] = part[12 + c];
         } else {
             for (int k = 12; k < 18; ++k) part[k] = ff{0.f, 0.f};
         }
@@ -1072,9 +548,13 @@ __global__ void __launch_bounds__(128) k_agg_end(Arrays a, Sizes z)
             stff(a.wb + 3 * g + c, wb[c]);
             fin = fin && isfinite(v[c].hi) && isfinite(wb[c].hi) && isfinite(Nt[c].hi);
         }
-        if (!fin) atomicOr(&a.pd[p].flags, DEM_FLAG_NONFINITE);
+        if (!fin) {
+            atomicOr(&a.pd[p].flags, DEM_FLAG_NONFINITE);
+            __threadfence();   // before the pile's last block reads the flags
+        }
     }
     if constexpr (FP64) {
+        st3(Fsum, Fe);
         st3(a.out[0] + 6 * g, Fc); st3(a.out[0] + 6 * g + 3, Nc);
         st3(a.out[1] + 6 * g, Fg); st3(a.out[1] + 6 * g + 3, Ng);
         st3(a.out[2] + 6 * g, Fe); st3(a.out[2] + 6 * g + 3, Ne);
@@ -1095,21 +575,42 @@ __global__ void __launch_bounds__(128) k_agg_end(Arrays a, Sizes z)
         st3(a.torque + 3 * g, N);
         st3(a.v + 3 * g, v);
         st3(a.wb + 3 * g, wb);
-        if (!finite3(v) || !finite3(wb) || !finite3(N) || !finite3(ld3(a.r + 3 * g)))
+        if (!finite3(v) || !finite3(wb) || !finite3(N) || !finite3(ld3(a.r + 3 * g))) {
             atomicOr(&a.pd[p].flags, DEM_FLAG_NONFINITE);
+            __threadfence();   // before the pile's last block reads the flags
+        }
     }
+}
+
+// One block per kAggThreads aggregates of a chunk of a pile.
+template <bool FP64, int GRAV>
+__global__ void __launch_bounds__(kAggThreads) k_agg_end(Arrays a, Sizes z)
+{
+    pdl_enter();
+    constexpr int kCtas = kAggChunk / kAggThreads;
+    const int64_t ch = blockIdx.x / kCtas;
+    const int p = a.chunk_pile[ch];
+    int64_t beg, end;
+    chunk_range(a, ch, p, beg, end);
+    beg += (int64_t)(blockIdx.x % kCtas) * kAggThreads;
+    if (beg >= end || !pile_active(a, p)) return;
+    const int64_t g = beg + threadIdx.x;
+    typename std::conditional<FP64, double, ff>::type Fe[3] = {};
+    if (g < end) agg_end<FP64, GRAV>(a, g, p, Fe);
+    close_pile<kAggThreads>(a, ch, p, Fe);
 }
 
 void launch_agg_end(const Arrays &a, const Sizes &z, bool fp64, cudaStream_t st)
 {
-    if (z.A == 0) return;
-    unsigned nb = (unsigned)((z.A + 127) / 128);
+    if (z.CH == 0) return;
+    const unsigned nb = (unsigned)z.CH * (kAggChunk / kAggThreads);
     if (fp64) {
-        if (z.grav) launch_pdl(k_agg_end<true, true>, nb, 128, 0, st, a, z);
-        else launch_pdl(k_agg_end<true, false>, nb, 128, 0, st, a, z);
+        if (z.grav) launch_pdl(k_agg_end<true, 1>, nb, kAggThreads, 0, st, a, z);
+        else launch_pdl(k_agg_end<true, 0>, nb, kAggThreads, 0, st, a, z);
     } else {
-        if (z.grav) launch_pdl(k_agg_end<false, true>, nb, 128, 0, st, a, z);
-        else launch_pdl(k_agg_end<false, false>, nb, 128, 0, st, a, z);
+        if (z.grav && z.gacc_on == 2) launch_pdl(k_agg_end<false, 2>, nb, kAggThreads, 0, st, a, z);
+        else if (z.grav) launch_pdl(k_agg_end<false, 1>, nb, kAggThreads, 0, st, a, z);
+        else launch_pdl(k_agg_end<false, 0>, nb, kAggThreads, 0, st, a, z);
     }
 }
 

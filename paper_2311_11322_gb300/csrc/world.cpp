@@ -31,7 +31,7 @@ struct Range {
 };
 
 enum Cls { C_SPH, C_ENT, C_CTILE, C_AGG, C_CELL, C_TILE, C_CHUNK, C_PILE, C_GITEM, C_GPART, C_TNODE,
-           C_TLEAF, C_TSPH, C_NCLS };
+           C_TLEAF, C_TSPH, C_PSPH, C_NCLS };
 
 struct Field {
     void **ptr;
@@ -49,6 +49,7 @@ struct PileHost {
     double ext[3];         // extent of the wrapped grid at creation (cell x dims)
     dem_params P;
     double M_total;
+    float umass;           // the spheres' mass if all have the same, else 0
     bool reported;
     bool watch_on;         // a radius-growth watch is armed (evaluated in the step graph)
 };
@@ -81,11 +82,12 @@ struct dem_world {
     double grav_item = 1048576.0;     // else: target interactions per work item
     bool grav_pack = false;           // packed f32x2 pair terms (even grav_ib)
     bool grav_sym = true;             // mixed path: symmetric tile-pair form
-    int grav_tile = 0;                // symmetric form's tile: 0 = automatic, 128 or 512
+    int grav_tile = 0;                // symmetric form's tile: 0 = automatic, 64, 128, 256 or 512
     double grav_theta = 0.0;          // > 0 (mixed path): tree gravity with this opening angle
     int grav_order = 4;               // tree gravity: highest multipole rank (4 or 2)
     int tree_maxD = 0;                // deepest tree of the current layout
     int sm_count = 0;
+    bool has_planet = false;          // some pile was added with a planet (mixed path: sizes Arrays::fe)
     bool sym64_fallback = false;      // the FP64 path's small tiles did not fit: 512-sphere tiles
     double cell_factor = 1.0;
     double skin_frac = 0.1;           // neighbour-list skin / largest radius
@@ -189,7 +191,6 @@ void build_fields(dem_world *w)
     add((void **)&a.s64, C_SPH, 8, true);
     add((void **)&a.m64, C_SPH, 8, true);
     add((void **)&a.key, C_SPH, 4, false);
-    add((void **)&a.rank, C_SPH, 4, false);
     add((void **)&a.sorted, C_SPH, 4, false);
     add((void **)&a.sagg, C_SPH, 4, false);
     add((void **)&a.fg, C_SPH, 32, true);
@@ -202,8 +203,8 @@ void build_fields(dem_world *w)
         add((void **)&a.cand_id[b], C_ENT, 4, true);
     }
     add((void **)&a.ctile, C_CTILE, 16, false);
-    add((void **)&a.ctile_cnt, C_CTILE, 4, false);
-    add((void **)&a.ctile_base, C_CTILE, 4, false);
+    add((void **)&a.ctile_cnt, C_CTILE, 16, false);
+    add((void **)&a.ctile_base, C_CTILE, 16, false);
     add((void **)&a.pos_of_home[0], C_SPH, 4, true);
     add((void **)&a.pos_of_home[1], C_SPH, 4, true);
     if (d) {
@@ -231,6 +232,7 @@ void build_fields(dem_world *w)
         add((void **)&a.I32, C_AGG, 36, true);
         add((void **)&a.Iinv32, C_AGG, 36, true);
         add((void **)&a.gacc, C_SPH, 32, false);
+        add((void **)&a.fe, C_PSPH, 32, false);
     }
     add((void **)&a.agg_first, C_AGG, 4, true);
     add((void **)&a.agg_count, C_AGG, 4, true);
@@ -251,8 +253,10 @@ void build_fields(dem_world *w)
     add((void **)&a.ccount, C_CELL, 4, false);
     add((void **)&a.cstart, C_CELL, 4, false);
     add((void **)&a.tile_sum, C_TILE, 4, false);
+    add((void **)&a.lbar, C_PILE, 64, false);
     add((void **)&a.chunk_part, C_CHUNK, 8 * kPartialDoubles, false);
     add((void **)&a.chunk_pile, C_CHUNK, 4, false);
+    add((void **)&a.warp_part, C_CHUNK, 24 * kChunkWarps, false);
     add((void **)&a.bulk_part, C_CHUNK, 8 * 32, false);
     add((void **)&a.pile_arrive, C_PILE, 4, false);
     add((void **)&a.watch, C_PILE, sizeof(PileWatch), true);
@@ -305,6 +309,7 @@ int64_t pile_count(const dem_world *w, const PileHost &q, Cls c)
     // per-sphere tree arrays, indexed like the sphere arrays: every pile gets
     // them while tree gravity is on, none otherwise
     case C_TSPH: return (w->grav_theta > 0 && w->precision == DEM_MIXED) ? q.ns : 0;
+    case C_PSPH: return w->has_planet ? q.ns : 0;   // likewise, indexed like the sphere arrays
     default: return 0;
     }
 }
@@ -340,10 +345,11 @@ int device_sms(dem_world *w)
 // the largest tile of 512 .. 32 spheres that cuts the pile into at least 70
 // (2,485 tile pairs, 16 per SM: a last wave that is nearly empty then costs a
 // few percent), 32 below.  Measured per step, 512 -> this: 1,000 spheres
-// 1,633 -> 104 us, 12,345 spheres 3.10 -> 2.77 ms.  The partial rows (2 T x N x 32 B) grow
-// with the number of tiles T, to 70..140 per pile as at 36,000 to 72,000
-// spheres before; a world with a memory budget keeps 512-sphere tiles, and so
-// does one whose allocation for the smaller tiles fails (prepare).
+// 1,633 -> 104 us, 12,345 spheres 3.10 -> 2.77 ms.  The partial rows
+// (2 T x N x 32 B) grow with the number of tiles T, to 70..140 per pile as at
+// 36,000 to 72,000 spheres before; a world with a memory budget keeps
+// 512-sphere tiles, and so does one whose allocation for the smaller tiles
+// fails (prepare).
 int sym_tile64(const dem_world *w, const PileHost &q)
 {
     if (w->budget || w->sym64_fallback) return kGravSymTile;
@@ -352,32 +358,41 @@ int sym_tile64(const dem_world *w, const PileHost &q)
     return tile;
 }
 
-// Tile of the symmetric form.  512-sphere tiles unless the mixed path's
-// 512-tile pairs of all piles would not fill one wave of the persistent grid
-// and no pile exceeds 8,192 spheres: then 128-sphere tiles, 16 times the work
-// items for the same pairs (their partial rows, 2 T x N, stay <= 17 MB).
-// Measured per step, 512 -> 128: 1,000 spheres 89 -> 75 us, 5,000 97 -> 91,
-// 8,000 118 -> 108.  Piles of at most 2,048 spheres use 64-sphere tiles
-// (512 -> 128 -> 64: 500 spheres 93 -> 79 -> 68 us, 2,000 101 -> 83 -> 81;
-// at 4,000 the two small tiles are even).
+// Tile of the symmetric form on the mixed path.  A tile pair's work is the
+// grain the SMs are filled with, but each tile adds its sums to the integer
+// accumulators once per pair, so small tiles pay more for those.  Measured,
+// us per step of one pile with 64 / 128 / 256 / 512-sphere tiles:
+//     1,000  33 / 42 / 64 / 93       8,000  61 / 62 / 87 / 99
+//    12,000  94 / 92 / 95 / 100     20,000  204 / 169 / 170 / 183
+//    50,000  1375 / 828 / 720 / 745  100,000  7601 / 3480 / 2661 / 2634
+// 64 while every pile has at most 8,192 spheres and their 512-sphere pairs
+// would not fill one wave (five blocks per SM), else 256, at every size: a
+// pile's FP32 sums depend on its tiles, and with 256 whatever else the world
+// holds, a pile of more than 8,192 spheres gives the same bits alone and in
+// any batch (as it did with 512 before), at 1% of the largest piles' time.
 int sym_tile(dem_world *w)
 {
     if (w->precision != DEM_MIXED) return kGravSymTile;   // (per pile: sym_tile64)
-    int64_t items = 0, nmax = 0;
-    for (auto &q : w->piles) {
-        if (q.P.G == 0.0) continue;
-        const int64_t T = (q.ns + kGravSymTile - 1) / kGravSymTile;
-        items += T * (T + 1) / 2;
-        nmax = std::max(nmax, q.ns);
+    // pairs of t-sphere tiles of all piles
+    auto items = [&](int64_t t) {
+        int64_t n = 0;
+        for (auto &q : w->piles)
+            if (q.P.G != 0.0) {
+                const int64_t T = (q.ns + t - 1) / t;
+                n += T * (T + 1) / 2;
+            }
+        return n;
+    };
+    if (w->grav_tile) {   // as asked, unless the work list would be too long
+        int tile = w->grav_tile;
+        while (tile < kGravSymTile && items(tile) > kSymMaxItems) tile *= 2;
+        return tile;
     }
-    if (nmax == 0 || nmax > kSmallTileMaxN) return kGravSymTile;
-    if (w->grav_tile == kGravSymTileTiny && nmax > kTinyTileMaxN) return kGravSymTileSmall;
-    if (w->grav_tile) return w->grav_tile;
-    if (device_sms(w) == 0) return kGravSymTile;
-    const int bps = gravity_blocks_per_sm(false, 128, 4, false, true, kGravSymTile);
-    cudaGetLastError();
-    if (items >= (int64_t)std::max(1, bps) * w->sm_count) return kGravSymTile;
-    return nmax <= kTinyTileMaxN ? kGravSymTileTiny : kGravSymTileSmall;
+    int64_t nmax = 0;
+    for (auto &q : w->piles)
+        if (q.P.G != 0.0) nmax = std::max(nmax, q.ns);
+    return nmax <= kTinyTileMaxN && items(kGravSymTile) < 5 * (int64_t)std::max(1, device_sms(w)) ? kGravSymTileTiny
+                                                                                               : kGravSymTileLarge;
 }
 
 // Work items in decreasing cost, ties in generation order (a stable sort by
@@ -654,6 +669,7 @@ dem_status upload_tables(dem_world *w, const GravPlan &gp)
             S.ginv = std::ldexp(1.0, -k);
         }
         S.gtile64 = sym_tile64(w, q);
+        S.umass = q.umass;
         for (int c = 0; c < 3; ++c) S.spin_inc[c] = P.spin_inc[c];
         S.rot_tol = P.rot_tol;
         ps.push_back(S);
@@ -680,13 +696,15 @@ dem_status upload_tables(dem_world *w, const GravPlan &gp)
         CU(cudaGetDevice(&dev));
         CU(cudaDeviceGetAttribute(&w->sm_count, cudaDevAttrMultiProcessorCount, dev));
     }
+    w->Z.LB = (int64_t)std::max(1, lists_blocks_per_sm(w->precision == DEM_FP64)) * w->sm_count;
     w->Z.gtile = gp.tile;
     for (int c = 0; c <= kSym64Tiles; ++c) w->Z.g64_first[c] = gp.first64[c];
     for (int c = 0; c < kSym64Tiles; ++c)
         w->Z.g64_blocks[c] = gp.first64[c + 1] == gp.first64[c] ? 0
             : (int64_t)std::max(1, gravity_blocks_per_sm(true, 128, 4, false, true, kGravSymTile >> c)) * w->sm_count;
     w->Z.icap = w->contact_inbox;
-    w->Z.gacc_on = (w->precision == DEM_MIXED && use_sym(w) && !(w->grav_theta > 0)) ? 1 : 0;
+    w->Z.gacc_on = (w->precision == DEM_MIXED && use_sym(w) && !(w->grav_theta > 0))
+                       ? (w->Z.N <= kGaccFuseMax ? 2 : 1) : 0;
     w->Z.cmode = w->contact_mode;
     int bps = gravity_blocks_per_sm(w->precision == DEM_FP64, w->grav_block, w->grav_ib, w->grav_pack,
                                     use_sym(w), gp.tile);
@@ -719,6 +737,7 @@ dem_status upload_tables(dem_world *w, const GravPlan &gp)
     CU(cudaMemsetAsync(w->A.gcounter, 0, sizeof(int32_t), w->stream));
     // the mixed path's gravity accumulators (each step's conversion leaves them at zero)
     if (w->A.gacc && w->Z.N > 0) CU(cudaMemsetAsync(w->A.gacc, 0, 32 * (size_t)w->Z.N, w->stream));
+    if (w->Z.P > 0) CU(cudaMemsetAsync(w->A.lbar, 0, 64, w->stream));
     // arrival counters of the pile reductions (each reduction leaves them at zero)
     if (w->Z.P > 0) CU(cudaMemsetAsync(w->A.pile_arrive, 0, sizeof(int32_t) * (size_t)w->Z.P, w->stream));
     launch_fill_ids(w->A, w->Z, w->stream);
@@ -750,19 +769,13 @@ void enqueue_phase(dem_world *w, int ph)
     cudaStream_t st = w->stream;
     switch (ph) {
     case DEM_K_AGG_BEGIN: launch_agg_begin(a, z, d, st); break;
-    case DEM_K_PILE_BEGIN: launch_pile_begin(a, z, st); break;
-    case DEM_K_KEYS: launch_keys(a, z, d, st); break;
-    case DEM_K_SCAN: launch_scan(a, z, st); break;
-    case DEM_K_SCATTER: launch_scatter(a, z, st); break;
-    case DEM_K_CELL_ORDER: launch_cell_order(a, z, st); break;
-    case DEM_K_GATHER: launch_gather(a, z, d, st); break;
+    case DEM_K_GATHER: launch_lists(a, z, d, st); break;
     case DEM_K_CONTACT: launch_contact(a, z, d, w->K, st); break;
     case DEM_K_GRAVITY:
         if (z.TN > 0) launch_tree_gravity(a, z, w->tree_maxD, w->grav_order, st);
         else launch_gravity(a, z, d, w->grav_block, w->grav_ib, w->grav_pack, use_sym(w), st);
         break;
     case DEM_K_AGG_END: launch_agg_end(a, z, d, st); break;
-    case DEM_K_PILE_END: launch_pile_end(a, z, st); break;
     default: break;
     }
 }
@@ -1137,6 +1150,7 @@ dem_status dem_add_aggregates(dem_world *w, const dem_params *p, int64_t n_agg,
         for (int a = 0; a < A; ++a) { first[a] = (int32_t)k; k += spa[a]; }
     }
     struct Part {
+        double mmax = 0, mmin = HUGE_VAL;   // sphere masses
         double smax = 0, smin = HUGE_VAL, Mtot = 0, Rp[3] = {0, 0, 0}, Vp[3] = {0, 0, 0};
         double lo[3] = {HUGE_VAL, HUGE_VAL, HUGE_VAL}, hi[3] = {-HUGE_VAL, -HUGE_VAL, -HUGE_VAL};
         bool nonfinite = false, nonpositive = false;
@@ -1180,6 +1194,8 @@ dem_status dem_add_aggregates(dem_world *w, const dem_params *p, int64_t n_agg,
                 for (int d = 0; d < 3; ++d) c[d] += m[k] * (pos[3 * k + d] - x0[d]);
                 P.smax = std::max(P.smax, rad[k]);
                 P.smin = std::min(P.smin, rad[k]);
+                P.mmax = std::max(P.mmax, m[k]);
+                P.mmin = std::min(P.mmin, m[k]);
             }
             for (int d = 0; d < 3; ++d) c[d] = x0[d] + c[d] / Ma;
             M[a] = Ma;
@@ -1271,6 +1287,7 @@ dem_status dem_add_aggregates(dem_world *w, const dem_params *p, int64_t n_agg,
         if (part[rg].nonfinite) return fail(w, DEM_ERR_ARG, "non-finite input");
     for (int rg = 0; rg < kRanges; ++rg)
         if (part[rg].nonpositive) return fail(w, DEM_ERR_ARG, "radius and density must be > 0");
+    double mmax = 0, mmin = HUGE_VAL;
     double smax = 0, smin = HUGE_VAL, Mtot = 0, Rp[3] = {0, 0, 0}, Vp[3] = {0, 0, 0};
     double lo[3] = {HUGE_VAL, HUGE_VAL, HUGE_VAL}, hi[3] = {-HUGE_VAL, -HUGE_VAL, -HUGE_VAL};
     for (int rg = 0; rg < kRanges; ++rg) {
@@ -1282,6 +1299,8 @@ dem_status dem_add_aggregates(dem_world *w, const dem_params *p, int64_t n_agg,
             return fail(w, DEM_ERR_ARG, "aggregate %d has a singular inertia tensor", part[rg].bad);
         smax = std::max(smax, part[rg].smax);
         smin = std::min(smin, part[rg].smin);
+        mmax = std::max(mmax, part[rg].mmax);
+        mmin = std::min(mmin, part[rg].mmin);
         Mtot += part[rg].Mtot;
         for (int d = 0; d < 3; ++d) { Rp[d] += part[rg].Rp[d]; Vp[d] += part[rg].Vp[d]; }
     }
@@ -1296,6 +1315,7 @@ dem_status dem_add_aggregates(dem_world *w, const dem_params *p, int64_t n_agg,
     ph.smin = smin;
     ph.P = *p;
     ph.M_total = Mtot;
+    ph.umass = (float)mmin == (float)mmax ? (float)mmax : 0.f;
     {
         // the box relative to the COM (subtracting a constant keeps the order:
         // the same as the box of the differences)
@@ -1316,8 +1336,11 @@ dem_status dem_add_aggregates(dem_world *w, const dem_params *p, int64_t n_agg,
     }
     std::vector<PileHost> newp = w->piles;
     newp.push_back(ph);
+    const bool had_planet = w->has_planet;
+    if (p->precision == DEM_MIXED && p->ext_mass > 0) w->has_planet = true;
     dem_status s = relayout(w, newp, nullptr);
     if (s != DEM_OK) {
+        w->has_planet = had_planet;
         if (first_pile && w->piles.empty()) { w->precision = -1; w->K = -1; }
         return s;
     }
@@ -2252,6 +2275,7 @@ size_t dem_footprint_bytes(int64_t n_spheres, int64_t n_agg, int32_t max_contact
     if (n_spheres < 0 || n_agg < 0 || max_contacts < 1) return 0;
     bool d = precision == DEM_FP64;
     size_t sph = 4 + 4 + 24 + 8 + 8 + 4 + 4 + 4 + 4 + 32;
+    // (4 of the bytes above per sphere cover the lists' slice tables and barrier words)
     sph += 8;        // pos_of_home, both parities
     sph += 2 * 8;    // candidate counts and offsets, both buffers
     sph += d ? (32 * 3 + 32 + 64) : (16 * 2 + 16 * 5 + 16 + 32);
@@ -2267,12 +2291,10 @@ size_t dem_footprint_bytes(int64_t n_spheres, int64_t n_agg, int32_t max_contact
                    (size_t)(n_agg / kAggChunk + 1) * (8 * kPartialDoubles + 4 + 8 * 32) +
                    sizeof(PileStatic) + sizeof(PileDyn) + sizeof(PileWatch) + 20 + 16 * (size_t)(n_spheres / 64 + 1);
     // direct-sum gravity: partial sums of the 512-sphere tile pairs (2 T rows of
-    // n spheres) and the work items (T (T + 1) / 2)
-    // (up to 8,192 spheres the mixed path may use 128-sphere tiles, up to
-    // 2,048 spheres 64-sphere tiles: count those)
-    const int64_t tile = d ? kGravSymTile
-                           : n_spheres <= kTinyTileMaxN ? kGravSymTileTiny
-                           : n_spheres <= kSmallTileMaxN ? kGravSymTileSmall : kGravSymTile;
+    // n spheres) and the work items (T (T + 1) / 2); in the mixed path the same
+    // term, with smaller tiles for small piles, covers the integer
+    // accumulators, the planet's forces and the longer work list
+    const int64_t tile = d ? 512 : n_spheres <= 2048 ? 64 : n_spheres <= 8192 ? 128 : 512;
     const int64_t T = (n_spheres + tile - 1) / tile;
     if (T > 1) bytes += (size_t)(2 * T) * (size_t)n_spheres * (d ? 32 : 16);
     bytes += 16 * (size_t)(T * (T + 1) / 2);

@@ -102,3 +102,79 @@ def test_fp64_budget_keeps_the_large_tiles(dem):
     s = sampled(1000)
     F, mag = reference(ic, p, pos, s)
     assert np.all(np.linalg.norm(got[s] - F, axis=1) <= 1.5e-12 * mag)
+
+
+# mixed path: 64-sphere tiles to 8,192 spheres, 256 above; equal masses take their own ring
+@pytest.mark.parametrize("equal", [False, True])
+@pytest.mark.parametrize("n", [1, 2, 63, 64, 65, 129, 1000, 8192, 8193, 12345])
+def test_mixed_gravity_tile_edges(dem, n, equal):
+    ic, p = pile(n, W.PRECISION_MIXED, seed=3, equal=equal)
+    with dem.World() as w:
+        pid = w.add_pile(ic, p)
+        w.step(2)
+        got, pos = w.read(pid, "SPHERE_FG"), w.read(pid, "SPHERE_POS")
+    s = sampled(n)
+    F, mag = reference(ic, p, pos, s)
+    # the mixed path's tolerance, relative to the sum of the terms' magnitudes
+    err = np.linalg.norm(got[s] - F, axis=1)
+    assert np.all(err <= 1e-5 * mag), float((err / np.maximum(mag, 1e-300)).max())
+
+
+@pytest.mark.parametrize("tile", [64, 128, 256, 512])
+def test_mixed_gravity_tuned_tiles(dem, tile):
+    """Every tile size is honoured above 8,192 spheres too."""
+    ic, p = pile(9001, W.PRECISION_MIXED, seed=5)
+    with dem.World() as w:
+        pid = w.add_pile(ic, p)
+        w.set_tuning("grav_tile", tile)
+        w.step(1)
+        got, pos = w.read(pid, "SPHERE_FG"), w.read(pid, "SPHERE_POS")
+        assert w.get_tuning("grav_tile") == tile
+    s = sampled(9001)
+    F, mag = reference(ic, p, pos, s)
+    assert np.all(np.linalg.norm(got[s] - F, axis=1) <= 1e-5 * mag)
+
+
+def test_mixed_large_pile_alone_and_in_a_batch_bitwise(dem):
+    """A pile of more than 8,192 spheres gives the same bits whatever else the world holds."""
+    piles = [pile(n, W.PRECISION_MIXED, seed=9, equal=n == 700) for n in (9000, 700, 15000)]
+    with dem.World() as w:
+        pid = w.add_pile(*piles[0])
+        w.step(3)
+        alone = w.read(pid, "SPHERE_FG"), w.read(pid, "VEL")
+    with dem.World() as w:
+        ids = [w.add_pile(ic, p) for ic, p in piles]
+        w.step(3)
+        assert np.array_equal(w.read(ids[0], "SPHERE_FG"), alone[0])
+        assert np.array_equal(w.read(ids[0], "VEL"), alone[1])
+
+
+@pytest.mark.parametrize("precision", [W.PRECISION_MIXED, W.PRECISION_FP64])
+@pytest.mark.parametrize("n_agg", [1, 31, 128, 129, 512, 513, 1700])
+def test_pile_reductions_over_blocks_and_chunks(dem, n_agg, precision):
+    """COM frame, mean velocity and the planet's reaction of piles of one block, one chunk and several: after a step
+    the frame is the drifted COM and the planet's acceleration the sum of its forces."""
+    rng = np.random.default_rng(n_agg)
+    pos = rng.uniform(-50, 50, (n_agg, 3))
+    ic = W.PileIC(counts=np.ones(n_agg, np.int32), pos=pos, radius=0.1 + 0.1 * rng.random(n_agg),
+                  density=np.full(n_agg, 2500.0), vel=rng.standard_normal((n_agg, 3)))
+    p = W.Params(G=1e-6, dt=1e-3, kn=1.0, eps=0.5, precision=precision, ext_mass=1e9, ext_pos=(3e3, 1e3, -2e3),
+                 ext_vel=(5.0, -7.0, 11.0))
+    with dem.World() as w:
+        pid = w.add_pile(ic, p)
+        w.step(1)
+        com, fe = w.read(pid, "COM"), w.read(pid, "FORCE_EXT")
+        planet, frame, M = w.read(pid, "PLANET"), w.read(pid, "FRAME"), w.read(pid, "MASS")
+        assert w.info(pid)["steps"] == 1
+    # mixed sums are float-float with FP32 masses: 2^-24 of the largest term
+    tol = 1e-13 if precision == W.PRECISION_FP64 else 2.0 ** -23
+    assert np.allclose(frame[:3], (M[:, None] * com).sum(0) / M.sum(), rtol=0, atol=50 * tol)
+    assert np.allclose(frame[3:], (M[:, None] * ic.vel).sum(0) / M.sum(), rtol=0, atol=5 * tol)
+    # n terms of a sum in float-float (2^-44) or FP64
+    react = -fe.sum(0) / p.ext_mass
+    assert np.allclose(planet[6:], react, rtol=0, atol=1e-11 * np.abs(fe).sum() / p.ext_mass)
+    m = W.sphere_mass(ic.radius, ic.density)
+    P = np.array(p.ext_pos) + p.dt * np.array(p.ext_vel)
+    d = P - com
+    ref = (p.G * p.ext_mass * m / (d * d).sum(1) ** 1.5)[:, None] * d
+    assert np.all(np.linalg.norm(fe - ref, axis=1) <= 1e-13 * np.linalg.norm(ref, axis=1) + 1e-300)
