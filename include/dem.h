@@ -114,9 +114,8 @@ enum dem_field {
 };
 
 /* Pile flag bits (dem_pile_flags). */
-/* DEM_FLAG_TREE: tree gravity ran out of traversal stack for some group of
- * spheres and took a cell as far that it would have opened (less accurate,
- * not fatal). */
+/* DEM_FLAG_TREE: reserved (the traversal stack of tree gravity holds every
+ * walk of the deepest tree). */
 /* DEM_FLAG_GRAV_RANGE (mixed precision, direct sum): a tile's gravity sum on
  * some sphere exceeded the range of the pile's fixed-point gravity
  * accumulators.  The range is set when the pile is added, from its total mass
@@ -465,7 +464,7 @@ dem_status dem_probe_peak(int32_t kind, int64_t size, int32_t reps, const void *
 
 /* Device bytes one pile of this size needs with direct-sum gravity (state, sorted
  * copies, cells, history, gravity partial sums).  Tree gravity (grav_theta > 0)
- * needs instead about 1.1 KB per sphere plus 280 B per tree cell. */
+ * needs instead about 0.4 KB per sphere plus 280 B per tree cell. */
 size_t dem_footprint_bytes(int64_t n_spheres, int64_t n_agg, int32_t max_contacts,
                            int32_t precision);
 

@@ -48,6 +48,8 @@ __host__ __device__ __forceinline__ int64_t cell_count(int nx, int ny, int nz)
     return (int64_t)((nx + 3) >> 2) * ((ny + 3) >> 2) * ((nz + 3) >> 2) * 64;
 }
 
+constexpr int kTreeParts = 16;      // tree gravity: warps that share a group's walk
+
 constexpr int kSym64Tiles = 5;   // FP64 symmetric gravity: tiles of 512, 256, 128, 64 or 32 spheres
 
 // Static description of one pile (host-owned; re-uploaded on membership change).
@@ -244,7 +246,7 @@ struct Arrays {
     int32_t *tkey, *trank, *tsorted;
     float4 *tpos;        // leaf-ordered positions (+mass)
     int32_t *tagg;       // leaf-ordered aggregates
-    float4 *tpart;       // [64][N] partial sums of the 64 subtrees at level 2
+    float4 *tpart;       // [kTreeParts][N] partial sums of the walk's warps
     int *tbox;
     float4 *tnode;       // per node 9 float4: COM, M, opening radius^2, traceless moments of ranks 2-4
     float4 *traw;        // per node 8 float4: raw moments of ranks 2-4 about the COM (upward pass)

@@ -10,7 +10,7 @@
 // about the COM (shifted exactly from child to parent), kept for evaluation
 // as their traceless parts -- quadrupole, octupole and hexadecapole, the
 // expansion order of the paper's tree code (Sec. 2.1) -- then each warp
-// walks the tree depth-first for 32 spheres at once.  A cell is accepted when
+// walks the tree for 32 spheres at once.  A cell is accepted when
 // the group of spheres is farther from its COM than size/theta +
 // |COM - centre| (so no sphere is inside an accepted cell) and contributes
 // the gradient of its multipole potential up to rank 4 (or rank 2, the
@@ -23,6 +23,7 @@
 // per-sphere gravity array as the direct sum.
 #include "dem_internal.h"
 #include "devmath.cuh"
+#include "f32x2.cuh"
 #include "launch.cuh"
 
 namespace dem {
@@ -53,49 +54,68 @@ __device__ __forceinline__ uint32_t spread3(uint32_t v)
     return v;
 }
 
-// One block per pile: reset the box and the leaf counts.
+// Reset the boxes and the leaf counts.
 __global__ void k_tree_init(Arrays a, Sizes z)
 {
     pdl_enter();
-    const int p = blockIdx.x;
-    if (p >= z.P || !tree_pile(a, p)) return;
-    const PileStatic &S = a.ps[p];
-    if (threadIdx.x < 3) {
-        a.tbox[8 * p + threadIdx.x] = f2o(3.0e38f);
-        a.tbox[8 * p + 3 + threadIdx.x] = f2o(-3.0e38f);
+    const int64_t g = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    if (g < 6 * z.P) {
+        const int p = (int)(g / 6), c = (int)(g % 6);
+        a.tbox[8 * p + c] = f2o(c < 3 ? 3.0e38f : -3.0e38f);
     }
-    const int64_t nl = (int64_t)1 << (3 * S.tD);
-    for (int64_t c = threadIdx.x; c < nl; c += blockDim.x) a.tleaf[S.tleaf0 + c] = make_int2(0, 0);
+    if (g >= z.TL) return;
+    const int p = a.tleaf_pile[g];
+    if (p >= 0 && tree_pile(a, p)) a.tleaf[g] = make_int2(0, 0);
 }
 
-// Box of each pile: per warp, lanes of the same pile reduce their min/max
-// first (piles are contiguous, so a warp holds one or two), then one atomic
-// per warp and pile (min/max do not depend on the order).
-__global__ void k_tree_box(Arrays a, Sizes z)
+// Box of each pile: every warp reduces its spheres' min/max (piles are
+// contiguous, so a warp holds one or two), a block that lies in one pile its
+// warps', then one atomic per component (min/max do not depend on the order).
+// An atomic per warp and component was 16 us at 100,000 spheres (ncu).
+constexpr int kBoxThreads = 256;
+__global__ void __launch_bounds__(kBoxThreads) k_tree_box(Arrays a, Sizes z)
 {
     pdl_enter();
     const unsigned FULL = 0xffffffffu;
-    const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    const int64_t b0 = (int64_t)blockIdx.x * kBoxThreads, i = b0 + threadIdx.x;
     const int p = i < z.N ? a.sph_pile[i] : -1;
     const bool act = p >= 0 && tree_pile(a, p);
     const float4 x = act ? a.gpos32[i] : make_float4(0.f, 0.f, 0.f, 0.f);
+    const int o[3] = {f2o(x.x), f2o(x.y), f2o(x.z)};
+    __shared__ int sh[kBoxThreads / 32][6];
+    const int p0 = a.sph_pile[b0], lane = threadIdx.x & 31;
+    const int64_t e = b0 + kBoxThreads < z.N ? b0 + kBoxThreads : z.N;
+    const bool one = a.sph_pile[e - 1] == p0;   // uniform over the block
     unsigned todo = __ballot_sync(FULL, act);
+    if (one && !tree_pile(a, p0)) return;
+    int v[6];
+    if (one) {
+        for (int c = 0; c < 3; ++c) {
+            v[c] = __reduce_min_sync(FULL, act ? o[c] : 0x7fffffff);
+            v[3 + c] = __reduce_max_sync(FULL, act ? o[c] : (int)0x80000000);
+        }
+        if (lane == 0)
+            for (int c = 0; c < 6; ++c) sh[threadIdx.x >> 5][c] = v[c];
+        __syncthreads();
+        if (threadIdx.x < 6) {
+            const int c = threadIdx.x;
+            int m = sh[0][c];
+            for (int w = 1; w < kBoxThreads / 32; ++w) m = c < 3 ? min(m, sh[w][c]) : max(m, sh[w][c]);
+            if (c < 3) atomicMin(&a.tbox[8 * p0 + c], m);
+            else atomicMax(&a.tbox[8 * p0 + c], m);
+        }
+        return;
+    }
     while (todo) {
         const int leader = __ffs(todo) - 1;
         const int pp = __shfl_sync(FULL, p, leader);
         const bool mine = act && p == pp;
         todo &= ~__ballot_sync(FULL, mine);
-        int v[6] = {f2o(x.x), f2o(x.y), f2o(x.z), f2o(x.x), f2o(x.y), f2o(x.z)};
-        if (!mine) {
-            v[0] = v[1] = v[2] = 0x7fffffff;
-            v[3] = v[4] = v[5] = (int)0x80000000;
+        for (int c = 0; c < 3; ++c) {
+            v[c] = __reduce_min_sync(FULL, mine ? o[c] : 0x7fffffff);
+            v[3 + c] = __reduce_max_sync(FULL, mine ? o[c] : (int)0x80000000);
         }
-        for (int o = 16; o > 0; o >>= 1)
-            for (int c = 0; c < 6; ++c) {
-                const int u = __shfl_xor_sync(FULL, v[c], o);
-                v[c] = c < 3 ? min(v[c], u) : max(v[c], u);
-            }
-        if ((threadIdx.x & 31) == leader)
+        if (lane == leader)
             for (int c = 0; c < 6; ++c) {
                 if (c < 3) atomicMin(&a.tbox[8 * pp + c], v[c]);
                 else atomicMax(&a.tbox[8 * pp + c], v[c]);
@@ -134,32 +154,76 @@ __global__ void k_tree_keys(Arrays a, Sizes z)
     a.trank[i] = atomicAdd(&a.tleaf[S.tleaf0 + key].y, 1);
 }
 
-// One block of 1024 threads per pile: exclusive scan of the leaf counts.
-__global__ void k_tree_scan(Arrays a, Sizes z)
+// Exclusive scan of each pile's leaf counts by blocks of kLeafTile leaves
+// (blockIdx.x: pile): first the tiles' sums, then every block adds the sums
+// before its own (at most 128) and scans its leaves.  One block per pile, each
+// thread walking its own range of leaves, was 60 us at 32,768 leaves (ncu).
+constexpr int kLeafTile = 2048, kScanThreads = 256;
+// scratch before the walk writes its partial sums: the leaf-sorted but not yet
+// ordered spheres, then the leaf tiles' sums (fewer than the pile's spheres)
+__device__ __forceinline__ int *tree_unordered(const Arrays &a) { return (int *)a.tpart; }
+__device__ __forceinline__ int *tree_tile_sums(const Arrays &a, const Sizes &z, const PileStatic &S)
+{
+    return (int *)a.tpart + z.N + S.s0;
+}
+
+// Inclusive prefix sum over the block's kScanThreads threads.
+__device__ __forceinline__ int scan256(int v, int *ws)
+{
+    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+    for (int o = 1; o < 32; o <<= 1) {
+        const int y = __shfl_up_sync(0xffffffffu, v, o);
+        if (lane >= o) v += y;
+    }
+    if (lane == 31) ws[wid] = v;
+    __syncthreads();
+    for (int k = 0; k < kScanThreads / 32; ++k)
+        if (k < wid) v += ws[k];
+    return v;
+}
+
+__global__ void __launch_bounds__(kScanThreads) k_tree_sums(Arrays a, Sizes z)
 {
     pdl_enter();
     const int p = blockIdx.x;
-    if (p >= z.P || !tree_pile(a, p)) return;
+    if (!tree_pile(a, p)) return;
     const PileStatic &S = a.ps[p];
-    const int64_t nl = (int64_t)1 << (3 * S.tD);
-    const int64_t per = (nl + blockDim.x - 1) / blockDim.x;
-    const int64_t b0 = threadIdx.x * per, b1 = min(nl, b0 + per);
-    int loc = 0;
-    for (int64_t c = b0; c < b1; ++c) loc += a.tleaf[S.tleaf0 + c].y;
-    __shared__ int buf[1024];
-    buf[threadIdx.x] = loc;
+    const int nl = 1 << (3 * S.tD), l0 = blockIdx.y * kLeafTile;
+    if (l0 >= nl || nl <= kLeafTile) return;
+    __shared__ int ws[kScanThreads / 32];
+    int s = 0;
+    for (int k = threadIdx.x; k < kLeafTile; k += kScanThreads) s += a.tleaf[S.tleaf0 + l0 + k].y;
+    s = scan256(s, ws);
+    if (threadIdx.x == kScanThreads - 1) tree_tile_sums(a, z, S)[blockIdx.y] = s;
+}
+
+__global__ void __launch_bounds__(kScanThreads) k_tree_scan(Arrays a, Sizes z)
+{
+    pdl_enter();
+    const int p = blockIdx.x;
+    if (!tree_pile(a, p)) return;
+    const PileStatic &S = a.ps[p];
+    const int nl = 1 << (3 * S.tD), l0 = blockIdx.y * kLeafTile;
+    if (l0 >= nl) return;
+    constexpr int kPer = kLeafTile / kScanThreads;
+    __shared__ int ws[kScanThreads / 32], before;
+    int2 *leaf = a.tleaf + S.tleaf0 + l0;
+    // tiles before this one (at most 127)
+    int s = threadIdx.x < blockIdx.y ? tree_tile_sums(a, z, S)[threadIdx.x] : 0;
+    s = scan256(s, ws);
+    if (threadIdx.x == kScanThreads - 1) before = s;
     __syncthreads();
-    for (int o = 1; o < 1024; o <<= 1) {
-        const int add = threadIdx.x >= (unsigned)o ? buf[threadIdx.x - o] : 0;
-        __syncthreads();
-        buf[threadIdx.x] += add;
-        __syncthreads();
+    int c[kPer], loc = 0;
+    for (int k = 0; k < kPer; ++k) {
+        const int l = threadIdx.x * kPer + k;
+        c[k] = l0 + l < nl ? leaf[l].y : 0;
+        loc += c[k];
     }
-    int run = buf[threadIdx.x] - loc;
-    for (int64_t c = b0; c < b1; ++c) {
-        int2 &L = a.tleaf[S.tleaf0 + c];
-        L.x = run;
-        run += L.y;
+    int run = before + scan256(loc, ws) - loc;
+    for (int k = 0; k < kPer; ++k) {
+        const int l = threadIdx.x * kPer + k;
+        if (l0 + l < nl) leaf[l].x = run;
+        run += c[k];
     }
 }
 
@@ -171,36 +235,15 @@ __global__ void k_tree_scatter(Arrays a, Sizes z)
     const int p = a.sph_pile[i];
     if (!tree_pile(a, p)) return;
     const PileStatic &S = a.ps[p];
-    a.tsorted[S.s0 + a.tleaf[S.tleaf0 + a.tkey[i]].x + a.trank[i]] = (int32_t)(i - S.s0);
+    tree_unordered(a)[S.s0 + a.tleaf[S.tleaf0 + a.tkey[i]].x + a.trank[i]] = (int32_t)(i - S.s0);
 }
 
-// The first position of each leaf orders the leaf by home index (insertion
-// sort; leaves hold a handful of spheres): deterministic sums.
-__global__ void k_tree_leaf_order(Arrays a, Sizes z)
-{
-    pdl_enter();
-    const int64_t k = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (k >= z.N) return;
-    const int p = a.sph_pile[k];
-    if (!tree_pile(a, p)) return;
-    const PileStatic &S = a.ps[p];
-    int32_t *srt = a.tsorted + S.s0;
-    const int kl = (int)(k - S.s0);
-    const int2 L = a.tleaf[S.tleaf0 + a.tkey[S.s0 + srt[kl]]];
-    if (kl != L.x) return;
-    for (int x = 1; x < L.y; ++x) {
-        const int v = srt[L.x + x];
-        int y = x - 1;
-        while (y >= 0 && srt[L.x + y] > v) {
-            srt[L.x + y + 1] = srt[L.x + y];
-            --y;
-        }
-        srt[L.x + y + 1] = v;
-    }
-}
-
-// Leaf-ordered copies of the spheres' positions (+mass) and aggregates, so
-// that a leaf's spheres are contiguous for the moments and the walk.
+// Every sphere finds its place in its leaf, ordered by home index (the number
+// of the leaf's spheres with a smaller one: leaves hold a handful), which makes
+// the sums deterministic, and puts its position (+mass) and aggregate there,
+// so that a leaf's spheres are contiguous for the moments and the walk.
+// (An insertion sort by each leaf's first thread and a gather after it were 20
+// and 6 us at 100,000 spheres.)
 __global__ void k_tree_gather(Arrays a, Sizes z)
 {
     pdl_enter();
@@ -208,10 +251,19 @@ __global__ void k_tree_gather(Arrays a, Sizes z)
     if (k >= z.N) return;
     const int p = a.sph_pile[k];
     if (!tree_pile(a, p)) return;
-    const int64_t s0 = a.ps[p].s0;
-    const int i = a.tsorted[k];
-    a.tpos[k] = a.gpos32[s0 + i];
-    a.tagg[k] = a.sph_agg[s0 + i];
+    const PileStatic &S = a.ps[p];
+    const int64_t s0 = S.s0;
+    const int *un = tree_unordered(a) + s0;
+    const int i = un[k - s0];
+    const int2 L = a.tleaf[S.tleaf0 + a.tkey[s0 + i]];
+    const float4 x = a.gpos32[s0 + i];
+    const int ag = a.sph_agg[s0 + i];
+    int r = 0;
+    for (int m = 0; m < L.y; ++m) r += un[L.x + m] < i ? 1 : 0;
+    const int64_t o = s0 + L.x + r;
+    a.tsorted[o] = i;
+    a.tpos[o] = x;
+    a.tagg[o] = ag;
 }
 
 // ---- multipole moments up to the hexadecapole
@@ -376,42 +428,36 @@ __global__ void k_tree_leaves(Arrays a, Sizes z)
 
 // Moments of level L from the 8 children: raw moments shifted from each
 // child's COM to the parent's, R_e += sum_{f <= e} C(e, f) R_child,f s^(e-f)
-// with s = child COM - parent COM (rank-1 terms vanish about a COM), one
-// thread per node of every tree pile deep enough.
-__global__ void k_tree_up(Arrays a, Sizes z, int L)
+// with s = child COM - parent COM (rank-1 terms vanish about a COM).  Eight
+// lanes per node, one per child, summed by a fixed tree; blockIdx.x:
+// pile.  With a thread per node a level of 4,096 nodes was 16
+// blocks, each thread shifting its 8 children in turn: 22 us a level (ncu).
+// Levels below the walk's start (kSplitL) are not needed.
+__global__ void __launch_bounds__(128) k_tree_up(Arrays a, Sizes z, int L)
 {
     pdl_enter();
-    const int64_t g = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (g >= z.TN) return;
-    const int p = a.tnode_pile[g];
-    if (p < 0 || !tree_pile(a, p)) return;
+    const int p = blockIdx.x;
+    if (!tree_pile(a, p)) return;
     const PileStatic &S = a.ps[p];
-    if (L >= S.tD) return;
-    const int64_t local = g - S.tnode0;
-    const int64_t o = lvl_off(L);
-    if (local < o || local >= o + ((int64_t)1 << (3 * L))) return;
-    const uint32_t m = (uint32_t)(local - o);
-    const int64_t c0 = S.tnode0 + lvl_off(L + 1) + 8 * (int64_t)m;
-    float M = 0.f;
-    float3 c = f3(0, 0, 0);
-    for (int k = 0; k < 8; ++k) {
-        const float4 A = a.tnode[kNodeF4 * (c0 + k)];
-        M += A.w;
-        c = c + A.w * f3(A.x, A.y, A.z);
-    }
+    const uint32_t t = blockIdx.y * 128 + threadIdx.x, m = t >> 3;
+    if (L >= S.tD || (blockIdx.y * 128 >> 3) >= (1u << (3 * L))) return;   // 16 nodes a block: whole blocks
+    const int64_t g = S.tnode0 + lvl_off(L) + m;
+    const int64_t cn = S.tnode0 + lvl_off(L + 1) + t;   // this lane's child
+    auto sum8 = [](float v) {
+        v += __shfl_xor_sync(0xffffffffu, v, 1);
+        v += __shfl_xor_sync(0xffffffffu, v, 2);
+        return v + __shfl_xor_sync(0xffffffffu, v, 4);
+    };
+    const float4 A = a.tnode[kNodeF4 * cn];
     float R[32];
 #pragma unroll
     for (int k = 0; k < 32; ++k) R[k] = 0.f;
-    if (M == 0.f) {
-        put_node(a, g, f3(0, 0, 0), 0.f, R, 0.f);
-        return;
-    }
-    c = (1.0f / M) * c;
-    for (int k = 0; k < 8; ++k) {
-        const float4 A = a.tnode[kNodeF4 * (c0 + k)];
-        if (A.w == 0.f) continue;
+    const float M = sum8(A.w);
+    float3 c = f3(sum8(A.w * A.x), sum8(A.w * A.y), sum8(A.w * A.z));
+    if (M > 0.f) c = (1.0f / M) * c;
+    if (A.w != 0.f) {
         float Rc[32];
-        const float4 *r = a.traw + kRawF4 * (c0 + k);
+        const float4 *r = a.traw + kRawF4 * cn;
 #pragma unroll
         for (int q = 0; q < kRawF4; ++q) {
             const float4 v = r[q];
@@ -441,8 +487,15 @@ __global__ void k_tree_up(Arrays a, Sizes z, int L)
                                 v += (binomf(ea, fa) * binomf(eb, fb) * binomf(ec, fc)) * Rf *
                                      (sx[ea - fa] * sy[eb - fb] * sz[ec - fc]);
                             }
-                    R[raw_off(n) + mono_idx(ea, eb, ec)] += v;
+                    R[raw_off(n) + mono_idx(ea, eb, ec)] = v;
                 }
+    }
+#pragma unroll
+    for (int k = 0; k < 31; ++k) R[k] = sum8(R[k]);
+    if ((t & 7) != 0) return;
+    if (M == 0.f) {
+        put_node(a, g, f3(0, 0, 0), 0.f, R, 0.f);
+        return;
     }
     float3 lo;
     float edge;
@@ -450,99 +503,119 @@ __global__ void k_tree_up(Arrays a, Sizes z, int L)
     put_node(a, g, c, M, R, opening2(c, cell_centre(lo, edge, L, m), edge / (float)(1 << L), S.theta));
 }
 
-// traversal stack per warp: each round pops up to 32 cells and pushes at most
-// 8 children of each, and cells of one level are all popped before their
-// parents' remaining siblings, so at most 8 x 32 cells of each level below
-// the walk's start wait on the stack: 256 x 4 = 1,024 for the deepest tree
-#ifndef DEM_TREE_STACK
-#define DEM_TREE_STACK 1024
-#endif
-constexpr int kTreeStack = DEM_TREE_STACK;
-// the walk of each group of spheres is split over the subtrees at this level
-#ifndef DEM_TREE_SPLIT_LEVEL
-#define DEM_TREE_SPLIT_LEVEL 2
-#endif
-constexpr int kSplitL = DEM_TREE_SPLIT_LEVEL, kSplit = 1 << (3 * kSplitL);
+// The walk of each group of spheres starts from the 64 cells of level kSplitL,
+// dealt round robin to kTreeParts warps (so that the cells around the group,
+// the long walks, go to different warps).  Measured, us per step with 8 / 16 /
+// 32 / 64 warps: 100,000-sphere cloud (theta 0.7) 530 / 508 / 545 / 632, dense
+// 50,000-sphere pile (0.5) 495 / 436 / 422 / 437, 10,000-sphere cloud 132 /
+// 116 / 118 / 122, dense 200,000-sphere pile (0.5) 1,766 / 1,814 / 1,840 /
+// 1,881; with four neighbouring cells each instead of every 16th, the first
+// two were 621 and 529.
+constexpr int kSplitL = 2;
 
-// The node's multipoles up to rank ORDER on the sphere at x: a / G.  With u
-// the unit vector from the node's COM to x and r the distance,
+// Traversal stack per warp: opened cells whose children are still to be
+// tested.  Each round pops at most 4 and tests their 32 children, so it pushes
+// at most 32, and a level's cells are pushed only when none of that level is
+// left on the stack (or the last of them are popped in the same round): at
+// most 32 cells of each of the levels 2..5 of the deepest tree.
+constexpr int kTreeStack = 32 * 4 + 4;
+
+// The multipoles up to rank ORDER of two cells on the sphere at x: a / G, one
+// cell in each half of the packed operands.  With u the unit vector from the
+// cell's COM to x and r the distance,
 //   a / G = -M u / r^2 + sum_n (n T_n . u^(n-1) - (2n+1) (T_n . u^n) u) / r^(n+2),
 // the gradient of the potential -G (M / r + sum_n T_n . x^n / r^(2n+1))
 // (unit-vector form: no power of r above the sixth is formed).
 template <int ORDER>
-__device__ __forceinline__ void node_force(const float *nd, const float4 &x, float &ax, float &ay, float &az)
+__device__ __forceinline__ void node_force2(const f2_t *nd, f2_t x, f2_t y, f2_t z, f2_t &ax, f2_t &ay, f2_t &az)
 {
-    const float dx = x.x - nd[0], dy = x.y - nd[1], dz = x.z - nd[2];
-    const float inv = rsqrtf(dx * dx + dy * dy + dz * dz);
-    const float ux = dx * inv, uy = dy * inv, uz = dz * inv;
-    float px[5], py[5], pz[5];
-    powers4(ux, px);
-    powers4(uy, py);
-    powers4(uz, pz);
-    float tx = 0.f, ty = 0.f, tz = 0.f;   // sum_n t_n / r^(n-2), Horner in 1/r from the top rank
+    const f2_t dx = f2_sub(x, nd[0]), dy = f2_sub(y, nd[1]), dz = f2_sub(z, nd[2]);
+    float ra, rb;
+    f2_unpack(f2_fma(dz, dz, f2_fma(dy, dy, f2_mul(dx, dx))), ra, rb);
+    const f2_t inv = f2_pack(rsqrtf(ra), rsqrtf(rb));
+    f2_t px[4], py[4], pz[4];
+    const f2_t one = f2_dup(1.f), zero = f2_dup(0.f);
+    auto powers = [&](f2_t d, f2_t *p) {
+        p[0] = one;
+        p[1] = f2_mul(d, inv);
+        p[2] = f2_mul(p[1], p[1]);
+        if (ORDER > 3) p[3] = f2_mul(p[2], p[1]);
+    };
+    powers(dx, px);
+    powers(dy, py);
+    powers(dz, pz);
+    f2_t tx = zero, ty = zero, tz = zero;   // sum_n t_n / r^(n-2), Horner in 1/r from the top rank
 #pragma unroll
     for (int n = ORDER; n >= 2; --n) {
-        const float *T = nd + node_off(n);
-        float vx = 0.f, vy = 0.f, vz = 0.f;   // T_n . u^(n-1)
+        const f2_t *T = nd + node_off(n);
+        f2_t vx = zero, vy = zero, vz = zero;   // T_n . u^(n-1)
 #pragma unroll
         for (int fa = n - 1; fa >= 0; --fa)
 #pragma unroll
             for (int fb = n - 1 - fa; fb >= 0; --fb) {
                 const int fc = n - 1 - fa - fb;
-                const float w = (factf(n - 1) / (factf(fa) * factf(fb) * factf(fc))) * (px[fa] * py[fb] * pz[fc]);
-                vx = fmaf(w, T[mono_idx(fa + 1, fb, fc)], vx);
-                vy = fmaf(w, T[mono_idx(fa, fb + 1, fc)], vy);
-                vz = fmaf(w, T[mono_idx(fa, fb, fc + 1)], vz);
+                const float wt = factf(n - 1) / (factf(fa) * factf(fb) * factf(fc));
+                f2_t w = fa == 0 ? (fb == 0 ? pz[fc] : fc == 0 ? py[fb] : f2_mul(py[fb], pz[fc]))
+                         : fb == 0 ? (fc == 0 ? px[fa] : f2_mul(px[fa], pz[fc]))
+                         : fc == 0 ? f2_mul(px[fa], py[fb]) : f2_mul(px[fa], f2_mul(py[fb], pz[fc]));
+                if (wt != 1.f) w = f2_mul(w, f2_dup(wt));
+                vx = f2_fma(w, T[mono_idx(fa + 1, fb, fc)], vx);
+                vy = f2_fma(w, T[mono_idx(fa, fb + 1, fc)], vy);
+                vz = f2_fma(w, T[mono_idx(fa, fb, fc + 1)], vz);
             }
-        const float sn = vx * ux + vy * uy + vz * uz;   // T_n . u^n
-        const float k1 = (float)n, k2 = (float)(2 * n + 1);
-        tx = tx * inv + (k1 * vx - k2 * sn * ux);
-        ty = ty * inv + (k1 * vy - k2 * sn * uy);
-        tz = tz * inv + (k1 * vz - k2 * sn * uz);
+        const f2_t sn = f2_fma(vz, pz[1], f2_fma(vy, py[1], f2_mul(vx, px[1])));   // T_n . u^n
+        const f2_t k1 = f2_dup((float)n), k2 = f2_mul(sn, f2_dup(-(float)(2 * n + 1)));
+        tx = f2_fma(k1, vx, f2_fma(k2, px[1], f2_mul(tx, inv)));
+        ty = f2_fma(k1, vy, f2_fma(k2, py[1], f2_mul(ty, inv)));
+        tz = f2_fma(k1, vz, f2_fma(k2, pz[1], f2_mul(tz, inv)));
     }
-    const float inv2 = inv * inv, M = nd[3];
-    ax += inv2 * (tx * inv2 - M * ux);
-    ay += inv2 * (ty * inv2 - M * uy);
-    az += inv2 * (tz * inv2 - M * uz);
+    const f2_t inv2 = f2_mul(inv, inv), M = f2_mul(nd[3], f2_dup(-1.f));
+    ax = f2_fma(inv2, f2_fma(tx, inv2, f2_mul(M, px[1])), ax);
+    ay = f2_fma(inv2, f2_fma(ty, inv2, f2_mul(M, py[1])), ay);
+    az = f2_fma(inv2, f2_fma(tz, inv2, f2_mul(M, pz[1])), az);
 }
 
-// One warp walks the tree for a group of 32 consecutive spheres in leaf order.  Each round takes up to 32 nodes off the warp's stack, one per lane,
-// and tests them in parallel against the group's bounding box: a cell is
+// One warp walks the tree for a group of 32 consecutive spheres in leaf
+// order.  Each round takes up to 4 opened cells off the warp's stack and tests
+// their children, one per lane, against the group's bounding box: a cell is
 // accepted when the box is farther from its COM than its opening radius (so
 // the test holds for every sphere of the group), an opened leaf is summed
-// directly, any other opened cell pushes its 8 children.  Every lane then
-// adds its own sphere's interaction with each accepted cell (cell data passed
-// by shuffles) and with the spheres of each opened leaf, so the arithmetic
-// has no divergence and the node loads of a round overlap.  Should the stack
-// ever fill, the cell is taken as accepted and the pile gets DEM_FLAG_TREE.
+// directly, any other opened cell goes on the stack.  Every lane then adds its
+// own sphere's interaction with the round's accepted cells, two at a time (the
+// lanes that accepted them stage them in shared memory as packed pairs), and
+// with the spheres of its opened leaves, also two at a time, so the arithmetic
+// has no divergence and the loads of a round overlap.
 // Groups are 32 consecutive spheres of one pile in leaf order, counted from
 // the pile's first sphere, so a pile's result does not depend on the other
-// piles of the batch.  The walk of each group is split over the kSplit
-// subtrees at level kSplitL (one warp each, grid dimension y), so that many
-// more warps hide the latency of the rounds; each writes its partial sum,
-// k_tree_combine adds them in order.
-#ifdef DEM_TREE_MINB
-#define DEM_TREE_BOUNDS __launch_bounds__(32, DEM_TREE_MINB)
-#else
-#define DEM_TREE_BOUNDS __launch_bounds__(32)
-#endif
+// piles of the batch.  The walk of each group is split over kTreeParts
+// warps (grid dimension y), each writing its partial sum, which k_tree_combine
+// adds in order.
+//
+// Latency-bound (the rounds depend on one another; 42% of the issue slots,
+// 28 warps an SM by registers).  A stack of cells still to be tested (4 KB)
+// held 22 warps an SM and a cell at a time took twice the instructions: the
+// 100,000-sphere cloud at theta 0.7 went from 758 to 432 us (ncu), its whole
+// step with the lighter build around the walk from 1,041 to 508 us.
 template <int ORDER>
-__global__ void DEM_TREE_BOUNDS k_tree_force(Arrays a, Sizes z)
+__global__ void __launch_bounds__(32) k_tree_force(Arrays a, Sizes z)
 {
     pdl_enter();
     // one warp per block: walks of very different lengths do not hold one
     // another's block resident
+    constexpr int kNC = ORDER > 2 ? 36 : 11;       // a cell's components in use
+    constexpr int kPairF2 = ORDER > 2 ? 38 : 14;   // components of a staged pair and padding (16-byte rows)
+    constexpr int kLeafStage = 192;                // spheres of opened leaves staged at a time
+    constexpr int kStageBytes = 16 * kPairF2 * 8 > kLeafStage * 20 ? 16 * kPairF2 * 8 : kLeafStage * 20;
     __shared__ int st[kTreeStack];
-    // accepted cells of a round (ranks above 2), then the spheres of its
-    // opened leaves, staged for every lane
-    constexpr int kStage = ORDER > 2 ? 32 * kNodeF4 : 128;
-    __shared__ float4 stage[kStage];
-    __shared__ int sagg[kStage];
+    __shared__ __align__(16) unsigned char stage[kStageBytes];
     __shared__ int lbase[32], lfirst[32];
+    f2_t *cells = (f2_t *)stage;                   // [16][kPairF2]
+    ulonglong2 *lxy = (ulonglong2 *)stage, *lzm = lxy + kLeafStage / 2;
+    int2 *lag = (int2 *)(lzm + kLeafStage / 2);
     const unsigned FULL = 0xffffffffu;
     const int lane = threadIdx.x & 31;
     const unsigned below = (1u << lane) - 1u;
-    const int sub = blockIdx.y;   // subtree: cell sub at level kSplitL
+    const int sub = blockIdx.y;      // subtree
     const int64_t wg = blockIdx.x;   // group
     if (wg >= z.TG) return;
     int lo = 0, hi = (int)z.P - 1;   // pile of the group
@@ -572,149 +645,137 @@ __global__ void DEM_TREE_BOUNDS k_tree_force(Arrays a, Sizes z)
         by1 = fmaxf(by1, __shfl_xor_sync(FULL, by1, o));
         bz1 = fmaxf(bz1, __shfl_xor_sync(FULL, bz1, o));
     }
-    const float eps2 = (float)S.eps2;
+    const f2_t e2 = f2_dup((float)S.eps2);
+    const f2_t xx = f2_dup(xi.x), xy = f2_dup(xi.y), xz = f2_dup(xi.z);
     const int D = S.tD;
     const float4 *nodes = a.tnode + kNodeF4 * S.tnode0;
     const int2 *leaves = a.tleaf + S.tleaf0;
     const float4 *tp = a.tpos + s0;
     const int32_t *tg = a.tagg + s0;
-    float ax = 0.f, ay = 0.f, az = 0.f;
-    bool full = false;
-    int sp = 1;
-    if (lane == 0) st[0] = ((int)(lvl_off(kSplitL) + sub) << 3) | kSplitL;   // this warp's subtree
-    __syncwarp();
-    while (sp > 0) {
-        const int cnt = min(sp, 32);
-        const int e = lane < cnt ? st[sp - 1 - lane] : -1;
-        sp -= cnt;
-        __syncwarp();
-        // test this lane's node
-        float4 A = make_float4(0.f, 0.f, 0.f, 0.f), B = A, C = A;
+    f2_t ax = f2_dup(0.f), ay = ax, az = ax;
+    int sp = 0;
+    // first round: this warp's cells of level kSplitL
+    int n = lane * kTreeParts < 64 ? (int)lvl_off(kSplitL) + sub + lane * kTreeParts : -1, L = kSplitL;
+    for (;;) {
+        // test this lane's cell
+        float4 A = make_float4(0.f, 0.f, 0.f, 0.f), B = A;
         bool acc = false, leaf = false, open = false;
         int2 lf = make_int2(0, 0);
-        if (e >= 0) {
-            const int n = e >> 3, L = e & 7;
+        if (n >= 0) {
             A = nodes[kNodeF4 * n];
+            B = nodes[kNodeF4 * n + 1];   // opening radius^2, T2
             if (A.w != 0.f) {
-                B = nodes[kNodeF4 * n + 1];   // opening radius^2, T2
                 const float gx = fmaxf(fmaxf(bx0 - A.x, A.x - bx1), 0.f);
                 const float gy = fmaxf(fmaxf(by0 - A.y, A.y - by1), 0.f);
                 const float gz = fmaxf(fmaxf(bz0 - A.z, A.z - bz1), 0.f);
                 acc = gx * gx + gy * gy + gz * gz > B.x;
                 leaf = !acc && L == D;
                 open = !acc && L < D;
-                if (acc) C = nodes[kNodeF4 * n + 2];
                 if (leaf) lf = leaves[n - lvl_off(D)];
             }
         }
-        // push the children of opened cells (compacted); a full stack
-        // turns the cell into an accepted one
+        // opened cells go on the stack
         const unsigned om = __ballot_sync(FULL, open);
-        const int need = 8 * __popc(om);
-        if (sp + need > kTreeStack) {
-            if (open) {
-                acc = true;
-                open = false;
-                C = nodes[kNodeF4 * (e >> 3) + 2];
-            }
-            full = true;
-        } else if (open) {
-            const int n = e >> 3, L = e & 7;
-            const int c0 = (int)(lvl_off(L + 1) + 8 * (n - lvl_off(L)));
-            const int at = sp + 8 * __popc(om & below);
-            for (int c = 0; c < 8; ++c) st[at + c] = ((c0 + 7 - c) << 3) | (L + 1);
-        }
-        if (sp + need <= kTreeStack) sp += need;
-        __syncwarp();
-        // accepted cells: every lane adds each of them (rank 2: the cell's 3
-        // float4 passed by shuffles; higher ranks: its 9 float4 staged in
-        // shared memory by the lane that accepted it)
-        unsigned am = __ballot_sync(FULL, acc);
-        if (ORDER > 2) {
+        if (open) st[sp + __popc(om & below)] = (n << 3) | L;
+        sp += __popc(om);
+        // accepted cells: staged in pairs (a last odd one with a massless cell
+        // far away), then every lane adds each pair
+        const unsigned am = __ballot_sync(FULL, acc);
+        const int na = __popc(am);
+        if (acc || (lane == 0 && (na & 1))) {
             if (acc) {
-                const float4 *nd = nodes + kNodeF4 * (e >> 3);
-                stage[kNodeF4 * lane] = A;
-                stage[kNodeF4 * lane + 1] = B;
-                stage[kNodeF4 * lane + 2] = C;
+                const int s = __popc(am & below);
+                float *c = (float *)(cells + (s >> 1) * kPairF2) + (s & 1);
+                const float4 *nd = nodes + kNodeF4 * n;
+                float v[36] = {A.x, A.y, A.z, A.w, B.x, B.y, B.z, B.w};
 #pragma unroll
-                for (int q = 3; q < kNodeF4; ++q) stage[kNodeF4 * lane + q] = nd[q];
-            }
-            __syncwarp();
-        }
-        while (am) {
-            const int b = __ffs(am) - 1;
-            am &= am - 1;
-            if (ORDER > 2) {
-                float nd[4 * kNodeF4];
-#pragma unroll
-                for (int q = 0; q < kNodeF4; ++q) {
-                    const float4 v = stage[kNodeF4 * b + q];
-                    nd[4 * q] = v.x; nd[4 * q + 1] = v.y; nd[4 * q + 2] = v.z; nd[4 * q + 3] = v.w;
+                for (int q = 2; q < (kNC + 3) / 4; ++q) {
+                    const float4 t = nd[q];
+                    v[4 * q] = t.x; v[4 * q + 1] = t.y; v[4 * q + 2] = t.z; v[4 * q + 3] = t.w;
                 }
-                if (mine) node_force<ORDER>(nd, xi, ax, ay, az);
-            } else {
-                float nd[12];
-                nd[0] = __shfl_sync(FULL, A.x, b); nd[1] = __shfl_sync(FULL, A.y, b);
-                nd[2] = __shfl_sync(FULL, A.z, b); nd[3] = __shfl_sync(FULL, A.w, b);
-                nd[4] = 0.f;
-                nd[5] = __shfl_sync(FULL, B.y, b); nd[6] = __shfl_sync(FULL, B.z, b);
-                nd[7] = __shfl_sync(FULL, B.w, b); nd[8] = __shfl_sync(FULL, C.x, b);
-                nd[9] = __shfl_sync(FULL, C.y, b); nd[10] = __shfl_sync(FULL, C.z, b);
-                nd[11] = 0.f;
-                if (mine) node_force<2>(nd, xi, ax, ay, az);
+#pragma unroll
+                for (int q = 0; q < kNC; ++q) c[2 * q] = v[q];
+            }
+            if (lane == 0 && (na & 1)) {
+                float *c = (float *)(cells + (na >> 1) * kPairF2) + 1;
+                for (int q = 0; q < kNC; ++q) c[2 * q] = q < 3 ? 1.0e18f : 0.f;
             }
         }
-        if (ORDER > 2) __syncwarp();
+        __syncwarp();
+        for (int p2 = 0; 2 * p2 < na; ++p2) node_force2<ORDER>(cells + p2 * kPairF2, xx, xy, xz, ax, ay, az);
+        __syncwarp();
         // opened leaves: the spheres of all of them (leaves in lane order,
-        // spheres in leaf order) are staged in shared memory kStage at a
-        // time, one round of loads for the whole round's leaves, then every
-        // lane adds each of them.  A sphere's own aggregate is skipped, and
-        // with it the sphere itself.
+        // spheres in leaf order) are staged in pairs, kLeafStage at a time, one
+        // round of loads for the whole round's leaves, then every lane adds
+        // each pair.  A sphere's own aggregate is skipped, and with it the
+        // sphere itself.
         const int lcnt = leaf ? lf.y : 0;
-        int incl = lcnt;
-        for (int o = 1; o < 32; o <<= 1) {
-            const int v = __shfl_up_sync(FULL, incl, o);
-            if (lane >= o) incl += v;
-        }
-        const int total = __shfl_sync(FULL, incl, 31);
-        if (total > 0) {
+        if (__ballot_sync(FULL, lcnt > 0)) {
+            int incl = lcnt;
+            for (int o = 1; o < 32; o <<= 1) {
+                const int v = __shfl_up_sync(FULL, incl, o);
+                if (lane >= o) incl += v;
+            }
+            const int total = __shfl_sync(FULL, incl, 31);
             lbase[lane] = incl - lcnt;   // first staged position of this lane's leaf
-            lfirst[lane] = lf.x;        // first sphere of the leaf (leaf order)
+            lfirst[lane] = lf.x;         // first sphere of the leaf (leaf order)
             __syncwarp();
-            for (int c0 = 0; c0 < total; c0 += kStage) {
-                const int nb = min(kStage, total - c0);
-                for (int t = lane; t < nb; t += 32) {
-                    // the leaf holding staged position c0 + t: the last lane whose
-                    // first staged position is not after it
-                    const int g = c0 + t;
-                    int lo2 = 0, hi2 = 31;
-                    while (lo2 < hi2) {
-                        const int mid = (lo2 + hi2 + 1) >> 1;
-                        if (lbase[mid] <= g) lo2 = mid; else hi2 = mid - 1;
+            for (int c0 = 0; c0 < total; c0 += kLeafStage) {
+                const int nb = min(kLeafStage, total - c0);
+                for (int t = lane; t < ((nb + 1) & ~1); t += 32) {
+                    float4 v = make_float4(1.0e18f, 1.0e18f, 1.0e18f, 0.f);
+                    int g = -1;
+                    if (t < nb) {
+                        // the leaf holding staged position c0 + t: the last lane
+                        // whose first staged position is not after it
+                        int lo2 = 0, hi2 = 31;
+                        while (lo2 < hi2) {
+                            const int mid = (lo2 + hi2 + 1) >> 1;
+                            if (lbase[mid] <= c0 + t) lo2 = mid; else hi2 = mid - 1;
+                        }
+                        const int idx = lfirst[lo2] + (c0 + t - lbase[lo2]);
+                        v = tp[idx];
+                        g = tg[idx];
                     }
-                    const int idx = lfirst[lo2] + (g - lbase[lo2]);
-                    stage[t] = tp[idx];
-                    sagg[t] = tg[idx];
+                    float *q = (float *)(lxy + (t >> 1)) + (t & 1), *r = (float *)(lzm + (t >> 1)) + (t & 1);
+                    q[0] = v.x; q[2] = v.y; r[0] = v.z; r[2] = v.w;
+                    ((int *)(lag + (t >> 1)))[t & 1] = g;
                 }
                 __syncwarp();
-                for (int u = 0; u < nb; ++u) {
-                    const float4 xj = stage[u];
-                    if (mine && sagg[u] != ai) {
-                        const float ex = xj.x - xi.x, ey = xj.y - xi.y, ez = xj.z - xi.z;
-                        const float q2 = fmaf(ez, ez, fmaf(ey, ey, fmaf(ex, ex, eps2)));
-                        const float iv = rsqrtf(q2);
-                        const float sj = xj.w * iv * iv * iv;
-                        ax = fmaf(ex, sj, ax);
-                        ay = fmaf(ey, sj, ay);
-                        az = fmaf(ez, sj, az);
-                    }
+#pragma unroll 2
+                for (int u = 0; 2 * u < nb; ++u) {
+                    const ulonglong2 ja = lxy[u], jb = lzm[u];
+                    const int2 g = lag[u];
+                    const f2_t ex = f2_sub(ja.x, xx), ey = f2_sub(ja.y, xy), ez = f2_sub(jb.x, xz);
+                    float ra, rb, sa, sb;
+                    f2_unpack(f2_fma(ez, ez, f2_fma(ey, ey, f2_fma(ex, ex, e2))), ra, rb);
+                    const f2_t iv = f2_pack(rsqrtf(ra), rsqrtf(rb));
+                    f2_unpack(f2_mul(f2_mul(jb.y, iv), f2_mul(iv, iv)), sa, sb);
+                    const f2_t sj = f2_pack(g.x == ai ? 0.f : sa, g.y == ai ? 0.f : sb);
+                    ax = f2_fma(ex, sj, ax);
+                    ay = f2_fma(ey, sj, ay);
+                    az = f2_fma(ez, sj, az);
                 }
                 __syncwarp();
             }
         }
+        // next round: the children of up to 4 opened cells
+        if (sp == 0) break;
+        const int cnt = min(sp, 4);
+        n = -1;
+        if ((lane >> 3) < cnt) {
+            const int e = st[sp - 1 - (lane >> 3)];
+            L = (e & 7) + 1;
+            n = (int)(lvl_off(L) + 8 * ((e >> 3) - lvl_off(L - 1))) + (lane & 7);
+        }
+        sp -= cnt;
+        __syncwarp();
     }
-    if (mine) a.tpart[(int64_t)sub * z.N + k] = make_float4(ax, ay, az, 0.f);
-    if (full && lane == 0) atomicOr(&a.pd[pp].flags, DEM_FLAG_TREE);
+    float x0, x1, y0, y1, z0, z1;
+    f2_unpack(ax, x0, x1);
+    f2_unpack(ay, y0, y1);
+    f2_unpack(az, z0, z1);
+    if (mine) a.tpart[(int64_t)sub * z.N + k] = make_float4(x0 + x1, y0 + y1, z0 + z1, 0.f);
 }
 
 // Sum the subtree partials of each sphere (float-float, fixed order).
@@ -727,7 +788,8 @@ __global__ void k_tree_combine(Arrays a, Sizes z)
     if (!tree_pile(a, p)) return;
     const PileStatic &S = a.ps[p];
     FFSum sx, sy, sz;
-    for (int s = 0; s < kSplit; ++s) {
+#pragma unroll 8
+    for (int s = 0; s < kTreeParts; ++s) {
         const float4 v = a.tpart[(int64_t)s * z.N + k];
         sx.add(v.x); sy.add(v.y); sz.add(v.z);
     }
@@ -740,18 +802,22 @@ void launch_tree_gravity(const Arrays &a, const Sizes &z, int max_depth, int ord
 {
     if (z.N == 0 || z.TN == 0) return;
     const unsigned nb = (unsigned)((z.N + 255) / 256);
-    launch_pdl(k_tree_init, (unsigned)z.P, 256, 0, st, a, z);
-    launch_pdl(k_tree_box, nb, 256, 0, st, a, z);
+    const int64_t ni = z.TL > 6 * z.P ? z.TL : 6 * z.P;
+    launch_pdl(k_tree_init, (unsigned)((ni + 255) / 256), 256, 0, st, a, z);
+    launch_pdl(k_tree_box, (unsigned)((z.N + kBoxThreads - 1) / kBoxThreads), kBoxThreads, 0, st, a, z);
     launch_pdl(k_tree_keys, nb, 256, 0, st, a, z);
-    launch_pdl(k_tree_scan, (unsigned)z.P, 1024, 0, st, a, z);
+    const int64_t nl = (int64_t)1 << (3 * max_depth);
+    const dim3 tiles((unsigned)z.P, (unsigned)((nl + kLeafTile - 1) / kLeafTile));
+    if (tiles.y > 1) launch_pdl(k_tree_sums, tiles, kScanThreads, 0, st, a, z);
+    launch_pdl(k_tree_scan, tiles, kScanThreads, 0, st, a, z);
     launch_pdl(k_tree_scatter, nb, 256, 0, st, a, z);
-    launch_pdl(k_tree_leaf_order, nb, 256, 0, st, a, z);
     launch_pdl(k_tree_gather, nb, 256, 0, st, a, z);
     launch_pdl(k_tree_leaves, (unsigned)((z.TL + 127) / 128), 128, 0, st, a, z);
-    for (int L = max_depth - 1; L >= 0; --L)
-        launch_pdl(k_tree_up, (unsigned)((z.TN + 255) / 256), 256, 0, st, a, z, L);
-    if (order == 2) launch_pdl(k_tree_force<2>, dim3((unsigned)z.TG, kSplit), 32, 0, st, a, z);
-    else launch_pdl(k_tree_force<4>, dim3((unsigned)z.TG, kSplit), 32, 0, st, a, z);
+    for (int L = max_depth - 1; L >= kSplitL; --L)
+        launch_pdl(k_tree_up, dim3((unsigned)z.P, (unsigned)((((int64_t)8 << (3 * L)) + 127) / 128)), 128, 0,
+                   st, a, z, L);
+    if (order == 2) launch_pdl(k_tree_force<2>, dim3((unsigned)z.TG, kTreeParts), 32, 0, st, a, z);
+    else launch_pdl(k_tree_force<4>, dim3((unsigned)z.TG, kTreeParts), 32, 0, st, a, z);
     launch_pdl(k_tree_combine, nb, 256, 0, st, a, z);
 }
 

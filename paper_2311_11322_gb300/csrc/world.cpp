@@ -273,7 +273,7 @@ void build_fields(dem_world *w)
     add((void **)&a.tsorted, C_TSPH, 4, false);
     add((void **)&a.tpos, C_TSPH, 16, false);
     add((void **)&a.tagg, C_TSPH, 4, false);
-    add((void **)&a.tpart, C_TSPH, 64 * 16, false);
+    add((void **)&a.tpart, C_TSPH, kTreeParts * 16, false);
     add((void **)&a.tbox, C_PILE, 32, false);
     add((void **)&a.tnode, C_TNODE, 144, false);
     add((void **)&a.traw, C_TNODE, 128, false);

@@ -178,3 +178,36 @@ def test_pile_reductions_over_blocks_and_chunks(dem, n_agg, precision):
     d = P - com
     ref = (p.G * p.ext_mass * m / (d * d).sum(1) ** 1.5)[:, None] * d
     assert np.all(np.linalg.norm(fe - ref, axis=1) <= 1e-13 * np.linalg.norm(ref, axis=1) + 1e-300)
+
+
+# tree depths 2 .. 5: leaf counts below, at and above one scan block; groups with a remainder
+@pytest.mark.parametrize("order", [2, 4])
+@pytest.mark.parametrize("n", [1, 2, 33, 300, 1025, 2049, 8300, 17001])
+def test_tree_gravity_small_angle_is_the_direct_sum(dem, n, order):
+    """With a small opening angle the accepted cells' expansions are exact to far below the mixed tolerance (their
+    relative error is about theta^(order + 1)), so the tree, its leaves and its moments must give the direct sum."""
+    ic, p = pile(n, W.PRECISION_MIXED, seed=11)
+    with dem.World() as w:
+        w.set_tuning("grav_theta", 0.05 if order == 4 else 0.01)
+        w.set_tuning("grav_order", order)
+        pid = w.add_pile(ic, p)
+        w.step(1)
+        got, pos = w.read(pid, "SPHERE_FG"), w.read(pid, "SPHERE_POS")
+    s = sampled(n)
+    F, mag = reference(ic, p, pos, s)
+    err = np.linalg.norm(got[s] - F, axis=1)
+    assert np.all(err <= 1e-5 * mag), float((err / np.maximum(mag, 1e-300)).max())
+
+
+def test_tree_piles_of_different_depths_alone_and_in_a_batch_bitwise(dem):
+    piles = [pile(n, W.PRECISION_MIXED, seed=13) for n in (3, 270, 2100, 9000, 40)]
+
+    def run(sel):
+        with dem.World() as w:
+            w.set_tuning("grav_theta", 0.6)
+            ids = [w.add_pile(*piles[k]) for k in sel]
+            w.step(2)
+            return [w.read(pid, "SPHERE_FG") for pid in ids]
+    alone = [run([k])[0] for k in range(len(piles))]
+    for got, ref in zip(run(range(len(piles))), alone):
+        assert np.array_equal(got, ref)
