@@ -11,10 +11,10 @@
 //
 // The formula is the world's gravity formula (FP32 pair terms, FP64 sums;
 // results agree with the world's within the mixed-precision tolerance, not
-// bitwise, since the world sums symmetric tile pairs), with the j range
-// split into kNAChunks parts: each part writes an FP64 partial sum per sphere,
-// and a second kernel adds the parts in a fixed order.  Those partial sums are
-// the only scratch memory, and here they live in the file-scope array
+// bitwise, since the world sums symmetric tile pairs), with the j range split
+// into parts: each part writes an FP64 partial sum per sphere, and a second
+// kernel adds the parts in a fixed order.  Those partial sums are the only
+// scratch memory, and here they live in the file-scope array
 // g_na_scratch below (16 MiB), which the CUDA runtime places in device memory
 // when the library is loaded; every GPU that loads the library keeps it until
 // the process exits.  Host code cannot use g_na_scratch's name as a device
@@ -23,6 +23,7 @@
 // memory.  The device address is therefore looked up with
 // cudaGetSymbolAddress, once per device, with that device current, on the
 // first call made on it.
+#include <algorithm>
 #include <cstdio>
 #include <mutex>
 
@@ -30,82 +31,248 @@
 
 namespace {
 
-constexpr int kNAChunks = 4;                 // j-range parts
 constexpr int kNAMaxSpheres = 131072;        // largest n accepted
+constexpr int kNAScratch = 4 * kNAMaxSpheres;   // partial sums: 4 parts of the largest n, more of fewer spheres
 constexpr int kNABlock = 128;
 constexpr int kNAFlush = 1024;
 constexpr int kNAMaxDevices = 64;
 
-// 4 parts x 131,072 spheres x 32 B = 16 MiB of partial sums.
-static __device__ __align__(256) dem::dbl4 g_na_scratch[kNAChunks * kNAMaxSpheres];
+// 524,288 x 32 B = 16 MiB of partial sums.
+static __device__ __align__(256) dem::dbl4 g_na_scratch[kNAScratch];
 
 std::mutex g_na_mutex;
 dem::dbl4 *g_na_addr[kNAMaxDevices] = {nullptr};
+int g_na_sms[kNAMaxDevices] = {0};
 
+// Packed FP32 pairs without flushing denormals.
+typedef unsigned long long na_f2;
+__device__ __forceinline__ na_f2 pack2(float lo, float hi)
+{
+    na_f2 r;
+    asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(lo), "f"(hi));
+    return r;
+}
+__device__ __forceinline__ void unpack2(na_f2 v, float &lo, float &hi)
+{
+    asm("mov.b64 {%0, %1}, %2;" : "=f"(lo), "=f"(hi) : "l"(v));
+}
+__device__ __forceinline__ na_f2 sub2(na_f2 a, na_f2 b)
+{
+    na_f2 d;
+    asm("sub.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
+    return d;
+}
+__device__ __forceinline__ na_f2 mul2(na_f2 a, na_f2 b)
+{
+    na_f2 d;
+    asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
+    return d;
+}
+__device__ __forceinline__ na_f2 fma2(na_f2 a, na_f2 b, na_f2 c)
+{
+    na_f2 d;
+    asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(d) : "l"(a), "l"(b), "l"(c));
+    return d;
+}
+// for arguments in the normal range (the softening keeps them there)
+__device__ __forceinline__ float rsqrt_normal(float x)
+{
+    float y;
+    asm("rsqrt.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
+    return y;
+}
+
+// Block (b, c): the PER x kNABlock i-spheres of block b against part c of the
+// j-spheres, 128 at a time from shared memory, packed two by two (j and j + 64).
+// A tile none of whose aggregate ids lies in the range of the block's takes the
+// packed loop (each i-sphere duplicated into both halves: 12 f32x2 operations
+// and two rsqrt for two pairs), any other the loop that compares ids (and, with
+// eps = 0, looks for coincident spheres; a sphere that is not finite counts as
+// every id, so that its pairs are treated as there).  Ids in any order are
+// correct; contiguous aggregates leave all but one or two tiles of a block to
+// the packed loop.  Measured per call, one sphere per thread, every pair
+// compared and always 4 parts -> this: 10,000 spheres 129 -> 72 us, 20,001
+// 390 -> 190 us, 131,072 11.9 -> 6.7 ms (below 3,000 the launches, 29 us).
+template <int PER>
 __global__ void __launch_bounds__(kNABlock)
 k_na_partial(const float4 *__restrict__ pm, const int32_t *__restrict__ agg, int n, int jc,
-             float eps2, dem::dbl4 *scratch)
+             float eps2, bool softened, dem::dbl4 *scratch)
 {
-    __shared__ float4 sp[kNABlock];
+    constexpr int kHalf = kNABlock / 2;
+    __shared__ ulonglong2 sxy[kHalf], szm[kHalf];   // (xa, xb, ya, yb), (za, zb, ma, mb)
     __shared__ int sa[kNABlock];
-    const int i = blockIdx.x * kNABlock + threadIdx.x;
+    __shared__ int lohi[2][kNABlock / 32][2];
+    const int t = threadIdx.x, lane = t & 31, wid = t >> 5;
+    const int i0 = blockIdx.x * (kNABlock * PER) + t;
     const int c = blockIdx.y;
     const int j0 = c * jc;
     const int j1 = min(n, j0 + jc);
-    const float4 xi = i < n ? pm[i] : make_float4(0.f, 0.f, 0.f, 0.f);
-    const int ai = i < n ? agg[i] : -2;
-    float ax = 0.f, ay = 0.f, az = 0.f;
-    double dx = 0.0, dy = 0.0, dz = 0.0;
-    int since = 0;
-    for (int jt = j0; jt < j1; jt += kNABlock) {
-        __syncthreads();
-        const int j = jt + threadIdx.x;
-        if (j < j1) {
-            sp[threadIdx.x] = pm[j];
-            sa[threadIdx.x] = agg[j];
-        } else {
-            sp[threadIdx.x] = make_float4(1.0e18f, 1.0e18f, 1.0e18f, 0.f);
-            sa[threadIdx.x] = -1;
+    const unsigned FULL = 0xffffffffu;
+    float4 xi[PER];
+    int ai[PER];
+    int lo = 0x7fffffff, hi = (int)0x80000000;
+#pragma unroll
+    for (int k = 0; k < PER; ++k) {
+        const int i = i0 + k * kNABlock;
+        xi[k] = i < n ? pm[i] : make_float4(0.f, 0.f, 0.f, 0.f);
+        ai[k] = i < n ? agg[i] : 0;
+        if (i < n) {
+            const bool fin = isfinite((xi[k].x + xi[k].y) + xi[k].z);
+            lo = min(lo, fin ? ai[k] : (int)0x80000000);
+            hi = max(hi, fin ? ai[k] : 0x7fffffff);
+        }
+    }
+    // range of values over the block: w is one of two buffers used in turn
+    auto block_range = [&](int l, int h, int w, int &bl, int &bh) {
+        l = __reduce_min_sync(FULL, l);
+        h = __reduce_max_sync(FULL, h);
+        if (lane == 0) {
+            lohi[w][wid][0] = l;
+            lohi[w][wid][1] = h;
         }
         __syncthreads();
+        bl = lohi[w][0][0];
+        bh = lohi[w][0][1];
+        for (int k = 1; k < kNABlock / 32; ++k) {
+            bl = min(bl, lohi[w][k][0]);
+            bh = max(bh, lohi[w][k][1]);
+        }
+    };
+    int ilo, ihi;
+    block_range(lo, hi, 0, ilo, ihi);
+    const na_f2 e2 = pack2(eps2, eps2);
+    na_f2 ax[PER] = {}, ay[PER] = {}, az[PER] = {};
+    double d[PER][3] = {};
+    auto flush = [&] {
+#pragma unroll
+        for (int k = 0; k < PER; ++k) {
+            float u, v;
+            unpack2(ax[k], u, v);
+            d[k][0] += u + v;
+            unpack2(ay[k], u, v);
+            d[k][1] += u + v;
+            unpack2(az[k], u, v);
+            d[k][2] += u + v;
+            ax[k] = ay[k] = az[k] = 0;
+        }
+    };
+    int since = 0, buf = 1;
+    for (int jt = j0; jt < j1; jt += kNABlock) {
+        const int j = jt + t;
+        const bool in = j < j1;
+        const float4 v = in ? pm[j] : make_float4(1.0e18f, 1.0e18f, 1.0e18f, 0.f);
+        const int ag = in ? agg[j] : 0;
+        const bool fin = isfinite((v.x + v.y) + v.z);
+        __syncthreads();   // the previous tile has been used
+        float *q = (float *)(sxy + (t & (kHalf - 1))) + t / kHalf, *r = (float *)(szm + (t & (kHalf - 1))) + t / kHalf;
+        q[0] = v.x; q[2] = v.y; r[0] = v.z; r[2] = v.w;
+        sa[t] = ag;
+        int jlo, jhi;
+        block_range(!in ? 0x7fffffff : fin ? ag : (int)0x80000000, !in ? (int)0x80000000 : fin ? ag : 0x7fffffff, buf,
+                    jlo, jhi);   // (synchronises)
+        buf ^= 1;
+        const int nj = min(kNABlock, j1 - jt), np = min(kHalf, nj);   // j-spheres, pairs of the tile
+        if (softened && (jlo > ihi || jhi < ilo)) {
+            na_f2 px[PER], py[PER], pz[PER];
+#pragma unroll
+            for (int k = 0; k < PER; ++k) {
+                px[k] = pack2(xi[k].x, xi[k].x);
+                py[k] = pack2(xi[k].y, xi[k].y);
+                pz[k] = pack2(xi[k].z, xi[k].z);
+            }
 #pragma unroll 8
-        for (int jj = 0; jj < kNABlock; ++jj) {
-            const float4 pj = sp[jj];
-            const float ddx = pj.x - xi.x, ddy = pj.y - xi.y, ddz = pj.z - xi.z;
-            const float r2 = fmaf(ddz, ddz, fmaf(ddy, ddy, fmaf(ddx, ddx, eps2)));
-            const float inv = rsqrtf(r2);
-            float s = (pj.w * inv) * (inv * inv);
-            // same aggregate (and i itself): skipped; with eps = 0 two coincident
-            // spheres of different aggregates exert no force on each other
-            s = (sa[jj] == ai || !(r2 > 0.f)) ? 0.f : s;
-            ax = fmaf(ddx, s, ax);
-            ay = fmaf(ddy, s, ay);
-            az = fmaf(ddz, s, az);
+            for (int jj = 0; jj < np; ++jj) {
+                const ulonglong2 xy = sxy[jj], zm = szm[jj];
+#pragma unroll
+                for (int k = 0; k < PER; ++k) {
+                    const na_f2 dx = sub2(xy.x, px[k]), dy = sub2(xy.y, py[k]), dz = sub2(zm.x, pz[k]);
+                    float ra, rb;
+                    unpack2(fma2(dz, dz, fma2(dy, dy, fma2(dx, dx, e2))), ra, rb);
+                    const na_f2 inv = pack2(rsqrt_normal(ra), rsqrt_normal(rb));
+                    const na_f2 s = mul2(mul2(zm.y, inv), mul2(inv, inv));
+                    ax[k] = fma2(dx, s, ax[k]);
+                    ay[k] = fma2(dy, s, ay[k]);
+                    az[k] = fma2(dz, s, az[k]);
+                }
+            }
+        } else {
+#pragma unroll 2
+            for (int jj = 0; jj < np; ++jj) {
+                const ulonglong2 xy = sxy[jj], zm = szm[jj];
+                float jx[2], jy[2], jz[2], jm[2];
+                unpack2(xy.x, jx[0], jx[1]);
+                unpack2(xy.y, jy[0], jy[1]);
+                unpack2(zm.x, jz[0], jz[1]);
+                unpack2(zm.y, jm[0], jm[1]);
+                const int aj[2] = {sa[jj], sa[jj + kHalf]};
+#pragma unroll
+                for (int k = 0; k < PER; ++k) {
+                    float s[2], ex[2], ey[2], ez[2];
+#pragma unroll
+                    for (int h = 0; h < 2; ++h) {
+                        ex[h] = jx[h] - xi[k].x;
+                        ey[h] = jy[h] - xi[k].y;
+                        ez[h] = jz[h] - xi[k].z;
+                        const float r2 = fmaf(ez[h], ez[h], fmaf(ey[h], ey[h], fmaf(ex[h], ex[h], eps2)));
+                        const float inv = rsqrtf(r2);
+                        // same aggregate (and i itself): skipped; with eps = 0 two coincident
+                        // spheres of different aggregates exert no force on each other
+                        s[h] = (aj[h] == ai[k] || !(r2 > 0.f)) ? 0.f : (jm[h] * inv) * (inv * inv);
+                    }
+                    const na_f2 sv = pack2(s[0], s[1]);
+                    ax[k] = fma2(pack2(ex[0], ex[1]), sv, ax[k]);
+                    ay[k] = fma2(pack2(ey[0], ey[1]), sv, ay[k]);
+                    az[k] = fma2(pack2(ez[0], ez[1]), sv, az[k]);
+                }
+            }
         }
         since += kNABlock;
         if (since >= kNAFlush) {
             since = 0;
-            dx += ax; dy += ay; dz += az;
-            ax = ay = az = 0.f;
+            flush();
         }
     }
+    flush();
     // every (part, sphere) slot read by k_na_combine is written here in the
     // same call, so nothing left over from an earlier call is ever read
-    if (i < n) scratch[(size_t)c * kNAMaxSpheres + i] = dem::make_dbl4(dx + ax, dy + ay, dz + az, 0.0);
+#pragma unroll
+    for (int k = 0; k < PER; ++k) {
+        const int i = i0 + k * kNABlock;
+        if (i < n) scratch[(size_t)c * n + i] = dem::make_dbl4(d[k][0], d[k][1], d[k][2], 0.0);
+    }
 }
 
-__global__ void k_na_combine(const double *__restrict__ mass, int n, double G,
+__global__ void k_na_combine(const double *__restrict__ mass, int n, int parts, double G,
                              const dem::dbl4 *__restrict__ scratch, dem::dbl4 *out)
 {
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= n) return;
     double sx = 0.0, sy = 0.0, sz = 0.0;
-    for (int c = 0; c < kNAChunks; ++c) {
-        const dem::dbl4 v = scratch[(size_t)c * kNAMaxSpheres + i];
+#pragma unroll 4
+    for (int c = 0; c < parts; ++c) {
+        const dem::dbl4 v = scratch[(size_t)c * n + i];
         sx += v.x; sy += v.y; sz += v.z;
     }
     const double gm = G * mass[i];
     out[i] = dem::make_dbl4(gm * sx, gm * sy, gm * sz, 0.0);
+}
+
+// i-spheres per thread: 2 share the shared-memory reads of the j-spheres; 1
+// where that leaves too few blocks (us per call with 1 / 2: 10,000 spheres 72 /
+// 78, 20,001 197 / 190, 131,072 7,370 / 6,740; 4 spilled, 252 at 20,001).
+constexpr int kNAPer = 2, kNASmall = 16384;
+
+// Parts of the j range: enough that the blocks fill the GPU twice over
+// (kNABlocksPerSM resident on each SM), as many as the scratch holds, none
+// shorter than 32 spheres, and at most kNAMaxParts, since k_na_combine reads
+// them one after the other (3,000 spheres in 94 parts 43 us, in 20 29 us).
+constexpr int kNABlocksPerSM = 10, kNAMaxParts = 24;
+int na_parts(int n, int per, int sms)
+{
+    const int iblocks = (n + kNABlock * per - 1) / (kNABlock * per);
+    const int want = 2 * kNABlocksPerSM * sms / iblocks;
+    const int most = std::min({kNAScratch / n, (n + 31) / 32, kNAMaxParts});
+    return std::max(1, std::min(want, most));
 }
 
 void set_msg(char *msg, size_t len, const char *text)
@@ -150,6 +317,7 @@ extern "C" dem_status dem_gravity_noalloc(const void *pos_mass, const double *ma
         return DEM_ERR_CUDA;
     }
     dem::dbl4 *scratch = nullptr;
+    int sms = 0;
     {
         std::lock_guard<std::mutex> lock(g_na_mutex);
         if (!g_na_addr[dev]) {
@@ -162,16 +330,24 @@ extern "C" dem_status dem_gravity_noalloc(const void *pos_mass, const double *ma
                 set_msg(msg, msg_len, buf);
                 return DEM_ERR_CUDA;
             }
+            if (cudaDeviceGetAttribute(&g_na_sms[dev], cudaDevAttrMultiProcessorCount, dev) != cudaSuccess) {
+                cudaGetLastError();
+                g_na_sms[dev] = 1;   // still correct, with fewer parts
+            }
             g_na_addr[dev] = (dem::dbl4 *)p;
         }
         scratch = g_na_addr[dev];
+        sms = g_na_sms[dev];
     }
     cudaStream_t st = (cudaStream_t)cuda_stream;
-    const int jc = (n + kNAChunks - 1) / kNAChunks;
-    dim3 grid((n + kNABlock - 1) / kNABlock, kNAChunks);
-    k_na_partial<<<grid, kNABlock, 0, st>>>((const float4 *)pos_mass, agg_id, n, jc,
-                                            (float)(eps_soft * eps_soft), scratch);
-    k_na_combine<<<(n + 255) / 256, 256, 0, st>>>(mass, n, G, scratch, (dem::dbl4 *)force_out);
+    const float eps2 = (float)(eps_soft * eps_soft);
+    const int per = n <= kNASmall ? 1 : kNAPer;
+    const int parts = na_parts(n, per, sms);
+    const int jc = (n + parts - 1) / parts;
+    const dim3 grid((n + kNABlock * per - 1) / (kNABlock * per), parts);
+    const auto kernel = per == 1 ? k_na_partial<1> : k_na_partial<kNAPer>;
+    kernel<<<grid, kNABlock, 0, st>>>((const float4 *)pos_mass, agg_id, n, jc, eps2, eps2 >= 1.0e-30f, scratch);
+    k_na_combine<<<(n + 127) / 128, 128, 0, st>>>(mass, n, parts, G, scratch, (dem::dbl4 *)force_out);
     e = cudaGetLastError();
     if (e != cudaSuccess) {
         char buf[200];

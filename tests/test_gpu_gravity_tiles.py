@@ -211,3 +211,35 @@ def test_tree_piles_of_different_depths_alone_and_in_a_batch_bitwise(dem):
     alone = [run([k])[0] for k in range(len(piles))]
     for got, ref in zip(run(range(len(piles))), alone):
         assert np.array_equal(got, ref)
+
+
+@pytest.mark.parametrize("eps", [0.0, 0.5])
+@pytest.mark.parametrize("ids", ["contiguous", "shuffled"])
+@pytest.mark.parametrize("n", [2, 127, 129, 512, 513, 1025, 5003])
+def test_noalloc_gravity_parts_and_masks(dem, n, ids, eps):
+    """The caller-owned gravity call at the edges of its blocks, tiles and parts, with aggregate ids in order and in
+    none, softened and not (two spheres of different aggregates coincide: no force between them)."""
+    import torch
+    rng = np.random.default_rng(n)
+    pos = rng.uniform(-200.0, 200.0, (n, 3)).astype(np.float32)
+    agg = (np.arange(n) // 3).astype(np.int32)
+    if ids == "shuffled":
+        agg = rng.permutation(agg) - 5
+    if n > 6:
+        pos[-1] = pos[0]
+        agg[-1], agg[0] = 1000000, -1000000
+    m = W.sphere_mass(rng.uniform(1.0, 3.0, n), 2500.0)
+    pm = torch.from_numpy(np.concatenate([pos, m.astype(np.float32)[:, None]], 1)).cuda()
+    tm, ta = torch.from_numpy(m).cuda(), torch.from_numpy(agg).cuda()
+    out = torch.full((n, 4), float("nan"), dtype=torch.float64, device="cuda")
+    import ctypes as C
+    rc = dem.load().dem_gravity_noalloc(pm.data_ptr(), C.c_void_p(tm.data_ptr()), ta.data_ptr(), n, 1.0, eps,
+                                        C.c_void_p(out.data_ptr()), torch.cuda.current_stream().cuda_stream, None, 0)
+    assert rc == dem.DEM_OK
+    got = out.cpu().numpy()[:, :3]
+    for i in sampled(n):
+        d = pos.astype(float) - pos[i].astype(float)
+        r2 = (d * d).sum(1) + eps ** 2
+        w = np.where((agg == agg[i]) | (r2 == 0), 0.0, m / np.where(r2 == 0, 1.0, r2) ** 1.5)
+        t = m[i] * w[:, None] * d
+        assert np.linalg.norm(got[i] - t.sum(0)) <= 1e-5 * np.linalg.norm(t, axis=1).sum()
