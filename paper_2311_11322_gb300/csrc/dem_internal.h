@@ -301,6 +301,10 @@ void launch_agg_end(const Arrays &a, const Sizes &z, bool fp64, cudaStream_t st)
 void launch_fill_ids(const Arrays &a, const Sizes &z, cudaStream_t st);
 // order: highest multipole rank of accepted cells (2 or 4)
 void launch_tree_gravity(const Arrays &a, const Sizes &z, int max_depth, int order, cudaStream_t st);
+// space-frame spin R(q) w_body of aggregates [a0, a0 + na) as FP64 [na][3]
+void launch_space_spin(const Arrays &a, int64_t a0, int64_t na, bool fp64, double *out, cudaStream_t st);
+// n state slots (FP64, or float-float pairs) as FP64
+void launch_state_values(const double *src, int64_t n, bool fp64, double *out, cudaStream_t st);
 void launch_force_rebuild(const Arrays &a, const Sizes &z, int slot, cudaStream_t st);
 // programmatic dependent launch for the launches that follow on this host
 // thread: on for worlds of at most kPdlMaxSpheres spheres (launch.cuh)

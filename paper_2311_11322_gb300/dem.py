@@ -118,7 +118,8 @@ class DemError(RuntimeError):
 
 
 def _ptr(a):
-    return None if a is None else a.ctypes.data_as(C.c_void_p)
+    """Address of an array that the caller keeps alive during the call."""
+    return None if a is None else a.ctypes.data
 
 
 def make_params(p) -> dem_params:
