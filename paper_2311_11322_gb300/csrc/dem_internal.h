@@ -193,10 +193,9 @@ struct Arrays {
     dbl4 *ftc64;
     // sorted position (pile-local) of each home sphere, double-buffered by parity
     int32_t *pos_of_home[2];
-    // contact history per candidate-list entry of the pair's owner (its lower
-    // home index): S from the owner's side and 1 in .w while the pair is in
-    // contact, double-buffered by pile parity; *_rm: the previous history
-    // carried over to new lists at a rebuild
+    // contact history per candidate-list entry: S from the listing sphere's
+    // side and 1 in .w while the pair is in contact, double-buffered by pile
+    // parity; *_rm: the previous history carried over to new lists at a rebuild
     float4 *hist32[2], *hist32_rm;
     dbl4 *hist64[2], *hist64_rm;
     // aggregates

@@ -22,8 +22,7 @@
 // Two forms of the pass, with bitwise the same results:
 //   k_contact_sphere (the default): one thread per sorted sphere evaluates
 //     every entry of its list with itself as sphere a (each pair twice, once
-//     per sphere) and sums its shares in list order; the owner's thread
-//     writes the history;
+//     per sphere), sums its shares in list order and writes its own history;
 //   k_contact (contact_mode 1): tiles of kCTile consecutive sorted spheres,
 //     which fill compact blocks of space (cells are numbered brick by brick);
 //     a pair inside a tile is evaluated once, by the thread that drew it from
@@ -36,10 +35,13 @@
 // the lists were rebuilt.  Nothing is written with atomics except error flags.
 //
 // History (Sec. 2.1: the tangential displacement is tracked while the two
-// spheres stay in contact) lives at the owner's list entry, from the owner's
-// side, with .w = 1 while in contact; the evaluation reads the owner's entry
-// and the owner's tile writes it.  A rebuild carries it over to the new lists
-// by partner index.
+// spheres stay in contact) lives at each sphere's own list entry, from its own
+// side, with .w = 1 while in contact: the two sides' evaluations give exactly
+// opposite displacements, so the copies never differ but in sign, and every
+// access is to consecutive entries of a warp and known ahead.  (Kept once, at
+// the owner's entry, the partner's side read it out of order, often a second
+// time from HBM: 272 us on the 1M lattice, 201 so.)  A rebuild carries it over
+// to the new lists by partner index.
 //
 // Mixed precision positions.  The overlap x = s_a + s_b - |d| of two nearby
 // spheres needs more than FP32's 24 bits of |d|.  Each sphere's position
@@ -302,13 +304,12 @@ __device__ __forceinline__ float4 as_f4(int4 v)
 }
 
 // ---------------------------------------------------------------- step
-// One sorted sphere k: every entry of its list is evaluated in the canonical
-// orientation (owner as sphere a, the same evaluation the tiles make) and the
-// sphere keeps its own share, summed in list order; the owner's side writes
-// the pair's history.  Each pair is evaluated twice (once per sphere), with
-// bitwise the same result both times, so the forces equal the tile form's bit
-// for bit.  s_x / s_v: the sorted spheres [kb0, kb0 + 128) staged in shared
-// memory (mixed path), or null.
+// One sorted sphere k: every entry of its list is evaluated with the sphere as
+// sphere a (see the file comment); it keeps its own share, summed in list order,
+// and its own history.  Each pair is evaluated twice (once per sphere), with
+// exactly opposite results, so the forces equal the tile form's bit for bit.
+// s_x / s_v: the sorted spheres [kb0, kb0 + 128) staged in shared memory
+// (mixed path), or null.
 template <bool FP64>
 __device__ __forceinline__ void sphere_contacts(const Arrays &a, const PileStatic &S, int lp,
                                                 const typename CT<FP64>::H *hread,
@@ -343,23 +344,21 @@ __device__ __forceinline__ void sphere_contacts(const Arrays &a, const PileStati
     // onto its negative or onto itself when the spheres swap (differences and
     // products of negated operands round to the negated or the same value),
     // so this evaluation's share a is bit for bit the share of this side of
-    // the owner's evaluation; the owner's S is seen from this side with the
-    // opposite sign.  The owner's side writes the history.
-    auto entry = [&](int f, bool owned, bool ok, const H &hp, const typename CT<FP64>::P &pp,
+    // the owner's evaluation, and S the owner's with its sign.
+    auto entry = [&](int f, bool ok, const H &hp, const typename CT<FP64>::P &pp,
                      const float4 &pr, const typename CT<FP64>::VR &pv, const typename CT<FP64>::VR &pw) {
         PairOut<T, V> o;
         bool hit = false;
-        const T sgn = owned ? T(1) : T(-1);
         if (ok) {
             if constexpr (FP64) {
-                const double3 Sprev = hp.w != 0 ? d3(sgn * hp.x, sgn * hp.y, sgn * hp.z) : d3(0, 0, 0);
+                const double3 Sprev = hp.w != 0 ? d3(hp.x, hp.y, hp.z) : d3(0, 0, 0);
                 hit = pair_64(mp, mv, mw, pp, pv, pw, Sprev, prm, o);
             } else {
-                const float3 Sprev = hp.w != 0.f ? f3(sgn * hp.x, sgn * hp.y, sgn * hp.z) : f3(0.f, 0.f, 0.f);
+                const float3 Sprev = hp.w != 0.f ? f3(hp.x, hp.y, hp.z) : f3(0.f, 0.f, 0.f);
                 hit = pair_mixed(mp, mr, pp, pr, q, mv, mw, pv, pw, Sprev, prm, o);
             }
         }
-        if (owned && ok) {
+        if (ok) {
             H h;
             if constexpr (FP64) h = hit ? make_dbl4(o.S.x, o.S.y, o.S.z, 1.0) : make_dbl4(0, 0, 0, 0);
             else h = hit ? make_float4(o.S.x, o.S.y, o.S.z, 1.f) : make_float4(0.f, 0.f, 0.f, 0.f);
@@ -373,23 +372,19 @@ __device__ __forceinline__ void sphere_contacts(const Arrays &a, const PileStati
         Tq.x = addr(Tq.x, sT.x); Tq.y = addr(Tq.y, sT.y); Tq.z = addr(Tq.z, sT.z);
         ++nc;
     };
-    // an entry's partner and history indices (clamped: the checks never fail)
-    auto where = [&](int2 c, int f, int64_t &g, int &hidx, bool &ok) {
+    // an entry's partner (clamped: the check never fails)
+    auto where = [&](int2 c, int64_t &g, bool &ok) {
         const int kk = c.x & 0x7fffffff;
-        hidx = c.x < 0 ? f : c.y;
-        ok = (unsigned)kk < (unsigned)S.ns && (unsigned)hidx < (unsigned)S.ne;
+        ok = (unsigned)kk < (unsigned)S.ns;
         g = s0 + (ok ? kk : 0);
-        if (!ok) hidx = 0;
     };
     if constexpr (FP64) {
         for (int e = 0; e < n; ++e) {
             const int f = off + 32 * e;
-            const int2 c = cand[f];
             int64_t g;
-            int hidx;
             bool ok;
-            where(c, f, g, hidx, ok);
-            entry(f, c.x < 0, ok, hread[hidx], a.dp_[g], make_float4(0.f, 0.f, 0.f, 0.f), a.dv_[g], a.dw_[g]);
+            where(cand[f], g, ok);
+            entry(f, ok, hread[f], a.dp_[g], make_float4(0.f, 0.f, 0.f, 0.f), a.dv_[g], a.dw_[g]);
         }
     } else {
         // partner data from the staged block when it is there, else from global memory
@@ -401,40 +396,34 @@ __device__ __forceinline__ void sphere_contacts(const Arrays &a, const PileStati
                 x = a.xqr[2 * g]; r = a.xqr[2 * g + 1]; v = a.svw[2 * g]; w = a.svw[2 * g + 1];
             }
         };
-        // software pipeline: the list entry two ahead and the partner data and
-        // history one ahead are in flight while an entry is evaluated
-        int2 c1 = make_int2(0, 0);
-        if (n > 1) c1 = cand[off + 32];
-        int2 cc = make_int2(0, 0);
-        int4 px = make_int4(0, 0, 0, 0), pr = px;
-        float4 pv = make_float4(0.f, 0.f, 0.f, 0.f), pw = pv;
-        H hp = make_float4(0.f, 0.f, 0.f, 0.f);
-        bool ok = false;
+        // the list entry and the history two ahead are in flight while an entry
+        // is evaluated (both are consecutive for the warp, so no address waits
+        // for a load); the partner's data is fetched where it is used, which
+        // leaves room for a fifth block per SM (96 registers): 201 us on the 1M
+        // lattice, 252 with it one entry ahead and four blocks, 210 with it
+        // prefetched to L2
+        const int last = off + 32 * (n - 1);   // (n > 0 where it is used)
+        auto at = [&](int e) { return min(off + 32 * e, last); };
+        int2 c0 = make_int2(0, 0), c1 = c0;
+        H hp = make_float4(0.f, 0.f, 0.f, 0.f), h1 = hp;
         if (n > 0) {
-            cc = cand[off];
-            int64_t g;
-            int hidx;
-            where(cc, off, g, hidx, ok);
-            fetch(g, px, pr, pv, pw);
-            hp = hread[hidx];
+            c0 = cand[off];
+            c1 = cand[at(1)];
+            hp = hread[off];
+            h1 = hread[at(1)];
         }
         for (int e = 0; e < n; ++e) {
-            const int f = off + 32 * e;
-            int4 nx = px, nr = pr;
-            float4 nv = pv, nw = pw;
-            H nh = hp;
-            bool nok = false;
-            if (e + 1 < n) {
-                int64_t g;
-                int hidx;
-                where(c1, f + 32, g, hidx, nok);
-                fetch(g, nx, nr, nv, nw);
-                nh = hread[hidx];
-            }
-            const int2 c2 = e + 2 < n ? cand[f + 64] : make_int2(0, 0);
-            entry(f, cc.x < 0, ok, hp, px, as_f4(pr), pv, pw);
-            cc = c1; c1 = c2;
-            px = nx; pr = nr; pv = nv; pw = nw; hp = nh; ok = nok;
+            int64_t g;
+            bool ok;
+            int4 px, pr;
+            float4 pv, pw;
+            where(c0, g, ok);
+            fetch(g, px, pr, pv, pw);
+            const int2 c2 = cand[at(e + 2)];
+            const H h2 = hread[at(e + 2)];
+            entry(off + 32 * e, ok, hp, px, as_f4(pr), pv, pw);
+            c0 = c1; c1 = c2;
+            hp = h1; h1 = h2;
         }
     }
     // stored at the sphere's home index (its aggregate's members are then
@@ -627,9 +616,9 @@ __global__ void __launch_bounds__(kCTile, FP64 ? 2 : 4) k_contact(Arrays a, Size
             // sphere a is the owner
             const int ia = owned ? i : kk - first, ib = owned ? kk - first : i;
             const bool a_loc = owned || inner, b_loc = !owned || inner;
-            const int hidx = owned ? f : c.y;
-            if ((unsigned)kk >= (unsigned)S.ns || (unsigned)hidx >= (unsigned)S.ne) continue;   // (never taken)
-            const H hp = hread[hidx];
+            if ((unsigned)kk >= (unsigned)S.ns || (unsigned)c.y >= (unsigned)S.ne) continue;   // (never taken)
+            const H hp = hread[f];        // from this sphere's side; the evaluation takes the owner's
+            const T sgn = owned ? T(1) : T(-1);
             PairOut<T, V> o;
             bool hit;
             if constexpr (FP64) {
@@ -639,7 +628,7 @@ __global__ void __launch_bounds__(kCTile, FP64 ? 2 : 4) k_contact(Arrays a, Size
                            aw = a_loc ? st[2 * kCTile + ia] : a.dw_[ga];
                 const dbl4 bp = b_loc ? st[ib] : a.dp_[gb], bv = b_loc ? st[kCTile + ib] : a.dv_[gb],
                            bw = b_loc ? st[2 * kCTile + ib] : a.dw_[gb];
-                const double3 Sprev = hp.w != 0 ? d3(hp.x, hp.y, hp.z) : d3(0, 0, 0);
+                const double3 Sprev = hp.w != 0 ? d3(sgn * hp.x, sgn * hp.y, sgn * hp.z) : d3(0, 0, 0);
                 hit = pair_64(ap, av, aw, bp, bv, bw, Sprev, prm, o);
             } else {
                 const int4 *sx = (const int4 *)stage;
@@ -650,15 +639,19 @@ __global__ void __launch_bounds__(kCTile, FP64 ? 2 : 4) k_contact(Arrays a, Size
                 const float4 RB = b_loc ? sv[2 * kCTile + ib] : as_f4(a.xqr[2 * gb + 1]);
                 const float4 av = a_loc ? sv[ia] : a.svw[2 * ga], aw = a_loc ? sv[kCTile + ia] : a.svw[2 * ga + 1];
                 const float4 bv = b_loc ? sv[ib] : a.svw[2 * gb], bw = b_loc ? sv[kCTile + ib] : a.svw[2 * gb + 1];
-                const float3 Sprev = hp.w != 0.f ? f3(hp.x, hp.y, hp.z) : f3(0.f, 0.f, 0.f);
+                const float3 Sprev = hp.w != 0.f ? f3(sgn * hp.x, sgn * hp.y, sgn * hp.z) : f3(0.f, 0.f, 0.f);
                 hit = pair_mixed(A, RA, B, RB, q, av, aw, bv, bw, Sprev, prm, o);
             }
-            if (owned) {
+            // this sphere's entry, and the partner's of an inner pair, each
+            // from its own side
+            auto keep = [&](int at, T sg) {
                 H h;
-                if constexpr (FP64) h = hit ? make_dbl4(o.S.x, o.S.y, o.S.z, 1.0) : make_dbl4(0, 0, 0, 0);
-                else h = hit ? make_float4(o.S.x, o.S.y, o.S.z, 1.f) : make_float4(0.f, 0.f, 0.f, 0.f);
-                hwrite[f] = h;
-            }
+                if constexpr (FP64) h = hit ? make_dbl4(sg * o.S.x, sg * o.S.y, sg * o.S.z, 1.0) : make_dbl4(0, 0, 0, 0);
+                else h = hit ? make_float4(sg * o.S.x, sg * o.S.y, sg * o.S.z, 1.f) : make_float4(0.f, 0.f, 0.f, 0.f);
+                hwrite[at] = h;
+            };
+            keep(f, sgn);
+            if (inner) keep(c.y, -sgn);
             if (hit && o.x > T(0.1) * o.rmin) myflags |= DEM_FLAG_OVERLAP;
             V F, Tq;
             if (a_loc) {
@@ -729,7 +722,7 @@ __global__ void __launch_bounds__(kCTile, FP64 ? 2 : 4) k_contact(Arrays a, Size
 // spheres are staged in shared memory in the mixed path (consecutive sorted
 // spheres fill a compact block of space, so most partners are among them).
 template <bool FP64>
-__global__ void __launch_bounds__(128) k_contact_sphere(Arrays a, Sizes z)
+__global__ void __launch_bounds__(128, FP64 ? 1 : 5) k_contact_sphere(Arrays a, Sizes z)
 {
     pdl_enter();
     typedef typename CT<FP64>::H H;

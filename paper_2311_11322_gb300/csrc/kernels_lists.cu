@@ -328,8 +328,8 @@ __device__ __forceinline__ void gather_sphere(const Arrays &a, int64_t k)
         a.dw_[k] = make_dbl4(w.x, w.y, w.z, (double)hl);
         if (grav) a.gpos64[i] = make_dbl4(pos.x, pos.y, pos.z, a.m64[i]);
     } else {
-        const AggRecMixed &rec = a.rec32[g];
         float4 bh = a.bh[i], bl = a.bl[i];
+        const AggRecMixed rec = load_rec(a.rec32, g);
         ff px, py, pz;
         expand_mixed(rec, bh, bl, px, py, pz);
         float3 rb = f3(rec.Rh[0] * bh.x + rec.Rh[1] * bh.y + rec.Rh[2] * bh.z,
@@ -650,7 +650,6 @@ __device__ __forceinline__ void cand_link_sphere(const Arrays &a, int p, int kl)
         if (mir < 0) atomicOr(&a.pd[p].flags, DEM_FLAG_SLOTS);   // lists not symmetric: cannot happen
         const bool owned = me < id;
         a.cand[lp][e0 + f] = make_int2(kk | (owned ? (int)0x80000000u : 0), mir < 0 ? 0 : mir);
-        if (!owned) continue;
         // carried history: the same partner in the previous list (both lists
         // are in partner order, so one forward cursor finds it)
         H h;
@@ -683,8 +682,10 @@ __host__ __device__ __forceinline__ int64_t lists_reducers(const Sizes &z)
     return z.CH < most ? z.CH : most;
 }
 
+// (7 blocks an SM: 72 registers; left alone the compiler takes 64 and spills,
+// 59 us for the gather of the 1M lattice, 51 so)
 template <bool FP64>
-__global__ void __launch_bounds__(kLB) k_lists(Arrays a, Sizes z)
+__global__ void __launch_bounds__(kLB, 7) k_lists(Arrays a, Sizes z)
 {
     pdl_enter();
     __shared__ int2 s_list[kFillCap][kLB];   // (partner home index, sorted position)

@@ -1862,7 +1862,7 @@ dem_status dem_write_state(dem_world *w, int32_t pile_id, int32_t field, const d
     case DEM_FIELD_CONTACTS: {
         // written as the pile's current candidate lists (one entry per
         // contact, both spheres of a pair listing each other, partner order)
-        // with the history at the owner entries; the next step rebuilds the
+        // with the history from each one's side; the next step rebuilds the
         // lists and carries S over by partner index
         const int K = w->K;
         const int64_t row = 1 + 4 * (int64_t)K;
@@ -1928,10 +1928,11 @@ dem_status dem_write_state(dem_world *w, int32_t pile_id, int32_t field, const d
                 ids[f] = J;
                 const bool owned = i < J;
                 cd[f] = make_int2(pos[J] | (owned ? (int)0x80000000u : 0), (int)mir);
-                if (owned) {
-                    const double *sl = in + (int64_t)i * row + 1 + 4 * rows[i][e].second;
-                    hs[4 * f] = sl[1]; hs[4 * f + 1] = sl[2]; hs[4 * f + 2] = sl[3]; hs[4 * f + 3] = 1.0;
-                }
+                // S as the lower-index sphere's row gives it, from this sphere's side
+                const double *sl = in + (int64_t)(owned ? i : J) * row + 1 + 4 * (owned ? rows[i][e].second : it->second);
+                const double sg = owned ? 1.0 : -1.0;
+                for (int c = 0; c < 3; ++c) hs[4 * f + c] = sg * sl[1 + c];
+                hs[4 * f + 3] = 1.0;
             }
         }
         CHK(put(D.ccnt[cp] + s0, cnt.data(), 4 * N));
