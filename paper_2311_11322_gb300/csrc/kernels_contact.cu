@@ -744,7 +744,7 @@ __global__ void __launch_bounds__(128, FP64 ? 1 : 5) k_contact_sphere(Arrays a, 
         __syncthreads();
     }
     if (k >= z.N) return;
-    const int p = a.sph_pile[k];
+    const int p = sphere_pile(a, z, k);
     if (!pile_active(a, p)) return;
     const PileStatic &S = a.ps[p];
     const PileDyn &D = a.pd[p];

@@ -147,7 +147,7 @@ template <typename Fn>
 __device__ __forceinline__ void rebuilding_spheres(const Arrays &a, const Sizes &z, Fn f)
 {
     for (int64_t i = (int64_t)blockIdx.x * kLB + threadIdx.x; i < z.N; i += (int64_t)gridDim.x * kLB) {
-        const int p = a.sph_pile[i];
+        const int p = sphere_pile(a, z, i);
         if (pile_rebuilds(a, p)) f(i, p);
     }
 }
@@ -297,9 +297,8 @@ __device__ __forceinline__ void order_cell(const Arrays &a, int64_t k, int p)
 // pred-vel), spin, ids; and the gravity input (position relative to the pile
 // frame, mass) at the sphere's home index.
 template <bool FP64>
-__device__ __forceinline__ void gather_sphere(const Arrays &a, int64_t k)
+__device__ __forceinline__ void gather_sphere(const Arrays &a, int64_t k, int p)
 {
-    const int p = a.sph_pile[k];
     if (!pile_active(a, p)) return;
     const PileStatic &S = a.ps[p];
     const int hl = a.sorted[k];
@@ -716,7 +715,8 @@ __global__ void __launch_bounds__(kLB, 7) k_lists(Arrays a, Sizes z)
         if (b < 0)
             for (int64_t ch = blockIdx.x; ch < z.CH; ch += nred) open_chunk<FP64, kLB>(a, ch);
         else
-            for (int64_t k = b * kLB + threadIdx.x; k < z.N; k += (gridDim.x - nred) * kLB) gather_sphere<FP64>(a, k);
+            for (int64_t k = b * kLB + threadIdx.x; k < z.N; k += (gridDim.x - nred) * kLB)
+                gather_sphere<FP64>(a, k, sphere_pile(a, z, k));
     }
     if (!rb) return;
     ok = ok && grid_barrier(a, 7);

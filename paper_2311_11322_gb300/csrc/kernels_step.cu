@@ -339,7 +339,7 @@ __global__ void __launch_bounds__(kAggThreads) k_agg_begin(Arrays a, Sizes z)
     pdl_enter();
     int64_t g = (int64_t)blockIdx.x * kAggThreads + threadIdx.x;
     if (g >= z.A) return;
-    int p = a.agg_pile[g];
+    int p = aggregate_pile(a, z, g);
     if (!pile_active(a, p)) return;
     if constexpr (FP64) agg_begin_64<ADAPT>(a, g, p);
     else agg_begin_mixed<ADAPT>(a, g, p);
@@ -621,7 +621,7 @@ __global__ void __launch_bounds__(kAggThreads) k_agg_end(Arrays a, Sizes z)
     pdl_enter();
     constexpr int kCtas = kAggChunk / kAggThreads;
     const int64_t ch = blockIdx.x / kCtas;
-    const int p = a.chunk_pile[ch];
+    const int p = z.P == 1 ? 0 : a.chunk_pile[ch];
     int64_t beg, end;
     chunk_range(a, ch, p, beg, end);
     beg += (int64_t)(blockIdx.x % kCtas) * kAggThreads;

@@ -24,11 +24,11 @@
 
 namespace dem {
 
-// Whether launch_pdl sets the attribute, chosen by the world before it
-// captures its step (per host thread: a world is used by one thread at a
-// time).  Measured per step with and without: 1,000 spheres 82 -> 76 us, but
-// 2e4 spheres 224 -> 231 us and 1e5 spheres 2.872 -> 2.891 ms, so worlds
-// above 8,192 spheres launch plainly.
+// Whether launch_pdl and launch_coop set the attribute, chosen by the world
+// before it captures its step (per host thread: a world is used by one thread
+// at a time).  Measured per step of 19 kernels without and with: 1,000 spheres
+// 82 -> 76 us, but 2e4 spheres 224 -> 231 us and 1e5 spheres 2.872 -> 2.891
+// ms, so worlds above 8,192 spheres launch plainly.
 inline thread_local bool tl_pdl = true;
 constexpr int64_t kPdlMaxSpheres = 8192;
 
@@ -58,8 +58,10 @@ inline void launch_pdl(void (*kernel)(KArgs...), dim3 grid, dim3 block, size_t s
 }
 
 // The same as a cooperative launch (all blocks resident at once, so that they
-// may wait for one another; the grid must fit the device), without the
-// programmatic attribute.
+// may wait for one another; the grid must fit the device).  The blocks wait
+// for one another only after pdl_enter(), and the next kernel's blocks are not
+// launched before every one of them has passed it, so the programmatic
+// attribute goes with it (1,000 spheres 33.3 -> 31.2 us per step).
 template <typename... KArgs, typename... Args>
 inline void launch_coop(void (*kernel)(KArgs...), dim3 grid, dim3 block, size_t smem, cudaStream_t st,
                         Args &&...args)
@@ -69,11 +71,13 @@ inline void launch_coop(void (*kernel)(KArgs...), dim3 grid, dim3 block, size_t 
     cfg.blockDim = block;
     cfg.dynamicSmemBytes = smem;
     cfg.stream = st;
-    cudaLaunchAttribute at[1];
+    cudaLaunchAttribute at[2];
     at[0].id = cudaLaunchAttributeCooperative;
     at[0].val.cooperative = 1;
+    at[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at[1].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = at;
-    cfg.numAttrs = 1;
+    cfg.numAttrs = (DEM_PDL && tl_pdl) ? 2 : 1;
     cudaLaunchKernelEx(&cfg, kernel, std::forward<Args>(args)...);
 }
 

@@ -28,6 +28,18 @@ __device__ __forceinline__ bool pile_active(const Arrays &a, int p)
     return a.enabled[p] != 0 && a.pd[p].failed == 0;
 }
 
+// Pile of sphere or aggregate i: in a world of one pile no load that all
+// others wait for (1,048,576 spheres: k_lists 51.1 -> 47.1 us, contact pass
+// 200.7 -> 196.6 us, step 334 -> 327.6 us).
+__device__ __forceinline__ int sphere_pile(const Arrays &a, const Sizes &z, int64_t i)
+{
+    return z.P == 1 ? 0 : a.sph_pile[i];
+}
+__device__ __forceinline__ int aggregate_pile(const Arrays &a, const Sizes &z, int64_t g)
+{
+    return z.P == 1 ? 0 : a.agg_pile[g];
+}
+
 constexpr int kSumThreads = 128;   // virtual threads of a sum
 static_assert(kAggChunk % kSumThreads == 0, "whole rounds per chunk");
 
