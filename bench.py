@@ -242,7 +242,7 @@ def run_contact_roofline(dem, W, peak_gbs, steps=5, n=1_048_576, warmup=3, mode=
         # the other kernels of the same steps, each between event nodes in the graph
         others = {}
         step_ms = []
-        for kname in ("AGG_BEGIN", "PILE_BEGIN", "KEYS", "GATHER", "AGG_END", "PILE_END"):
+        for kname in ("AGG_BEGIN", "GATHER", "AGG_END"):
             w.set_timed_kernel(kname)
             km = []
             for _ in range(steps):
@@ -252,24 +252,28 @@ def run_contact_roofline(dem, W, peak_gbs, steps=5, n=1_048_576, warmup=3, mode=
                 km.append(k_)
                 step_ms.append(sm_)
             others[kname] = statistics.median(km) * 1e3
-        w.set_timed_kernel("CONTACT")
         cnt = w.read(pid, "CONTACTS")[:, 0]
-        # rebuild steps: a state write (the same velocities) forces one
+        # rebuild steps: a state write (the same velocities) forces one; the lists
+        # are built in the gather's kernel, so both kernels count
         vel = w.read(pid, "VEL")
-        rb = []
-        for _ in range(3):
-            w.write(pid, "VEL", vel)
-            with torch.cuda.stream(st):
-                flush.zero_()
-            rb.append(w.step_timed()[1])
+        rb = {}
+        for kname in ("GATHER", "CONTACT"):
+            w.set_timed_kernel(kname)
+            km = []
+            for _ in range(3):
+                w.write(pid, "VEL", vel)
+                with torch.cuda.stream(st):
+                    flush.zero_()
+                km.append(w.step_timed()[1])
+            rb[kname] = statistics.median(km)
     z = float(cnt.sum())
     N = ic.n_sph
     # this library's own compulsory bytes per step: own sorted records (fixed-
     # point position with its rounding remainders 32 B, velocity and spin 32 B),
-    # list offset and length (8 B), F and tau out (32 B); per list entry the
-    # entry (partner, mirror: 8 B); per pair its history record read and written
-    # (16 B each)
-    layout = N * (64 + 8 + 32) + z * 8 + (z / 2) * 32
+    # list offset and length (8 B), F and tau out (32 B); per list entry (each
+    # pair has one at either sphere) the entry (partner, mirror: 8 B) and its
+    # history record read and written (16 B each)
+    layout = N * (64 + 8 + 32) + z * (8 + 32)
     algo = N * CONTACT_BYTES_PER_SPHERE + (z / 2) * CONTACT_BYTES_PER_PAIR
     ms = statistics.median(ks)
     achieved = algo / (ms / 1e3) / 1e9
@@ -279,23 +283,23 @@ def run_contact_roofline(dem, W, peak_gbs, steps=5, n=1_048_576, warmup=3, mode=
             "kernel": ("k_contact_sphere (one thread per sphere over its kept candidate list)" if mode_used == 0
                        else "k_contact (128-sphere tiles, each inner pair once, shared-memory inbox)"),
             "kernel_ms": ms, "rebuilds_in_timed_steps": info["rebuilds"] - r0,
-            "rebuild_step_contact_ms": statistics.median(rb),
+            "rebuild_step_contact_ms": rb["GATHER"] + rb["CONTACT"],
             "n_spheres": N, "contacts_per_sphere": z / N,
             "algorithmic_bytes_per_launch": algo,
             "algorithmic_bytes": "84 B per sphere (position, velocity, spin 16 B each, cell range 4 B "
                                  "read; F, tau 32 B written) + 32 B per contact pair (16-byte history "
                                  "record read and written)",
             "layout_bytes_per_launch": layout, "frac_on_layout_bytes": layout / (ms / 1e3) / 1e9 / peak_gbs,
-            "layout_bytes": "this library's own layout: 104 B per sphere + 8 B per list entry + 32 B per "
-                            "contact pair",
+            "layout_bytes": "this library's own layout: 104 B per sphere + 40 B per list entry (8 B entry, "
+                            "16-byte history record read and written at either side)",
             "other_kernels_us": others, "step_ms": statistics.median(step_ms),
             "other_kernels": "CUDA events around each kernel inside the step graph, median over the steps "
-                             "(the rebuild-only kernels return at once in these steps)",
+                             "(GATHER is k_lists, which in these steps rebuilds nothing)",
             "workload": "dense FCC tetrahedra lattice, %d spheres, overlaps 0.5%% R, gravity off" % N}
 
 
-PHASES = {"aggregate": ("AGG_BEGIN", "PILE_BEGIN", "AGG_END", "PILE_END"),
-          "search_and_contact": ("KEYS", "SCAN", "SCATTER", "CELL_ORDER", "GATHER", "CONTACT"),
+PHASES = {"aggregate": ("AGG_BEGIN", "AGG_END"),
+          "search_and_contact": ("GATHER", "CONTACT"),
           "gravity": ("GRAVITY",)}
 
 
