@@ -278,7 +278,9 @@ def run_contact_roofline(dem, W, peak_gbs, steps=5, n=1_048_576, warmup=3, mode=
     ms = statistics.median(ks)
     achieved = algo / (ms / 1e3) / 1e9
     return {"bound": "hbm", "achieved": achieved, "peak": peak_gbs, "unit": "GB/s",
-            "frac": achieved / peak_gbs, "peak_source": "measured (MEASURED_PEAKS.json hbm_gbs)",
+            "frac": achieved / peak_gbs,
+            "peak_source": ("measured (MEASURED_PEAKS.json hbm_gbs)" if "hbm_gbs" in peaks()
+                            else "fallback: an earlier copy measurement"),
             "traffic": traffic_for("kernels_contact.cu", "k_contact_sphere" if mode_used == 0 else "k_contact"),
             "kernel": ("k_contact_sphere (one thread per sphere over its kept candidate list)" if mode_used == 0
                        else "k_contact (128-sphere tiles, each inner pair once, shared-memory inbox)"),

@@ -40,7 +40,7 @@
 // opposite displacements, so the copies never differ but in sign, and every
 // access is to consecutive entries of a warp and known ahead.  (Kept once, at
 // the owner's entry, the partner's side read it out of order, often a second
-// time from HBM: 272 us on the 1M lattice, 201 so.)  A rebuild carries it over
+// time from HBM: 272 us on the 1M lattice, 197 so.)  A rebuild carries it over
 // to the new lists by partner index.
 //
 // Mixed precision positions.  The overlap x = s_a + s_b - |d| of two nearby
@@ -399,7 +399,7 @@ __device__ __forceinline__ void sphere_contacts(const Arrays &a, const PileStati
         // the list entry and the history two ahead are in flight while an entry
         // is evaluated (both are consecutive for the warp, so no address waits
         // for a load); the partner's data is fetched where it is used, which
-        // leaves room for a fifth block per SM (96 registers): 201 us on the 1M
+        // leaves room for a fifth block per SM (96 registers): 201 us (now 197) on the 1M
         // lattice, 252 with it one entry ahead and four blocks, 210 with it
         // prefetched to L2
         const int last = off + 32 * (n - 1);   // (n > 0 where it is used)
