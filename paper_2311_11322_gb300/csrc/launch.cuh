@@ -26,9 +26,11 @@ namespace dem {
 
 // Whether launch_pdl and launch_coop set the attribute, chosen by the world
 // before it captures its step (per host thread: a world is used by one thread
-// at a time).  Measured per step of 19 kernels without and with: 1,000 spheres
-// 82 -> 76 us, but 2e4 spheres 224 -> 231 us and 1e5 spheres 2.872 -> 2.891
-// ms, so worlds above 8,192 spheres launch plainly.
+// at a time).  Measured per step without and with: 1,000 spheres 82 -> 76 us
+// (19 kernels); of the present 5 or 6 kernels, 2e4 spheres 161.2 -> 160.0 us,
+// but 65,536 without gravity 50.2 -> 53.2 us, 1e5 2.665 -> 2.667 ms and 5e4
+// with tree gravity 438 -> 443 us, so worlds above 8,192 spheres launch
+// plainly.
 inline thread_local bool tl_pdl = true;
 constexpr int64_t kPdlMaxSpheres = 8192;
 
