@@ -299,6 +299,9 @@ dem_status dem_remove_pile(dem_world *w, int32_t pile_id);
  * with more entries are split into sphere ranges that fit, and pairs across
  * ranges are evaluated from both sides: results are bitwise the same for
  * every value, only the speed changes),
+ * "list_wait" (polls after which a block of the list kernel that waits for the
+ * others' part of a rebuild leaves the rest to those still working, 0..2^30,
+ * default 2^23, some seconds; results are bitwise the same for every value),
  * "cell_factor" (cell edge / (2 x
  * largest radius), >= 1), "skin" (neighbour-list skin as a fraction of the
  * pile's largest radius, in [0, 4], default 0.1; 0 = search contacts afresh

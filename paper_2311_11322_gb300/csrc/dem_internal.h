@@ -22,6 +22,7 @@ constexpr int kScanTile = 2048;    // cells per scan block (256 threads x 8)
 constexpr int kAggChunk = 512;     // aggregates per chunk of a pile reduction
 constexpr int kPartialDoubles = 16;
 constexpr int kChunkWarps = kAggChunk / 32;
+constexpr int kListWords = 32;     // phase counters of the list kernel
 // Contact pass: tiles of consecutive sorted spheres, one block each; the
 // candidate lists of a pile hold kEntPerSphere entries per sphere on average
 // at the default skin (more for larger skins, in proportion to the candidate
@@ -221,7 +222,7 @@ struct Arrays {
     float *aref;
     // cells
     int32_t *ccount, *cstart, *tile_sum;
-    unsigned *lbar;                // barrier words of k_lists (zero between launches)
+    unsigned *lbar;                // [kListWords] phase counters of k_lists (zero between launches)
     // pile reductions
     double *chunk_part;            // [chunks][kPartialDoubles]
     int32_t *chunk_pile;           // [chunks] pile slot of each chunk
@@ -273,7 +274,8 @@ struct Sizes {
     // FP64 symmetric form: items of the piles with tiles of 512 >> c spheres
     // are [g64_first[c], g64_first[c + 1]), run by at most g64_blocks[c] blocks
     int64_t g64_first[6], g64_blocks[5];
-    int64_t LB;      // blocks of k_lists that are resident at once
+    int64_t LB;      // blocks of k_lists that the GPU holds at once
+    int32_t lwait;   // polls after which a waiting block of k_lists leaves the rest of a rebuild to the others
 };
 
 // ---- kernel launchers (kernels_*.cu) -------------------------------------

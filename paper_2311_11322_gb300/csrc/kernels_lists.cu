@@ -7,14 +7,24 @@
 // and gathers the spheres (HBM-bound: about 250 B per sphere).  In a step in
 // which some pile does (its aggregates may have moved half the skin, or the
 // host wrote its state), the same launch also sorts that pile's spheres into
-// cells and builds its lists, the phases separated by a barrier over the grid
-// (a cooperative launch: every block is resident).  As eleven kernels of
-// their own -- clear, keys, three scans, scatter, order, count, scan, fill,
-// link -- the rebuild phases cost a launch each in every step, although they
-// returned at once in all but one of several hundred.  A step of 1,000
-// spheres went from 50.8 to 31.2 us with this launch and the reductions folded
-// into it and its neighbours (19 kernels -> 5), of 7,466 spheres with a planet
-// from 98.7 to 61 us.
+// cells and builds its lists, in phases, each of which starts when all of the
+// one before is done.  As eleven kernels of their own -- clear, keys, three
+// scans, scatter, order, count, scan, fill, link -- the rebuild phases cost a
+// launch each in every step, although they returned at once in all but one of
+// several hundred.  A step of 1,000 spheres went from 50.8 to 33.3 us with this
+// launch and the reductions folded into it and its neighbours (19 kernels ->
+// 5; 31.2 with its programmatic launch), of 7,466 spheres with a planet from
+// 98.7 to 61 us.
+//
+// The phases' order (run_phase).  A phase is cut into items, which the blocks
+// draw from a counter; a block that finds none left waits until all drawn ones
+// are done.  A block never waits while it holds an item, so every item that was
+// drawn gets done, and the block that does a phase's last one goes on to the
+// next whatever the others do.  Nothing therefore depends on how many blocks
+// run at the same time (an ordinary launch: the grid need not be resident, and
+// kernels of other streams take their share of the chip), nor on how long a
+// wait lasts: it is bounded, and a block that gives up leaves the rest of the
+// rebuild to those still working.
 //
 // Cells: a wrapped uniform grid numbered brick by brick (cell_id); a counting
 // sort, each cell ordered by home index, so the order of neighbours is
@@ -55,20 +65,43 @@ __device__ __forceinline__ bool any_rebuild(const Arrays &a, const Sizes &z)
     return __syncthreads_or(mine) != 0;
 }
 
-// Barrier number `word` of this launch over all blocks (cooperative launch:
-// all are resident).  The wait is bounded, a second or so; a block that gives
-// up answers false, as do then all others.
-constexpr int kBarWords = 16;   // the last one counts the blocks that are done
-__device__ __forceinline__ bool grid_barrier(const Arrays &a, int word)
+// Phases of a rebuild, in order, and the words of Arrays::lbar: per phase the
+// next item and the items done, then the blocks that are done with the launch.
+enum { kClear, kKeys, kScanTiles, kScanPiles, kScanCells, kScatter, kOrder, kGather, kCount, kListScan, kFill, kLink,
+       kPhases };
+static_assert(2 * kPhases < kListWords, "the words of all phases and the last one");
+
+// Phase ph (see the file comment): f(item), by the whole block, for the items
+// of [0, items) that this block draws, then the wait for those of the others.
+// False if the wait ran out.  sh: a shared word.  Measured, us of a step that
+// rebuilds, with a fixed share of the items for every block and a barrier over
+// a resident grid -> this: 1,000 spheres 107 -> 115, 100,000 278 -> 276,
+// 1,048,576 1,729 -> 1,797 (three items a draw there: 1,911; the next item
+// drawn ahead: 163 at 1,000).
+template <typename Fn>
+__device__ __forceinline__ bool run_phase(const Arrays &a, const Sizes &z, int ph, int64_t items, unsigned *sh, Fn f)
 {
-    __syncthreads();
+    unsigned *next = a.lbar + 2 * ph, *done = next + 1;
+    const unsigned n = (unsigned)items;
+    for (bool held = false;; held = true) {
+        __syncthreads();   // the block has done its item (and read *sh)
+        if (threadIdx.x == 0) {
+            if (held) {
+                __threadfence();   // visible before it counts as done
+                atomicAdd(done, 1u);
+            }
+            *sh = atomicAdd(next, 1u);
+        }
+        __syncthreads();
+        const unsigned item = *sh;
+        if (item >= n) break;
+        f((int64_t)item);
+    }
     int ok = 1;
     if (threadIdx.x == 0) {
-        volatile unsigned *w = a.lbar + word;
-        __threadfence();
-        atomicAdd(a.lbar + word, 1u);
-        for (int it = 0; *w < gridDim.x; ++it) {
-            if (it > (1 << 23)) {
+        const volatile unsigned *w = done;
+        for (int it = 0; *w < n; ++it) {
+            if (it >= z.lwait) {
                 ok = 0;
                 break;
             }
@@ -79,14 +112,14 @@ __device__ __forceinline__ bool grid_barrier(const Arrays &a, int word)
     return __syncthreads_and(ok) != 0;
 }
 
-// The last block of a rebuild puts the barrier words back to zero.
-__device__ __forceinline__ void grid_done(const Arrays &a)
+// The last block of a launch that rebuilds puts the words back to zero.
+__device__ __forceinline__ void phases_done(const Arrays &a)
 {
     __syncthreads();
     if (threadIdx.x != 0) return;
     __threadfence();
-    if (atomicAdd(a.lbar + kBarWords - 1, 1u) == gridDim.x - 1)
-        for (int k = 0; k < kBarWords; ++k) a.lbar[k] = 0;
+    if (atomicAdd(a.lbar + kListWords - 1, 1u) == gridDim.x - 1)
+        for (int k = 0; k < kListWords; ++k) a.lbar[k] = 0;
 }
 
 // Exclusive prefix sum over the block's kLB threads; *total gets the sum.
@@ -142,43 +175,45 @@ __device__ __forceinline__ int tile_pile(const Arrays &a, const Sizes &z, int64_
     return lo;
 }
 
-// f(i, p) for this block's spheres of rebuilding piles (index i in all piles)
+// f(i, p) for the spheres of rebuilding piles among the kLB of an item (index
+// i in all piles)
 template <typename Fn>
-__device__ __forceinline__ void rebuilding_spheres(const Arrays &a, const Sizes &z, Fn f)
+__device__ __forceinline__ void rebuilding_spheres(const Arrays &a, const Sizes &z, int64_t item, Fn f)
 {
-    for (int64_t i = (int64_t)blockIdx.x * kLB + threadIdx.x; i < z.N; i += (int64_t)gridDim.x * kLB) {
-        const int p = sphere_pile(a, z, i);
-        if (pile_rebuilds(a, p)) f(i, p);
+    const int64_t i = item * kLB + threadIdx.x;
+    if (i >= z.N) return;
+    const int p = sphere_pile(a, z, i);
+    if (pile_rebuilds(a, p)) f(i, p);
+}
+
+// New neighbour-list reference of a chunk's aggregates (as the test in the
+// drift forms it).
+template <bool FP64>
+__device__ __forceinline__ void reference_chunk(const Arrays &a, int64_t ch)
+{
+    const int p = a.chunk_pile[ch];
+    if (!pile_rebuilds(a, p)) return;
+    const PileStatic &S = a.ps[p];
+    const PileDyn &D = a.pd[p];
+    const int64_t beg = S.a0 + (ch - S.ch0) * kAggChunk, end = min(beg + kAggChunk, S.a0 + S.na);
+    for (int64_t g = beg + threadIdx.x; g < end; g += kLB) {
+        float *ar = a.aref + 8 * g;
+        if constexpr (FP64) {
+            for (int c = 0; c < 3; ++c) ar[c] = (float)(a.r[3 * g + c] - D.O[c] - S.h * D.V[c]);
+            for (int c = 0; c < 4; ++c) ar[3 + c] = (float)a.q[4 * g + c];
+        } else {
+            for (int c = 0; c < 3; ++c) ar[c] = ff_sub(ldff(a.r + 3 * g + c), ff_of2(D.Of[c])).hi - D.hVf[c];
+            for (int c = 0; c < 4; ++c) ar[3 + c] = ldff(a.q + 4 * g + c).hi;
+        }
     }
 }
 
-// New neighbour-list reference of the rebuilding piles' aggregates (as the
-// test in the drift forms it) and zero cell counts.
-template <bool FP64>
-__device__ void clear_phase(const Arrays &a, const Sizes &z)
+// Zero cell counts of scan tile t.
+__device__ __forceinline__ void clear_tile(const Arrays &a, const Sizes &z, int64_t t)
 {
-    for (int64_t ch = blockIdx.x; ch < z.CH; ch += gridDim.x) {
-        const int p = a.chunk_pile[ch];
-        if (!pile_rebuilds(a, p)) continue;
-        const PileStatic &S = a.ps[p];
-        const PileDyn &D = a.pd[p];
-        const int64_t beg = S.a0 + (ch - S.ch0) * kAggChunk, end = min(beg + kAggChunk, S.a0 + S.na);
-        for (int64_t g = beg + threadIdx.x; g < end; g += kLB) {
-            float *ar = a.aref + 8 * g;
-            if constexpr (FP64) {
-                for (int c = 0; c < 3; ++c) ar[c] = (float)(a.r[3 * g + c] - D.O[c] - S.h * D.V[c]);
-                for (int c = 0; c < 4; ++c) ar[3 + c] = (float)a.q[4 * g + c];
-            } else {
-                for (int c = 0; c < 3; ++c) ar[c] = ff_sub(ldff(a.r + 3 * g + c), ff_of2(D.Of[c])).hi - D.hVf[c];
-                for (int c = 0; c < 4; ++c) ar[3 + c] = ldff(a.q + 4 * g + c).hi;
-            }
-        }
-    }
-    for (int64_t t = blockIdx.x; t < z.T; t += gridDim.x) {
-        if (!pile_rebuilds(a, tile_pile(a, z, t))) continue;
-        int4 *c = (int4 *)(a.ccount + t * kScanTile);
-        for (int k = threadIdx.x; k < kScanTile / 4; k += kLB) c[k] = make_int4(0, 0, 0, 0);
-    }
+    if (!pile_rebuilds(a, tile_pile(a, z, t))) return;
+    int4 *c = (int4 *)(a.ccount + t * kScanTile);
+    for (int k = threadIdx.x; k < kScanTile / 4; k += kLB) c[k] = make_int4(0, 0, 0, 0);
 }
 
 // Cell key and rank among the spheres counted into the cell (the rank waits
@@ -207,58 +242,53 @@ __device__ __forceinline__ void key_sphere(const Arrays &a, int64_t i, int p)
     a.sagg[i] = atomicAdd(a.ccount + S.c0 + key, 1);
 }
 
-// Sums of the scan tiles' cell counts.
-__device__ void scan_tiles_phase(const Arrays &a, const Sizes &z, int *ws)
+// Sum of scan tile t's cell counts.
+__device__ __forceinline__ void sum_tile(const Arrays &a, const Sizes &z, int64_t t, int *ws)
 {
-    for (int64_t t = blockIdx.x; t < z.T; t += gridDim.x) {
-        if (!pile_rebuilds(a, tile_pile(a, z, t))) continue;
-        const int4 *c = (const int4 *)(a.ccount + t * kScanTile);
-        int s = 0, tot;
-        for (int k = threadIdx.x; k < kScanTile / 4; k += kLB) {
-            const int4 v = c[k];
-            s += (v.x + v.y) + (v.z + v.w);
-        }
-        block_scan(s, ws, &tot);
-        if (threadIdx.x == 0) a.tile_sum[t] = tot;
+    if (!pile_rebuilds(a, tile_pile(a, z, t))) return;
+    const int4 *c = (const int4 *)(a.ccount + t * kScanTile);
+    int s = 0, tot;
+    for (int k = threadIdx.x; k < kScanTile / 4; k += kLB) {
+        const int4 v = c[k];
+        s += (v.x + v.y) + (v.z + v.w);
+    }
+    block_scan(s, ws, &tot);
+    if (threadIdx.x == 0) a.tile_sum[t] = tot;
+}
+
+// Exclusive scan of pile p's tile sums, in place.
+__device__ __forceinline__ void scan_pile(const Arrays &a, int p, int *ws)
+{
+    if (!pile_rebuilds(a, p)) return;
+    const PileStatic &S = a.ps[p];
+    int carry = 0;
+    for (int64_t base = 0; base < S.nt; base += kLB) {
+        const int64_t t = base + threadIdx.x;
+        int tot;
+        const int at = block_scan(t < S.nt ? a.tile_sum[S.t0 + t] : 0, ws, &tot);
+        if (t < S.nt) a.tile_sum[S.t0 + t] = carry + at;
+        carry += tot;
     }
 }
 
-// Exclusive scan of each pile's tile sums, in place.
-__device__ void scan_piles_phase(const Arrays &a, const Sizes &z, int *ws)
-{
-    for (int p = blockIdx.x; p < z.P; p += gridDim.x) {
-        if (!pile_rebuilds(a, p)) continue;
-        const PileStatic &S = a.ps[p];
-        int carry = 0;
-        for (int64_t base = 0; base < S.nt; base += kLB) {
-            const int64_t t = base + threadIdx.x;
-            int tot;
-            const int at = block_scan(t < S.nt ? a.tile_sum[S.t0 + t] : 0, ws, &tot);
-            if (t < S.nt) a.tile_sum[S.t0 + t] = carry + at;
-            carry += tot;
-        }
-    }
-}
-
-// Start of every cell: exclusive scan inside each tile plus the tile's offset.
-__device__ void scan_cells_phase(const Arrays &a, const Sizes &z, int *ws)
+// Start of every cell of scan tile t: exclusive scan inside the tile plus the
+// tile's offset.
+__device__ __forceinline__ void scan_cells(const Arrays &a, const Sizes &z, int64_t t, int *ws)
 {
     constexpr int kPer = kScanTile / kLB;
-    for (int64_t t = blockIdx.x; t < z.T; t += gridDim.x) {
-        if (!pile_rebuilds(a, tile_pile(a, z, t))) continue;
-        const int4 *c = (const int4 *)(a.ccount + t * kScanTile) + threadIdx.x * (kPer / 4);
-        int4 *o = (int4 *)(a.cstart + t * kScanTile) + threadIdx.x * (kPer / 4);
-        int loc = 0, tot;
-        for (int k = 0; k < kPer / 4; ++k) {
-            const int4 v = c[k];
-            loc += (v.x + v.y) + (v.z + v.w);
-        }
-        int run = a.tile_sum[t] + block_scan(loc, ws, &tot);
-        for (int k = 0; k < kPer / 4; ++k) {
-            const int4 v = c[k];
-            o[k] = make_int4(run, run + v.x, run + v.x + v.y, run + v.x + v.y + v.z);
-            run += (v.x + v.y) + (v.z + v.w);
-        }
+    if (!pile_rebuilds(a, tile_pile(a, z, t))) return;
+    const int4 *c = (const int4 *)(a.ccount + t * kScanTile) + threadIdx.x * (kPer / 4);
+    int4 *o = (int4 *)(a.cstart + t * kScanTile) + threadIdx.x * (kPer / 4);
+    int loc = 0, tot;
+    for (int k = 0; k < kPer / 4; ++k) {
+        const int4 v = c[k];
+        loc += (v.x + v.y) + (v.z + v.w);
+    }
+    int run = a.tile_sum[t] + block_scan(loc, ws, &tot);
+    for (int k = 0; k < kPer / 4; ++k) {
+        const int4 v = c[k];
+        o[k] = make_int4(run, run + v.x, run + v.x + v.y, run + v.x + v.y + v.z);
+        run += (v.x + v.y) + (v.z + v.w);
     }
 }
 
@@ -482,25 +512,22 @@ __device__ __forceinline__ void load_me(const Arrays &a, int64_t k, CandMe &m)
 
 // Slices: the 32 consecutive sorted spheres a warp takes; slice s of tile t
 // (four to a tile) has entry 4 t + s of ctile_cnt and ctile_base.
-// f(p, first sorted position, spheres, slice) for this block's slices of
-// rebuilding piles, one warp each; whole warps call it.
+// f(p, first sorted position, spheres, slice) for the slices of tile t, one
+// warp each, if its pile rebuilds; whole warps call it.
 template <typename Fn>
-__device__ __forceinline__ void rebuilding_slices(const Arrays &a, const Sizes &z, Fn f)
+__device__ __forceinline__ void rebuilding_slices(const Arrays &a, int64_t t, Fn f)
 {
     const int wid = threadIdx.x >> 5;
-    for (int64_t t = blockIdx.x; t < z.CT; t += gridDim.x) {
-        const int4 tl = a.ctile[t];
-        if (!pile_rebuilds(a, tl.x)) continue;
-        f(tl.x, tl.y + 32 * wid, min(32, tl.z - 32 * wid), 4 * t + wid);
-    }
+    const int4 tl = a.ctile[t];
+    if (pile_rebuilds(a, tl.x)) f(tl.x, tl.y + 32 * wid, min(32, tl.z - 32 * wid), 4 * t + wid);
 }
 
 // Candidates per sphere (new list buffer) and entries per slice: a slice is
 // as wide as its longest list.
 template <bool FP64>
-__device__ void count_phase(const Arrays &a, const Sizes &z)
+__device__ __forceinline__ void count_tile(const Arrays &a, int64_t t)
 {
-    rebuilding_slices(a, z, [&](int p, int first, int ns, int64_t slice) {
+    rebuilding_slices(a, t, [&](int p, int first, int ns, int64_t slice) {
         const PileStatic &S = a.ps[p];
         const int lp = a.pd[p].cpar ^ 1, lane = threadIdx.x & 31;
         int n = 0;
@@ -516,35 +543,33 @@ __device__ void count_phase(const Arrays &a, const Sizes &z)
     });
 }
 
-// Exclusive scan of each pile's slices.  Lists that do not fit the pile's
+// Exclusive scan of pile p's slices.  Lists that do not fit the pile's
 // entries flag the pile (frozen at the end of the step).
-__device__ void list_scan_phase(const Arrays &a, const Sizes &z, long long *ws)
+__device__ __forceinline__ void scan_lists(const Arrays &a, int p, long long *ws)
 {
     constexpr int kPer = 8;
-    for (int p = blockIdx.x; p < z.P; p += gridDim.x) {
-        if (!pile_rebuilds(a, p)) continue;
-        const PileStatic &S = a.ps[p];
-        const int64_t n = 4 * S.nct, o = 4 * S.ct0;
-        long long carry = 0;
-        for (int64_t base = 0; base < n; base += kPer * kLB) {
-            const int64_t t = base + (int64_t)kPer * threadIdx.x;
-            long long v[kPer], loc = 0, tot;
-            for (int k = 0; k < kPer; ++k) {
-                v[k] = t + k < n ? a.ctile_cnt[o + t + k] : 0;
-                loc += v[k];
-            }
-            long long run = carry + block_scan(loc, ws, &tot);
-            for (int k = 0; k < kPer; ++k) {
-                if (t + k < n) a.ctile_base[o + t + k] = (int32_t)run;
-                run += v[k];
-            }
-            carry += tot;
+    if (!pile_rebuilds(a, p)) return;
+    const PileStatic &S = a.ps[p];
+    const int64_t n = 4 * S.nct, o = 4 * S.ct0;
+    long long carry = 0;
+    for (int64_t base = 0; base < n; base += kPer * kLB) {
+        const int64_t t = base + (int64_t)kPer * threadIdx.x;
+        long long v[kPer], loc = 0, tot;
+        for (int k = 0; k < kPer; ++k) {
+            v[k] = t + k < n ? a.ctile_cnt[o + t + k] : 0;
+            loc += v[k];
         }
-        if (carry > S.ne) {
-            if (threadIdx.x == 0) atomicOr(&a.pd[p].flags, DEM_FLAG_SLOTS);
-            __syncthreads();
-            for (int64_t t = threadIdx.x; t < n; t += kLB) a.ctile_base[o + t] = -1;
+        long long run = carry + block_scan(loc, ws, &tot);
+        for (int k = 0; k < kPer; ++k) {
+            if (t + k < n) a.ctile_base[o + t + k] = (int32_t)run;
+            run += v[k];
         }
+        carry += tot;
+    }
+    if (carry > S.ne) {
+        if (threadIdx.x == 0) atomicOr(&a.pd[p].flags, DEM_FLAG_SLOTS);
+        __syncthreads();
+        for (int64_t t = threadIdx.x; t < n; t += kLB) a.ctile_base[o + t] = -1;
     }
 }
 
@@ -600,9 +625,9 @@ __device__ __forceinline__ void fill_sphere(const Arrays &a, const PileStatic &S
 }
 
 template <bool FP64>
-__device__ void fill_phase(const Arrays &a, const Sizes &z, int2 (*s_list)[kLB])
+__device__ __forceinline__ void fill_tile(const Arrays &a, int64_t t, int2 (*s_list)[kLB])
 {
-    rebuilding_slices(a, z, [&](int p, int first, int ns, int64_t slice) {
+    rebuilding_slices(a, t, [&](int p, int first, int ns, int64_t slice) {
         const PileStatic &S = a.ps[p];
         const int lane = threadIdx.x & 31, base = a.ctile_base[slice];
         if (base < 0 || lane >= ns) return;
@@ -664,9 +689,9 @@ __device__ __forceinline__ void cand_link_sphere(const Arrays &a, int p, int kl)
 }
 
 template <bool FP64>
-__device__ void link_phase(const Arrays &a, const Sizes &z)
+__device__ __forceinline__ void link_tile(const Arrays &a, int64_t t)
 {
-    rebuilding_slices(a, z, [&](int p, int first, int ns, int64_t slice) {
+    rebuilding_slices(a, t, [&](int p, int first, int ns, int64_t slice) {
         const int lane = threadIdx.x & 31;
         if (a.ctile_base[slice] >= 0 && lane < ns) cand_link_sphere<FP64>(a, p, first + lane);
     });
@@ -690,48 +715,47 @@ __global__ void __launch_bounds__(kLB, 7) k_lists(Arrays a, Sizes z)
     __shared__ int2 s_list[kFillCap][kLB];   // (partner home index, sorted position)
     __shared__ long long ws[kLB / 32];
     int *wsi = (int *)ws;
-    const bool rb = any_rebuild(a, z);
-    bool ok = true;
-    if (rb) {
-        clear_phase<FP64>(a, z);
-        ok = ok && grid_barrier(a, 0);
-        if (ok) rebuilding_spheres(a, z, [&](int64_t i, int p) { key_sphere<FP64>(a, i, p); });
-        ok = ok && grid_barrier(a, 1);
-        if (ok) scan_tiles_phase(a, z, wsi);
-        ok = ok && grid_barrier(a, 2);
-        if (ok) scan_piles_phase(a, z, wsi);
-        ok = ok && grid_barrier(a, 3);
-        if (ok) scan_cells_phase(a, z, wsi);
-        ok = ok && grid_barrier(a, 4);
-        if (ok) rebuilding_spheres(a, z, [&](int64_t i, int p) { scatter_sphere(a, i, p); });
-        ok = ok && grid_barrier(a, 5);
-        if (ok) rebuilding_spheres(a, z, [&](int64_t k, int p) { order_cell(a, k, p); });
-        ok = ok && grid_barrier(a, 6);
-    }
-    // the first blocks sum the piles' chunks (a long chain of loads and
-    // shuffles beside the others' gather), the rest gather
-    if (ok) {
+    const int64_t nsb = (z.N + kLB - 1) / kLB;   // blocks' worth of spheres
+    auto gather = [&](int64_t k) {
+        if (k < z.N) gather_sphere<FP64>(a, k, sphere_pile(a, z, k));
+    };
+    if (!any_rebuild(a, z)) {
+        // the first blocks sum the piles' chunks (a long chain of loads and
+        // shuffles beside the others' gather), the rest gather
         const int64_t nred = lists_reducers(z), b = (int64_t)blockIdx.x - nred;
         if (b < 0)
             for (int64_t ch = blockIdx.x; ch < z.CH; ch += nred) open_chunk<FP64, kLB>(a, ch);
         else
-            for (int64_t k = b * kLB + threadIdx.x; k < z.N; k += (gridDim.x - nred) * kLB)
-                gather_sphere<FP64>(a, k, sphere_pile(a, z, k));
+            for (int64_t k = b * kLB + threadIdx.x; k < z.N; k += (gridDim.x - nred) * kLB) gather(k);
+        return;
     }
-    if (!rb) return;
-    ok = ok && grid_barrier(a, 7);
-    if (ok) count_phase<FP64>(a, z);
-    ok = ok && grid_barrier(a, 8);
-    if (ok) list_scan_phase(a, z, ws);
-    ok = ok && grid_barrier(a, 9);
-    if (ok) fill_phase<FP64>(a, z, s_list);
-    ok = ok && grid_barrier(a, 10);
-    if (ok) link_phase<FP64>(a, z);
-    else
-        // a barrier timed out: the rebuilding piles have no lists and are frozen
-        for (int p = threadIdx.x; p < z.P; p += kLB)
-            if (pile_rebuilds(a, p)) atomicOr(&a.pd[p].flags, DEM_FLAG_SLOTS);
-    grid_done(a);
+    __shared__ unsigned drawn;
+    auto phase = [&](int ph, int64_t items, auto f) { return run_phase(a, z, ph, items, &drawn, f); };
+    if (phase(kClear, z.CH + z.T, [&](int64_t t) {
+            if (t < z.CH) reference_chunk<FP64>(a, t);
+            else clear_tile(a, z, t - z.CH);
+        }) &&
+        phase(kKeys, nsb, [&](int64_t t) {
+            rebuilding_spheres(a, z, t, [&](int64_t i, int p) { key_sphere<FP64>(a, i, p); });
+        }) &&
+        phase(kScanTiles, z.T, [&](int64_t t) { sum_tile(a, z, t, wsi); }) &&
+        phase(kScanPiles, z.P, [&](int64_t p) { scan_pile(a, (int)p, wsi); }) &&
+        phase(kScanCells, z.T, [&](int64_t t) { scan_cells(a, z, t, wsi); }) &&
+        phase(kScatter, nsb, [&](int64_t t) {
+            rebuilding_spheres(a, z, t, [&](int64_t i, int p) { scatter_sphere(a, i, p); });
+        }) &&
+        phase(kOrder, nsb, [&](int64_t t) {
+            rebuilding_spheres(a, z, t, [&](int64_t k, int p) { order_cell(a, k, p); });
+        }) &&
+        phase(kGather, z.CH + nsb, [&](int64_t t) {
+            if (t < z.CH) open_chunk<FP64, kLB>(a, t);
+            else gather((t - z.CH) * kLB + threadIdx.x);
+        }) &&
+        phase(kCount, z.CT, [&](int64_t t) { count_tile<FP64>(a, t); }) &&
+        phase(kListScan, z.P, [&](int64_t p) { scan_lists(a, (int)p, ws); }) &&
+        phase(kFill, z.CT, [&](int64_t t) { fill_tile<FP64>(a, t, s_list); }))
+        phase(kLink, z.CT, [&](int64_t t) { link_tile<FP64>(a, t); });
+    phases_done(a);
 }
 
 int lists_blocks_per_sm(bool fp64)
@@ -747,8 +771,8 @@ void launch_lists(const Arrays &a, const Sizes &z, bool fp64, cudaStream_t st)
     if (z.N == 0) return;
     const int64_t want = (z.N + kLB - 1) / kLB + lists_reducers(z);
     const unsigned nb = (unsigned)(want < z.LB ? want : z.LB);
-    if (fp64) launch_coop(k_lists<true>, nb, kLB, 0, st, a, z);
-    else launch_coop(k_lists<false>, nb, kLB, 0, st, a, z);
+    if (fp64) launch_pdl(k_lists<true>, nb, kLB, 0, st, a, z);
+    else launch_pdl(k_lists<false>, nb, kLB, 0, st, a, z);
 }
 
 }  // namespace dem

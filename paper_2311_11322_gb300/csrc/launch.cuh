@@ -24,9 +24,9 @@
 
 namespace dem {
 
-// Whether launch_pdl and launch_coop set the attribute, chosen by the world
-// before it captures its step (per host thread: a world is used by one thread
-// at a time).  Measured per step without and with: 1,000 spheres 82 -> 76 us
+// Whether launch_pdl sets the attribute, chosen by the world before it
+// captures its step (per host thread: a world is used by one thread at a
+// time).  Measured per step without and with: 1,000 spheres 82 -> 76 us
 // (19 kernels); of the present 5 or 6 kernels, 2e4 spheres 161.2 -> 160.0 us,
 // but 65,536 without gravity 50.2 -> 53.2 us, 1e5 2.665 -> 2.667 ms and 5e4
 // with tree gravity 438 -> 443 us, so worlds above 8,192 spheres launch
@@ -56,30 +56,6 @@ inline void launch_pdl(void (*kernel)(KArgs...), dim3 grid, dim3 block, size_t s
     at[0].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = at;
     cfg.numAttrs = (DEM_PDL && tl_pdl) ? 1 : 0;
-    cudaLaunchKernelEx(&cfg, kernel, std::forward<Args>(args)...);
-}
-
-// The same as a cooperative launch (all blocks resident at once, so that they
-// may wait for one another; the grid must fit the device).  The blocks wait
-// for one another only after pdl_enter(), and the next kernel's blocks are not
-// launched before every one of them has passed it, so the programmatic
-// attribute goes with it (1,000 spheres 33.3 -> 31.2 us per step).
-template <typename... KArgs, typename... Args>
-inline void launch_coop(void (*kernel)(KArgs...), dim3 grid, dim3 block, size_t smem, cudaStream_t st,
-                        Args &&...args)
-{
-    cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = grid;
-    cfg.blockDim = block;
-    cfg.dynamicSmemBytes = smem;
-    cfg.stream = st;
-    cudaLaunchAttribute at[2];
-    at[0].id = cudaLaunchAttributeCooperative;
-    at[0].val.cooperative = 1;
-    at[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    at[1].val.programmaticStreamSerializationAllowed = 1;
-    cfg.attrs = at;
-    cfg.numAttrs = (DEM_PDL && tl_pdl) ? 2 : 1;
     cudaLaunchKernelEx(&cfg, kernel, std::forward<Args>(args)...);
 }
 

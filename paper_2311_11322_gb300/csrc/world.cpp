@@ -91,6 +91,7 @@ struct dem_world {
     bool sym64_fallback = false;      // the FP64 path's small tiles did not fit: 512-sphere tiles
     double cell_factor = 1.0;
     double skin_frac = 0.1;           // neighbour-list skin / largest radius
+    int list_wait = 1 << 23;          // polls of a waiting block of k_lists, seconds (testing: fewer)
     int contact_inbox = kInboxCap;    // contact inbox entries per tile range (testing: smaller splits more)
     int contact_mode = 0;             // 0: one thread per sphere, 1: tiles with a shared-memory inbox
     // flags readback
@@ -253,7 +254,7 @@ void build_fields(dem_world *w)
     add((void **)&a.ccount, C_CELL, 4, false);
     add((void **)&a.cstart, C_CELL, 4, false);
     add((void **)&a.tile_sum, C_TILE, 4, false);
-    add((void **)&a.lbar, C_PILE, 64, false);
+    add((void **)&a.lbar, C_PILE, 4 * kListWords, false);
     add((void **)&a.chunk_part, C_CHUNK, 8 * kPartialDoubles, false);
     add((void **)&a.chunk_pile, C_CHUNK, 4, false);
     add((void **)&a.warp_part, C_CHUNK, 24 * kChunkWarps, false);
@@ -702,6 +703,7 @@ dem_status upload_tables(dem_world *w, const GravPlan &gp)
     for (int c = 0; c < kSym64Tiles; ++c)
         w->Z.g64_blocks[c] = gp.first64[c + 1] == gp.first64[c] ? 0
             : (int64_t)std::max(1, gravity_blocks_per_sm(true, 128, 4, false, true, kGravSymTile >> c)) * w->sm_count;
+    w->Z.lwait = w->list_wait;
     w->Z.icap = w->contact_inbox;
     w->Z.gacc_on = (w->precision == DEM_MIXED && use_sym(w) && !(w->grav_theta > 0))
                        ? (w->Z.N <= kGaccFuseMax ? 2 : 1) : 0;
@@ -737,7 +739,7 @@ dem_status upload_tables(dem_world *w, const GravPlan &gp)
     CU(cudaMemsetAsync(w->A.gcounter, 0, sizeof(int32_t), w->stream));
     // the mixed path's gravity accumulators (each step's conversion leaves them at zero)
     if (w->A.gacc && w->Z.N > 0) CU(cudaMemsetAsync(w->A.gacc, 0, 32 * (size_t)w->Z.N, w->stream));
-    if (w->Z.P > 0) CU(cudaMemsetAsync(w->A.lbar, 0, 64, w->stream));
+    if (w->Z.P > 0) CU(cudaMemsetAsync(w->A.lbar, 0, 4 * kListWords, w->stream));
     // arrival counters of the pile reductions (each reduction leaves them at zero)
     if (w->Z.P > 0) CU(cudaMemsetAsync(w->A.pile_arrive, 0, sizeof(int32_t) * (size_t)w->Z.P, w->stream));
     launch_fill_ids(w->A, w->Z, w->stream);
@@ -2038,6 +2040,10 @@ dem_status dem_set_tuning(dem_world *w, const char *key, double value)
         if (!(value >= 1.0) || value > kInboxCap)
             return fail(w, DEM_ERR_ARG, "contact_inbox must be in [1, %d]", kInboxCap);
         w->contact_inbox = (int)value;
+    } else if (k == "list_wait") {
+        if (!(value >= 0.0) || value > (double)(1 << 30))
+            return fail(w, DEM_ERR_ARG, "list_wait must be in [0, %d]", 1 << 30);
+        w->list_wait = (int)value;
     } else if (k == "cell_factor" || k == "skin") {
         if (k == "cell_factor" && (!(value >= 1.0) || value > 16.0))
             return fail(w, DEM_ERR_ARG, "cell_factor must be in [1, 16]");
@@ -2074,6 +2080,7 @@ dem_status dem_get_tuning(dem_world *w, const char *key, double *value_out)
     else if (k == "skin") *value_out = w->skin_frac;
     else if (k == "contact_inbox") *value_out = w->contact_inbox;
     else if (k == "contact_mode") *value_out = w->contact_mode;
+    else if (k == "list_wait") *value_out = w->list_wait;
     else return fail(w, DEM_ERR_ARG, "unknown tuning key '%s'", key);
     return DEM_OK;
 }
