@@ -292,33 +292,41 @@ __device__ __forceinline__ void scan_cells(const Arrays &a, const Sizes &z, int6
     }
 }
 
+// The pile's spheres (home indices) by cell, not yet ordered inside the cells:
+// in a sorted copy that the gather, a later phase, writes anew.
+template <bool FP64>
+__device__ __forceinline__ int32_t *unordered(const Arrays &a, const PileStatic &S)
+{
+    if constexpr (FP64) return (int32_t *)(a.dp_ + S.s0);
+    else return (int32_t *)(a.sph_ + S.s0);
+}
+
+template <bool FP64>
 __device__ __forceinline__ void scatter_sphere(const Arrays &a, int64_t i, int p)
 {
     const PileStatic &S = a.ps[p];
     const int slot = a.cstart[S.c0 + a.key[i]] + a.sagg[i];
-    a.sorted[S.s0 + slot] = (int32_t)(i - S.s0);
+    unordered<FP64>(a, S)[slot] = (int32_t)(i - S.s0);
 }
 
-// The thread at the first position of each cell sorts that cell's entries by
-// home index (insertion sort; cells hold a handful of spheres).
-__device__ __forceinline__ void order_cell(const Arrays &a, int64_t k, int p)
+// The sphere in place k of the cells takes its place by home index: the number
+// of its cell's spheres with a smaller one.  Cells hold a handful of spheres,
+// but a wide range of radii, a large cell_size or a fragment far away can put
+// a whole pile into a few, and sorting such a cell in one thread takes seconds
+// (40,000 spheres beside one of 60 times their radius: 13 s for the step that
+// rebuilds, 0.03 s so).
+template <bool FP64>
+__device__ __forceinline__ void order_sphere(const Arrays &a, int64_t k, int p)
 {
     const PileStatic &S = a.ps[p];
-    int32_t *srt = a.sorted + S.s0;
-    const int kl = (int)(k - S.s0);
-    const int key = a.key[S.s0 + srt[kl]];
-    const int start = a.cstart[S.c0 + key];
-    if (kl != start) return;
-    const int n = a.ccount[S.c0 + key];
-    for (int x = 1; x < n; ++x) {
-        const int v = srt[start + x];
-        int y = x - 1;
-        while (y >= 0 && srt[start + y] > v) {
-            srt[start + y + 1] = srt[start + y];
-            --y;
-        }
-        srt[start + y + 1] = v;
-    }
+    const int32_t *un = unordered<FP64>(a, S);
+    const int me = un[k - S.s0];
+    const int key = a.key[S.s0 + me];
+    const int start = a.cstart[S.c0 + key], n = a.ccount[S.c0 + key];
+    int r = 0;
+#pragma unroll 4
+    for (int x = 0; x < n; ++x) r += un[start + x] < me ? 1 : 0;
+    a.sorted[S.s0 + start + r] = me;
 }
 
 // ---------------------------------------------------------------- gather
@@ -742,10 +750,10 @@ __global__ void __launch_bounds__(kLB, 7) k_lists(Arrays a, Sizes z)
         phase(kScanPiles, z.P, [&](int64_t p) { scan_pile(a, (int)p, wsi); }) &&
         phase(kScanCells, z.T, [&](int64_t t) { scan_cells(a, z, t, wsi); }) &&
         phase(kScatter, nsb, [&](int64_t t) {
-            rebuilding_spheres(a, z, t, [&](int64_t i, int p) { scatter_sphere(a, i, p); });
+            rebuilding_spheres(a, z, t, [&](int64_t i, int p) { scatter_sphere<FP64>(a, i, p); });
         }) &&
         phase(kOrder, nsb, [&](int64_t t) {
-            rebuilding_spheres(a, z, t, [&](int64_t k, int p) { order_cell(a, k, p); });
+            rebuilding_spheres(a, z, t, [&](int64_t k, int p) { order_sphere<FP64>(a, k, p); });
         }) &&
         phase(kGather, z.CH + nsb, [&](int64_t t) {
             if (t < z.CH) open_chunk<FP64, kLB>(a, t);

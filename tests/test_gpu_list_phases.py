@@ -100,3 +100,61 @@ def test_worlds_that_share_the_gpu(dem, prec):
     finally:
         for w in worlds:
             w.close()
+
+
+@pytest.mark.parametrize("prec", [W.PRECISION_FP64, W.PRECISION_MIXED])
+@pytest.mark.parametrize("n", [28, 3_001, 40_000])
+def test_cells_of_any_population(dem, prec, n):
+    """Cells far larger than the spheres (the whole pile in a few of them) give the bits of ordinary cells."""
+    ic, p = W.dense_lattice(n_spheres=n, seed=n, precision=prec, speed=0.01)
+    got = []
+    for cell in (0.0, 1.0e4):
+        with dem.World() as w:
+            w.set_tuning("skin", 0.02)
+            pid = w.add_pile(ic, p.replace(cell_size=cell))
+            w.step(20)
+            w.sync()
+            info = w.info(pid)
+            assert info["rebuilds"] > 1 and not int(info["flags"]) & (1 | 2 | 16)
+            got.append(state(w, pid))
+            if cell:
+                assert info["nx"] * info["ny"] * info["nz"] == 27
+    same(got[1], got[0])
+
+
+@pytest.mark.parametrize("prec", [W.PRECISION_FP64, W.PRECISION_MIXED])
+def test_a_boulder_among_grains(dem, prec):
+    """One sphere 60 times as large as the 40,000 others makes cells that hold thousands of them: the pile steps
+    without a flag, and the first step's contacts are those of a search over all pairs."""
+    spatial = pytest.importorskip("scipy.spatial")
+    ic, p = W.dense_lattice(n_spheres=40_000, seed=3, precision=prec)
+    R = 60.0
+    top = ic.pos[:, 2].max() + 1.0 + R + 3.0       # clear of the grains
+    ic.counts = np.append(ic.counts, 1).astype(np.int32)
+    ic.pos = np.vstack([ic.pos, [[0.0, 0.0, top]]])
+    ic.radius = np.append(ic.radius, R)
+    ic.density = np.append(ic.density, 2500.0)
+    ic.vel = np.vstack([ic.vel, np.zeros((1, 3))])
+    ic.omega = np.vstack([ic.omega, np.zeros((1, 3))])
+    with dem.World() as w:
+        w.set_tuning("skin", 0.002)    # (0.1 of the boulder's radius would list hundreds of neighbours per grain)
+        pid = w.add_pile(ic, p)
+        info = w.info(pid)
+        assert info["cell"] > 2 * R
+        w.step(1)
+        w.sync()
+        pairs, _ = w.contacts(pid)
+        pos = w.read(pid, "SPHERE_POS")
+        assert not w.flags(pid) & (1 | 2 | 16)
+        w.step(3)
+        w.sync()
+        assert not w.flags(pid) & (1 | 2 | 16)
+    agg = np.repeat(np.arange(len(ic.counts)), ic.counts)
+    near = spatial.cKDTree(pos[:-1]).query_pairs(2.0, output_type="ndarray")
+    near = near[agg[near[:, 0]] != agg[near[:, 1]]]
+    gap = 2.0 - np.linalg.norm(pos[near[:, 0]] - pos[near[:, 1]], axis=1)
+    # pairs that only just touch (within the rounding of the positions) may be on either side
+    sure = {tuple(sorted(map(int, q))) for q, g in zip(near, gap) if g > 1e-6}
+    maybe = {tuple(sorted(map(int, q))) for q in near}
+    got = set(pairs)
+    assert len(sure) > 40_000 and sure <= got <= maybe
