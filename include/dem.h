@@ -466,8 +466,10 @@ dem_status dem_probe_peak(int32_t kind, int64_t size, int32_t reps, const void *
                           char *msg, size_t msg_len);
 
 /* Device bytes one pile of this size needs with direct-sum gravity (state, sorted
- * copies, cells, history, gravity partial sums).  Tree gravity (grav_theta > 0)
- * needs instead about 0.4 KB per sphere plus 280 B per tree cell. */
+ * copies, cells, history, gravity partial sums).  In the FP64 path it counts the
+ * partial sums of the tile size that a world without a memory budget uses; one
+ * with a budget takes larger tiles and needs less.  Tree gravity (grav_theta >
+ * 0) needs instead about 0.4 KB per sphere plus 280 B per tree cell. */
 size_t dem_footprint_bytes(int64_t n_spheres, int64_t n_agg, int32_t max_contacts,
                            int32_t precision);
 

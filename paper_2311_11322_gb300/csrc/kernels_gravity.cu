@@ -469,8 +469,9 @@ __device__ __forceinline__ void grav_accumulate(const Arrays &a, int64_t s, floa
     if (!ok) atomicOr(bad, (vx != vx || vy != vy || vz != vz) ? DEM_FLAG_NONFINITE : DEM_FLAG_GRAV_RANGE);
 }
 
-// Partial slots of pile p: i-sums of tile pair (a, b) at [b][i], j-sums at
-// [T + a][j], rows of ns spheres from gpart_base[p].
+// Partial slots of pile p, rows of ns spheres from gpart_base[p]: i-sums of
+// tile pair (a, b) at [b][i], j-sums at [a][j].  A sphere of tile t thus has its
+// i-sums in rows t..T-1 and its j-sums in rows 0..t-1: T rows hold them all.
 __device__ __forceinline__ int64_t sym_slot(const Arrays &a, int p, int64_t ns, int64_t row, int64_t i)
 {
     return a.gpart_base[p] + row * ns + i;
@@ -892,7 +893,7 @@ __device__ __forceinline__ void gravity64s_item(const Arrays &a, const int4 it, 
                 u.y += t.y;
                 u.z += t.z;
             }
-            ((dbl4 *)a.gpart)[sym_slot(a, p, ns, T + ta, jb0 + m)] = make_dbl4(u.x, u.y, u.z, 0.0);
+            ((dbl4 *)a.gpart)[sym_slot(a, p, ns, ta, jb0 + m)] = make_dbl4(u.x, u.y, u.z, 0.0);
         }
     }
 #pragma unroll
@@ -959,10 +960,10 @@ __global__ void __launch_bounds__(kCombThreads) k_grav_combine_sym64(Arrays a, S
         const int64_t il = i - S.s0;
         const int t = (int)(il / S.gtile64);
         const dbl4 *gp = (const dbl4 *)a.gpart;
-        // rows t..T-1 (i-sums of the pairs (t, b)), then T..T+t-1 (j-sums of (r, t))
+        // rows t..T-1 (i-sums of the pairs (t, b)), then 0..t-1 (j-sums of (r, t))
 #pragma unroll 4
         for (int r = t + q; r < T + t; r += kCombLanes) {
-            const dbl4 v = gp[sym_slot(a, p, S.ns, r, il)];
+            const dbl4 v = gp[sym_slot(a, p, S.ns, r < T ? r : r - T, il)];
             sx += v.x; sy += v.y; sz += v.z;
         }
     }

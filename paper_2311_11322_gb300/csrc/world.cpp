@@ -346,17 +346,21 @@ int device_sms(dem_world *w)
 // the largest tile of 512 .. 32 spheres that cuts the pile into at least 70
 // (2,485 tile pairs, 16 per SM: a last wave that is nearly empty then costs a
 // few percent), 32 below.  Measured per step, 512 -> this: 1,000 spheres
-// 1,633 -> 104 us, 12,345 spheres 3.10 -> 2.77 ms.  The partial rows
-// (2 T x N x 32 B) grow with the number of tiles T, to 70..140 per pile as at
-// 36,000 to 72,000 spheres before; a world with a memory budget keeps
-// 512-sphere tiles, and so does one whose allocation for the smaller tiles
-// fails (prepare).
+// 1,633 -> 104 us, 12,345 spheres 3.10 -> 2.77 ms.  The partial rows (T x N x
+// 32 B) grow with the number of tiles T, to 70..140 for a pile of 2,240 to
+// 35,000 spheres (20 MB at 4,416, 56 at 17,600); dem_footprint_bytes counts
+// them.  A world with a memory budget keeps 512-sphere tiles, and so does one
+// whose allocation for the smaller tiles fails (prepare).
+int sym64_tile(int64_t ns)
+{
+    int tile = kGravSymTile;
+    while (tile > 32 && (ns + tile - 1) / tile < 70) tile /= 2;
+    return tile;
+}
+
 int sym_tile64(const dem_world *w, const PileHost &q)
 {
-    if (w->budget || w->sym64_fallback) return kGravSymTile;
-    int tile = kGravSymTile;
-    while (tile > 32 && (q.ns + tile - 1) / tile < 70) tile /= 2;
-    return tile;
+    return w->budget || w->sym64_fallback ? kGravSymTile : sym64_tile(q.ns);
 }
 
 // Tile of the symmetric form on the mixed path.  A tile pair's work is the
@@ -415,8 +419,8 @@ void order_items(const std::vector<GravItem> &its, std::vector<int4> &out)
 }
 
 // FP64 symmetric form: every pair of tiles (a, b), a <= b, of every pile,
-// grouped by tile size; partial rows [b][i] and [T + a][j] (2 T rows of ns)
-// for piles with more than one tile.
+// grouped by tile size; T partial rows of ns ([b][i] and [a][j]) for piles with
+// more than one tile.
 void plan_sym64(const dem_world *w, GravPlan &g)
 {
     std::vector<GravItem> its[kSym64Tiles];
@@ -431,7 +435,7 @@ void plan_sym64(const dem_world *w, GravPlan &g)
         g.tile = (int)std::min<int64_t>(g.tile, tile);
         g.nch.push_back((int32_t)T);
         g.base.push_back(T > 1 ? g.gp : -1);
-        if (T > 1) g.gp += 2 * T * q.ns;
+        if (T > 1) g.gp += T * q.ns;
         int c = 0;
         while (kGravSymTile >> c > tile) ++c;
         for (int64_t ta = 0; ta < T; ++ta)
@@ -2299,7 +2303,7 @@ size_t dem_footprint_bytes(int64_t n_spheres, int64_t n_agg, int32_t max_contact
     if (n_spheres < 0 || n_agg < 0 || max_contacts < 1) return 0;
     bool d = precision == DEM_FP64;
     size_t sph = 4 + 4 + 24 + 8 + 8 + 4 + 4 + 4 + 4 + 32;
-    // (4 of the bytes above per sphere cover the lists' slice tables and barrier words)
+    // (4 of the bytes above per sphere cover the lists' slice tables)
     sph += 8;        // pos_of_home, both parities
     sph += 2 * 8;    // candidate counts and offsets, both buffers
     sph += d ? (32 * 3 + 32 + 64) : (16 * 2 + 16 * 5 + 16 + 32);
@@ -2312,15 +2316,16 @@ size_t dem_footprint_bytes(int64_t n_spheres, int64_t n_agg, int32_t max_contact
     size_t bytes = sph * (size_t)n_spheres + ent * (size_t)n_spheres * (size_t)kEntPerSphere +
                    24 * (size_t)((n_spheres + kCTile - 1) / kCTile) +
                    agg * (size_t)n_agg + 8 * (size_t)cells + 4 * (size_t)(cells / kScanTile + 1) +
-                   (size_t)(n_agg / kAggChunk + 1) * (8 * kPartialDoubles + 4 + 8 * 32) +
-                   sizeof(PileStatic) + sizeof(PileDyn) + sizeof(PileWatch) + 20 + 16 * (size_t)(n_spheres / 64 + 1);
-    // direct-sum gravity: partial sums of the 512-sphere tile pairs (2 T rows of
-    // n spheres) and the work items (T (T + 1) / 2); in the mixed path the same
-    // term, with smaller tiles for small piles, covers the integer
+                   (size_t)(n_agg / kAggChunk + 1) * (8 * kPartialDoubles + 4 + 8 * 32 + 24 * kChunkWarps) +
+                   sizeof(PileStatic) + sizeof(PileDyn) + sizeof(PileWatch) + 24 + 4 * kListWords +
+                   16 * (size_t)(n_spheres / 64 + 1);
+    // direct-sum gravity: the work items (T (T + 1) / 2 pairs of T tiles) and, in
+    // the FP64 path, the tile pairs' partial sums (T rows of n spheres); in the
+    // mixed path a term of 2 T rows, as its tiles once had, covers the integer
     // accumulators, the planet's forces and the longer work list
-    const int64_t tile = d ? 512 : n_spheres <= 2048 ? 64 : n_spheres <= 8192 ? 128 : 512;
+    const int64_t tile = d ? sym64_tile(n_spheres) : n_spheres <= 2048 ? 64 : n_spheres <= 8192 ? 128 : 512;
     const int64_t T = (n_spheres + tile - 1) / tile;
-    if (T > 1) bytes += (size_t)(2 * T) * (size_t)n_spheres * (d ? 32 : 16);
+    if (T > 1) bytes += (size_t)(d ? T * 32 : 2 * T * 16) * (size_t)n_spheres;
     bytes += 16 * (size_t)(T * (T + 1) / 2);
     bytes += 256 * 80;   // each of the world's arrays starts on a 256-byte boundary of one slab
     return bytes;

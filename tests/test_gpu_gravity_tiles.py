@@ -104,6 +104,20 @@ def test_fp64_budget_keeps_the_large_tiles(dem):
     assert np.all(np.linalg.norm(got[s] - F, axis=1) <= 1.5e-12 * mag)
 
 
+@pytest.mark.parametrize("planet", [0.0, 5.972e24])
+@pytest.mark.parametrize("prec", [W.PRECISION_FP64, W.PRECISION_MIXED])
+@pytest.mark.parametrize("n", [1, 40, 1000, 4416, 8192, 8193, 12345, 20000])
+def test_stated_footprint_covers_a_world_without_a_budget(dem, n, prec, planet):
+    """A pile's stated footprint holds for the tiles that a world uses which has no memory budget."""
+    ic, p = pile(n, prec)
+    p = p.replace(ext_mass=planet, ext_pos=(3.0e7, 0.0, 0.0))
+    with dem.World() as w:
+        w.add_pile(ic, p)
+        w.step(1)
+        w.sync()
+        assert w.bytes() <= dem.dem_footprint_bytes(ic.n_sph, ic.n_agg, p.max_contacts, prec)
+
+
 # mixed path: 64-sphere tiles to 8,192 spheres, 256 above; equal masses take their own ring
 @pytest.mark.parametrize("equal", [False, True])
 @pytest.mark.parametrize("n", [1, 2, 63, 64, 65, 129, 1000, 8192, 8193, 12345])
