@@ -87,7 +87,7 @@ struct dem_world {
     int grav_order = 4;               // tree gravity: highest multipole rank (4 or 2)
     int tree_maxD = 0;                // deepest tree of the current layout
     int sm_count = 0;
-    bool has_planet = false;          // some pile was added with a planet (mixed path: sizes Arrays::fe)
+    bool has_planet = false;          // some pile has a planet (mixed path: sizes Arrays::fe)
     bool sym64_fallback = false;      // the FP64 path's small tiles did not fit: 512-sphere tiles
     double cell_factor = 1.0;
     double skin_frac = 0.1;           // neighbour-list skin / largest radius
@@ -1996,6 +1996,9 @@ dem_status dem_remove_pile(dem_world *w, int32_t pile_id)
     dem_status s = relayout(w, newp, nullptr);
     if (s != DEM_OK) return s;
     w->piles = newp;
+    w->has_planet = false;   // the planet's forces are sized by the piles that are left
+    for (auto &q : w->piles)
+        if (w->precision == DEM_MIXED && q.P.ext_mass > 0) w->has_planet = true;
     w->graph_valid = false;
     return DEM_OK;
 }

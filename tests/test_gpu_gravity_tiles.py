@@ -257,3 +257,44 @@ def test_noalloc_gravity_parts_and_masks(dem, n, ids, eps):
         w = np.where((agg == agg[i]) | (r2 == 0), 0.0, m / np.where(r2 == 0, 1.0, r2) ** 1.5)
         t = m[i] * w[:, None] * d
         assert np.linalg.norm(got[i] - t.sum(0)) <= 1e-5 * np.linalg.norm(t, axis=1).sum()
+
+
+def test_planet_pile_comes_and_goes(dem):
+    """A planet pile added to and removed from a world without planets: every pile steps as it does alone, and later
+    piles are not charged for a planet's forces."""
+    sets = []
+    for n, mass in ((900, 0.0), (700, 5.972e24), (333, 0.0)):
+        ic, p = pile(n, W.PRECISION_MIXED, seed=n)
+        sets.append((ic, p.replace(ext_mass=mass, ext_pos=(3.0e7, 1.0e6, 0.0), ext_vel=(0.0, 9.0e3, 0.0))))
+    fields = ("COM", "VEL", "QUAT", "FORCE_EXT", "TORQUE", "SPHERE_FG")
+    alone = []
+    for (ic, p), steps in zip(sets, (9, 3, 6)):
+        with dem.World() as w:
+            pid = w.add_pile(ic, p)
+            w.step(steps)
+            alone.append({f: w.read(pid, f) for f in fields})
+    with dem.World() as w:
+        a = w.add_pile(*sets[0])
+        w.step(3)
+        b = w.add_pile(*sets[1])       # the world's first planet
+        w.step(3)
+        assert all(np.array_equal(w.read(b, f), alone[1][f]) for f in fields)
+        assert np.abs(alone[1]["FORCE_EXT"]).max() > 0
+        w.remove(b)
+        c = w.add_pile(*sets[2])
+        w.step(3)
+        b = w.add_pile(*sets[1])       # and again, beside both
+        w.step(3, piles=[b, c])
+        for pid, ref in ((a, alone[0]), (b, alone[1]), (c, alone[2])):
+            assert all(np.array_equal(w.read(pid, f), ref[f]) for f in fields)
+    big = pile(30_000, W.PRECISION_MIXED)
+    held = []
+    for planet_first in (False, True):
+        with dem.World() as w:
+            pid = w.add_pile(*sets[1 if planet_first else 0])
+            w.step(1)
+            w.remove(pid)
+            w.add_pile(*big)
+            w.step(1)
+            held.append(w.bytes())
+    assert held[1] < held[0] + 32 * 900 + 4096    # the first pile's own spheres at most
