@@ -50,6 +50,7 @@ __host__ __device__ __forceinline__ int64_t cell_count(int nx, int ny, int nz)
 }
 
 constexpr int kTreeParts = 16;      // tree gravity: warps that share a group's walk
+constexpr int kTreeMaxDepth = 6;    // levels below the root of the deepest tree
 
 constexpr int kSym64Tiles = 5;   // FP64 symmetric gravity: tiles of 512, 256, 128, 64 or 32 spheres
 

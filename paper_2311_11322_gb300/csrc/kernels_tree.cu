@@ -514,11 +514,12 @@ __global__ void __launch_bounds__(128) k_tree_up(Arrays a, Sizes z, int L)
 constexpr int kSplitL = 2;
 
 // Traversal stack per warp: opened cells whose children are still to be
-// tested.  Each round pops at most 4 and tests their 32 children, so it pushes
-// at most 32, and a level's cells are pushed only when none of that level is
-// left on the stack (or the last of them are popped in the same round): at
-// most 32 cells of each of the levels 2..5 of the deepest tree.
-constexpr int kTreeStack = 32 * 4 + 4;
+// tested.  A round takes the 4 top entries (or what is left) and puts at most
+// 32 children in their place, so a child lies at most 31 places above its
+// parent.  The walk's first cells fill at most 64 / kTreeParts places, and
+// the cells on the stack are of the levels kSplitL .. kTreeMaxDepth - 1 (the
+// deepest level's are leaves): no place above the last is ever used.
+constexpr int kTreeStack = 64 / kTreeParts + 31 * (kTreeMaxDepth - 1 - kSplitL);
 
 // The multipoles up to rank ORDER of two cells on the sphere at x: a / G, one
 // cell in each half of the packed operands.  With u the unit vector from the

@@ -284,12 +284,12 @@ void build_fields(dem_world *w)
 }
 
 // Tree depth of a pile under tree gravity (0 = direct sum): leaves of ~4
-// spheres, 2..6 levels below the root.
+// spheres, 2..kTreeMaxDepth levels below the root.
 int tree_depth(const dem_world *w, const PileHost &q)
 {
     if (!(w->grav_theta > 0) || w->precision != DEM_MIXED || q.P.G == 0.0) return 0;
     int D = 2;   // the walk starts at the 64 cells of level 2
-    while (D < 6 && ((int64_t)1 << (3 * D)) * 4 < q.ns) ++D;
+    while (D < kTreeMaxDepth && ((int64_t)1 << (3 * D)) * 4 < q.ns) ++D;
     return D;
 }
 
