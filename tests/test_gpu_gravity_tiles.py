@@ -213,6 +213,57 @@ def test_tree_gravity_small_angle_is_the_direct_sum(dem, n, order):
     assert np.all(err <= 1e-5 * mag), float((err / np.maximum(mag, 1e-300)).max())
 
 
+# tree depths 2 (53 and 81 spheres), 3 and 4
+@pytest.mark.parametrize("order", [2, 4])
+@pytest.mark.parametrize("k", [3, 7, 40, 300, 1200])
+def test_tree_expansions_of_accepted_cells(dem, k, order):
+    """Moments and expansions by themselves: seven rods of k spheres in corners of a cube, pointing at the eighth
+    corner, where one aggregate of 32 spheres (no forces of its own) probes them.  Its group is the first of the leaf
+    order, and at this angle it accepts each rod whole, as the one cell of the walk's first level that holds it."""
+    rng = np.random.default_rng(k)
+    edge, b, eps = 100.0, 6.0, 0.01
+
+    def ball(m, radius):
+        v = rng.standard_normal((m, 3))
+        return v * (radius * rng.random(m) ** (1 / 3) / np.linalg.norm(v, axis=1))[:, None]
+    pos, rod = [ball(32, 3.0)], [np.full(32, -1)]
+    for c in range(1, 8):
+        corner = edge * np.array([c & 1, c >> 1 & 1, c >> 2 & 1], float)
+        end = np.where(np.arange(k) % 3 == 0, -0.9, 0.9)      # a third at one end: all ranks of moments
+        pos.append(corner + b * end[:, None] * corner / np.linalg.norm(corner) + ball(k, 0.08 * b))
+        rod.append(np.full(k, c))
+    pos, rod = np.concatenate(pos), np.concatenate(rod)
+    n = len(pos)
+    ic = W.PileIC(counts=np.concatenate([[32], np.ones(7 * k, int)]).astype(np.int32), pos=pos,
+                  radius=rng.uniform(0.001, 0.0015, n), density=np.full(n, 2500.0))
+    p = W.Params(G=1.0, dt=1e-9, kn=1.0, eps=eps, precision=W.PRECISION_MIXED)
+    with dem.World() as w:
+        w.set_tuning("grav_theta", 0.45)
+        w.set_tuning("grav_order", order)
+        pid = w.add_pile(ic, p)
+        w.step(1)
+        got, x = w.read(pid, "SPHERE_FG")[:32], w.read(pid, "SPHERE_POS")
+    m = W.sphere_mass(ic.radius, ic.density)
+    F, mag, tol = np.zeros((32, 3)), np.zeros(32), np.zeros(32)
+    for c in range(1, 8):
+        mine = rod == c
+        com = (m[mine, None] * x[mine]).sum(0) / m[mine].sum()
+        radius = np.linalg.norm(x[mine] - com, axis=1).max()
+        d = x[mine][None] - x[:32, None]
+        r = np.linalg.norm(d, axis=2)
+        F += m[:32, None] * ((m[mine] / (r * r + eps ** 2) ** 1.5)[:, :, None] * d).sum(1)
+        part = m[:32] * (m[mine] / (r * r)).sum(1)
+        q = radius / np.linalg.norm(com - x[:32], axis=1)
+        # the ranks left out: (n + 1) q^n of M / d^2 each, M / d^2 at most (1 + q)^2 of the terms' sum
+        tol += part * (1 + q) ** 2 * sum((j + 1) * q ** j for j in range(order + 1, 40))
+        mag += part
+    err = np.linalg.norm(got - F, axis=1)
+    # FP32: some ten roundings of 2^-24 on the way to each term, the sums, and the positions
+    assert np.all(err <= tol + 3e-6 * mag), float((err / mag).max())
+    if order == 2:
+        assert np.all(err > 1e-5 * mag)      # the rods were not summed sphere by sphere
+
+
 def test_tree_piles_of_different_depths_alone_and_in_a_batch_bitwise(dem):
     piles = [pile(n, W.PRECISION_MIXED, seed=13) for n in (3, 270, 2100, 9000, 40)]
 
