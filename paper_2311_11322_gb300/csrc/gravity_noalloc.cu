@@ -92,7 +92,7 @@ __device__ __forceinline__ float rsqrt_normal(float x)
 // correct; contiguous aggregates leave all but one or two tiles of a block to
 // the packed loop.  Measured per call, one sphere per thread, every pair
 // compared and always 4 parts -> this: 10,000 spheres 129 -> 72 us, 20,001
-// 390 -> 190 us, 131,072 11.9 -> 6.7 ms (below 3,000 the launches, 29 us).
+// 390 -> 200 us, 131,072 11.9 -> 6.7 ms (below 3,000 the launches, 29 us).
 template <int PER>
 __global__ void __launch_bounds__(kNABlock)
 k_na_partial(const float4 *__restrict__ pm, const int32_t *__restrict__ agg, int n, int jc,

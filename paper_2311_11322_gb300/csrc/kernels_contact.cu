@@ -399,9 +399,9 @@ __device__ __forceinline__ void sphere_contacts(const Arrays &a, const PileStati
         // the list entry and the history two ahead are in flight while an entry
         // is evaluated (both are consecutive for the warp, so no address waits
         // for a load); the partner's data is fetched where it is used, which
-        // leaves room for a fifth block per SM (96 registers): 201 us (now 197) on the 1M
+        // leaves room for a fifth block per SM (96 registers): 201 us on the 1M
         // lattice, 252 with it one entry ahead and four blocks, 210 with it
-        // prefetched to L2
+        // prefetched to L2 (197 without the pile lookup, see sphere_pile)
         const int last = off + 32 * (n - 1);   // (n > 0 where it is used)
         auto at = [&](int e) { return min(off + 32 * e, last); };
         int2 c0 = make_int2(0, 0), c1 = c0;

@@ -74,10 +74,11 @@ static_assert(2 * kPhases < kListWords, "the words of all phases and the last on
 // Phase ph (see the file comment): f(item), by the whole block, for the items
 // of [0, items) that this block draws, then the wait for those of the others.
 // False if the wait ran out.  sh: a shared word.  Measured, us of a step that
-// rebuilds, with a fixed share of the items for every block and a barrier over
-// a resident grid -> this: 1,000 spheres 107 -> 115, 100,000 278 -> 276,
-// 1,048,576 1,729 -> 1,797 (three items a draw there: 1,911; the next item
-// drawn ahead: 163 at 1,000).
+// rebuilds, with a fixed share of the items for every block, barriers over a
+// resident grid and cells sorted by a thread each -> this: 1,000 spheres 105 ->
+// 103, 100,000 271 -> 264, 1,048,576 1,717 -> 1,785 (three items a draw there:
+// 1,911, in the phases before the count alone 1,760; the next item drawn while
+// one is worked on: 163 at 1,000).
 template <typename Fn>
 __device__ __forceinline__ bool run_phase(const Arrays &a, const Sizes &z, int ph, int64_t items, unsigned *sh, Fn f)
 {

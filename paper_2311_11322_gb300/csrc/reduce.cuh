@@ -15,7 +15,8 @@
 // the 1M lattice and 13 and 6 us (ncu) of a 1,000-sphere step.  Finishing the
 // opening sums at the end of k_agg_begin instead, by its last blocks, put
 // their chain of fences, atomics and FP64 divisions on the step's: 96 us per
-// step of 7,466 spheres with a planet; at the end of k_lists 83; as it is 73.
+// step of 7,466 spheres with a planet, at the end of k_lists 83, as it is 73 (60
+// with the other kernels as they are now).
 #pragma once
 
 #include "dem_internal.h"
