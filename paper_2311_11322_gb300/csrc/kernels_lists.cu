@@ -71,32 +71,40 @@ enum { kClear, kKeys, kScanTiles, kScanPiles, kScanCells, kScatter, kOrder, kGat
        kPhases };
 static_assert(2 * kPhases < kListWords, "the words of all phases and the last one");
 
+// Count n items at `done`, with the block's writes before it (those of the
+// threads it has synchronised with) visible to whoever sees the count.
+__device__ __forceinline__ void count_done(unsigned *done, unsigned n)
+{
+    asm volatile("red.release.gpu.global.add.u32 [%0], %1;" ::"l"(done), "r"(n) : "memory");
+}
+
 // Phase ph (see the file comment): f(item), by the whole block, for the items
 // of [0, items) that this block draws, then the wait for those of the others.
-// False if the wait ran out.  sh: a shared word.  Measured, us of a step that
-// rebuilds, with a fixed share of the items for every block, barriers over a
-// resident grid and cells sorted by a thread each -> this: 1,000 spheres 105 ->
-// 103, 100,000 271 -> 264, 1,048,576 1,717 -> 1,785 (three items a draw there:
-// 1,911, in the phases before the count alone 1,760; the next item drawn while
-// one is worked on: 163 at 1,000).
+// False if the wait ran out.  sh: a shared word.  Where there are several items
+// for every block, a draw takes some together in the phases whose items are
+// alike and short; a tile's candidates take long and unlike times and are drawn
+// one by one.  Measured, us of a step that rebuilds, with a fixed share of the
+// items for every block, barriers over a resident grid and cells sorted by a
+// thread each -> this: 1,000 spheres 105 -> 104, 100,000 267 -> 257, 1,048,576
+// 1,700 -> 1,719 (always one a draw 1,747, with a full fence 1,774, several in
+// every phase 1,911; the next item drawn while one is worked on: 163 at 1,000).
 template <typename Fn>
 __device__ __forceinline__ bool run_phase(const Arrays &a, const Sizes &z, int ph, int64_t items, unsigned *sh, Fn f)
 {
     unsigned *next = a.lbar + 2 * ph, *done = next + 1;
-    const unsigned n = (unsigned)items;
-    for (bool held = false;; held = true) {
-        __syncthreads();   // the block has done its item (and read *sh)
+    const unsigned n = (unsigned)items, per = ph <= kGather ? max(1u, n / (2 * gridDim.x)) : 1u;
+    for (unsigned held = 0;;) {
+        __syncthreads();   // the block has done what it held (and read *sh)
         if (threadIdx.x == 0) {
-            if (held) {
-                __threadfence();   // visible before it counts as done
-                atomicAdd(done, 1u);
-            }
-            *sh = atomicAdd(next, 1u);
+            if (held) count_done(done, held);
+            *sh = atomicAdd(next, per);
         }
         __syncthreads();
-        const unsigned item = *sh;
-        if (item >= n) break;
-        f((int64_t)item);
+        const unsigned beg = *sh;
+        if (beg >= n) break;
+        const unsigned end = min(beg + per, n);
+        for (unsigned i = beg; i < end; ++i) f((int64_t)i);
+        held = end - beg;
     }
     int ok = 1;
     if (threadIdx.x == 0) {
