@@ -595,7 +595,7 @@ __device__ __forceinline__ void node_force2(const f2_t *nd, f2_t x, f2_t y, f2_t
 // Latency-bound (the rounds depend on one another; 42% of the issue slots,
 // 28 warps an SM by registers).  A stack of cells still to be tested (4 KB)
 // held 22 warps an SM and a cell at a time took twice the instructions: the
-// 100,000-sphere cloud at theta 0.7 went from 758 to 423 us (ncu), its whole
+// 100,000-sphere cloud at theta 0.7 went from 758 to 427 us (ncu), its whole
 // step with the lighter build around the walk from 1,041 to 508 us.
 template <int ORDER>
 __global__ void __launch_bounds__(32) k_tree_force(Arrays a, Sizes z)
