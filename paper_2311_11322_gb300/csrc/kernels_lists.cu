@@ -67,8 +67,7 @@ __device__ __forceinline__ bool any_rebuild(const Arrays &a, const Sizes &z)
 
 // Phases of a rebuild, in order, and the words of Arrays::lbar: per phase the
 // next item and the items done, then the blocks that are done with the launch.
-enum { kClear, kKeys, kScanTiles, kScanPiles, kScanCells, kScatter, kOrder, kGather, kCount, kListScan, kFill, kLink,
-       kPhases };
+enum { kKeys, kScanTiles, kScanPiles, kScanCells, kScatter, kPlace, kCount, kListScan, kFill, kLink, kPhases };
 static_assert(2 * kPhases < kListWords, "the words of all phases and the last one");
 
 // Count n items at `done`, with the block's writes before it (those of the
@@ -83,16 +82,17 @@ __device__ __forceinline__ void count_done(unsigned *done, unsigned n)
 // False if the wait ran out.  sh: a shared word.  Where there are several items
 // for every block, a draw takes some together in the phases whose items are
 // alike and short; a tile's candidates take long and unlike times and are drawn
-// one by one.  Measured, us of a step that rebuilds, with a fixed share of the
-// items for every block, barriers over a resident grid and cells sorted by a
-// thread each -> this: 1,000 spheres 105 -> 104, 100,000 267 -> 257, 1,048,576
-// 1,700 -> 1,719 (always one a draw 1,747, with a full fence 1,774, several in
-// every phase 1,911; the next item drawn while one is worked on: 163 at 1,000).
+// one by one.  Measured, us of a step that rebuilds, with twelve phases, a fixed
+// share of the items for every block, barriers over a resident grid and cells
+// sorted by a thread each -> this, ten phases: 1,000 spheres 105 -> 103, 100,000
+// 268 -> 247, 1,048,576 1,710 -> 1,726 (always one a draw 1,747, several in every
+// phase 1,911), 256 piles of 1.1 million a few of which rebuild 3,250 -> 3,265.
+// The next item drawn while one is worked on: 163 at 1,000.
 template <typename Fn>
 __device__ __forceinline__ bool run_phase(const Arrays &a, const Sizes &z, int ph, int64_t items, unsigned *sh, Fn f)
 {
     unsigned *next = a.lbar + 2 * ph, *done = next + 1;
-    const unsigned n = (unsigned)items, per = ph <= kGather ? max(1u, n / (2 * gridDim.x)) : 1u;
+    const unsigned n = (unsigned)items, per = ph <= kPlace ? max(1u, n / (2 * gridDim.x)) : 1u;
     for (unsigned held = 0;;) {
         __syncthreads();   // the block has done what it held (and read *sh)
         if (threadIdx.x == 0) {
@@ -217,7 +217,7 @@ __device__ __forceinline__ void reference_chunk(const Arrays &a, int64_t ch)
     }
 }
 
-// Zero cell counts of scan tile t.
+// Zero cell counts of scan tile t, for the next rebuild.
 __device__ __forceinline__ void clear_tile(const Arrays &a, const Sizes &z, int64_t t)
 {
     if (!pile_rebuilds(a, tile_pile(a, z, t))) return;
@@ -302,12 +302,12 @@ __device__ __forceinline__ void scan_cells(const Arrays &a, const Sizes &z, int6
 }
 
 // The pile's spheres (home indices) by cell, not yet ordered inside the cells:
-// in a sorted copy that the gather, a later phase, writes anew.
+// in the buffer for the carried-over history, which the last phase writes.
 template <bool FP64>
 __device__ __forceinline__ int32_t *unordered(const Arrays &a, const PileStatic &S)
 {
-    if constexpr (FP64) return (int32_t *)(a.dp_ + S.s0);
-    else return (int32_t *)(a.sph_ + S.s0);
+    if constexpr (FP64) return (int32_t *)(a.hist64_rm + S.e0);
+    else return (int32_t *)(a.hist32_rm + S.e0);
 }
 
 template <bool FP64>
@@ -318,14 +318,15 @@ __device__ __forceinline__ void scatter_sphere(const Arrays &a, int64_t i, int p
     unordered<FP64>(a, S)[slot] = (int32_t)(i - S.s0);
 }
 
-// The sphere in place k of the cells takes its place by home index: the number
-// of its cell's spheres with a smaller one.  Cells hold a handful of spheres,
+// The sphere in place k of the cells, and its place by home index: the number of
+// its cell's spheres with a smaller one (returned with the sphere in hl).  Cells
+// hold a handful of spheres,
 // but a wide range of radii, a large cell_size or a fragment far away can put
 // a whole pile into a few, and sorting such a cell in one thread takes seconds
 // (40,000 spheres beside one of 60 times their radius: 13 s for the step that
 // rebuilds, 0.03 s so).
 template <bool FP64>
-__device__ __forceinline__ void order_sphere(const Arrays &a, int64_t k, int p)
+__device__ __forceinline__ int64_t order_sphere(const Arrays &a, int64_t k, int p, int &hl)
 {
     const PileStatic &S = a.ps[p];
     const int32_t *un = unordered<FP64>(a, S);
@@ -335,20 +336,21 @@ __device__ __forceinline__ void order_sphere(const Arrays &a, int64_t k, int p)
     int r = 0;
 #pragma unroll 4
     for (int x = 0; x < n; ++x) r += un[start + x] < me ? 1 : 0;
+    hl = me;
     a.sorted[S.s0 + start + r] = me;
+    return S.s0 + start + r;
 }
 
 // ---------------------------------------------------------------- gather
 // Sorted copies for the contact pass: position (fixed point in the mixed
 // path), predicted velocity v_i = [v_A + h/2 a_A] + w_A x (r_i - r_A) (Eq.
 // pred-vel), spin, ids; and the gravity input (position relative to the pile
-// frame, mass) at the sphere's home index.
+// frame, mass) at the sphere's home index.  k: sorted position of home sphere hl
+// of an active pile.
 template <bool FP64>
-__device__ __forceinline__ void gather_sphere(const Arrays &a, int64_t k, int p)
+__device__ __forceinline__ void gather_sphere(const Arrays &a, int64_t k, int p, int hl)
 {
-    if (!pile_active(a, p)) return;
     const PileStatic &S = a.ps[p];
-    const int hl = a.sorted[k];
     const int64_t i = S.s0 + hl;
     // the sorted order changes only at rebuilds: the sorted aggregate ids are
     // written in a rebuild step (and read here otherwise); the home -> sorted
@@ -733,9 +735,6 @@ __global__ void __launch_bounds__(kLB, 7) k_lists(Arrays a, Sizes z)
     __shared__ long long ws[kLB / 32];
     int *wsi = (int *)ws;
     const int64_t nsb = (z.N + kLB - 1) / kLB;   // blocks' worth of spheres
-    auto gather = [&](int64_t k) {
-        if (k < z.N) gather_sphere<FP64>(a, k, sphere_pile(a, z, k));
-    };
     if (!any_rebuild(a, z)) {
         // the first blocks sum the piles' chunks (a long chain of loads and
         // shuffles beside the others' gather), the rest gather
@@ -743,17 +742,17 @@ __global__ void __launch_bounds__(kLB, 7) k_lists(Arrays a, Sizes z)
         if (b < 0)
             for (int64_t ch = blockIdx.x; ch < z.CH; ch += nred) open_chunk<FP64, kLB>(a, ch);
         else
-            for (int64_t k = b * kLB + threadIdx.x; k < z.N; k += (gridDim.x - nred) * kLB) gather(k);
+            for (int64_t k = b * kLB + threadIdx.x; k < z.N; k += (gridDim.x - nred) * kLB) {
+                const int p = sphere_pile(a, z, k);
+                if (pile_active(a, p)) gather_sphere<FP64>(a, k, p, a.sorted[k]);
+            }
         return;
     }
     __shared__ unsigned drawn;
     auto phase = [&](int ph, int64_t items, auto f) { return run_phase(a, z, ph, items, &drawn, f); };
-    if (phase(kClear, z.CH + z.T, [&](int64_t t) {
+    if (phase(kKeys, z.CH + nsb, [&](int64_t t) {
             if (t < z.CH) reference_chunk<FP64>(a, t);
-            else clear_tile(a, z, t - z.CH);
-        }) &&
-        phase(kKeys, nsb, [&](int64_t t) {
-            rebuilding_spheres(a, z, t, [&](int64_t i, int p) { key_sphere<FP64>(a, i, p); });
+            else rebuilding_spheres(a, z, t - z.CH, [&](int64_t i, int p) { key_sphere<FP64>(a, i, p); });
         }) &&
         phase(kScanTiles, z.T, [&](int64_t t) { sum_tile(a, z, t, wsi); }) &&
         phase(kScanPiles, z.P, [&](int64_t p) { scan_pile(a, (int)p, wsi); }) &&
@@ -761,17 +760,29 @@ __global__ void __launch_bounds__(kLB, 7) k_lists(Arrays a, Sizes z)
         phase(kScatter, nsb, [&](int64_t t) {
             rebuilding_spheres(a, z, t, [&](int64_t i, int p) { scatter_sphere<FP64>(a, i, p); });
         }) &&
-        phase(kOrder, nsb, [&](int64_t t) {
-            rebuilding_spheres(a, z, t, [&](int64_t k, int p) { order_sphere<FP64>(a, k, p); });
-        }) &&
-        phase(kGather, z.CH + nsb, [&](int64_t t) {
-            if (t < z.CH) open_chunk<FP64, kLB>(a, t);
-            else gather((t - z.CH) * kLB + threadIdx.x);
+        // the gather of every pile and, in the same pass, the order inside the
+        // cells of those that rebuild
+        phase(kPlace, z.CH + nsb, [&](int64_t t) {
+            if (t < z.CH) {
+                open_chunk<FP64, kLB>(a, t);
+                return;
+            }
+            int64_t k = (t - z.CH) * kLB + threadIdx.x;
+            if (k >= z.N) return;
+            const int p = sphere_pile(a, z, k);
+            if (!pile_active(a, p)) return;
+            int hl;
+            if (a.pd[p].rebuild) k = order_sphere<FP64>(a, k, p, hl);
+            else hl = a.sorted[k];
+            gather_sphere<FP64>(a, k, p, hl);
         }) &&
         phase(kCount, z.CT, [&](int64_t t) { count_tile<FP64>(a, t); }) &&
         phase(kListScan, z.P, [&](int64_t p) { scan_lists(a, (int)p, ws); }) &&
         phase(kFill, z.CT, [&](int64_t t) { fill_tile<FP64>(a, t, s_list); }))
-        phase(kLink, z.CT, [&](int64_t t) { link_tile<FP64>(a, t); });
+        phase(kLink, z.CT + z.T, [&](int64_t t) {
+            if (t < z.CT) link_tile<FP64>(a, t);
+            else clear_tile(a, z, t - z.CT);
+        });
     phases_done(a);
 }
 

@@ -751,7 +751,9 @@ dem_status upload_tables(dem_world *w, const GravPlan &gp)
     CU(cudaMemsetAsync(w->A.gcounter, 0, sizeof(int32_t), w->stream));
     // the mixed path's gravity accumulators (each step's conversion leaves them at zero)
     if (w->A.gacc && w->Z.N > 0) CU(cudaMemsetAsync(w->A.gacc, 0, 32 * (size_t)w->Z.N, w->stream));
+    // the list kernel's phase counters and cell counts (each rebuild leaves them at zero)
     if (w->Z.P > 0) CU(cudaMemsetAsync(w->A.lbar, 0, 4 * kListWords, w->stream));
+    if (w->Z.C > 0) CU(cudaMemsetAsync(w->A.ccount, 0, 4 * (size_t)w->Z.C, w->stream));
     // arrival counters of the pile reductions (each reduction leaves them at zero)
     if (w->Z.P > 0) CU(cudaMemsetAsync(w->A.pile_arrive, 0, sizeof(int32_t) * (size_t)w->Z.P, w->stream));
     launch_fill_ids(w->A, w->Z, w->stream);
